@@ -1,8 +1,8 @@
 """Build the GP-MOOD CUDA library (libgpmood.so) for sm_103a, in-tree.
 
 Translation units are compiled in parallel: the host driver with the
-precision-independent kernels, one file per precision for the stage kernels,
-and the binary128 weight solver (plain C, gcc).
+precision-independent kernels, three files per precision (stage, batched and
+reverse-mode kernels), and the binary128 weight solver (plain C, gcc).
 """
 from __future__ import annotations
 
@@ -20,7 +20,8 @@ INCLUDE = os.path.join(ROOT, "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-prec-div=true", "-prec-sqrt=true", "-ftz=false"]
-CUDA_SOURCES = ["gpmood_api.cu", "gpmood_batch.cu", "kernels_f64.cu", "kernels_f32.cu"]
+CUDA_SOURCES = ["gpmood_api.cu", "gpmood_batch.cu"] + [
+    f"kernels_{p}{k}.cu" for p in ("f64", "f32") for k in ("", "_batch", "_adjoint")]
 C_SOURCES = ["gp_weights.c"]
 
 

@@ -1,0 +1,130 @@
+// fixed_dot.h -- weighted sums of doubles in 64-bit fixed point, on the
+// integer pipes.
+//
+// An FP64 instruction holds a GB300 SM sub-partition for 64 cycles; a
+// 32 x 32 + 64-bit integer multiply-add takes 2 and a 64-bit add takes 2
+// (measured).  So a stencil sum sum_m z_m x_m is formed as
+//   x_m  -> X_m, an integer multiple of 2^-57 of the largest power of two in
+//           the stencil (57 bits and a sign; bits below are cut off),
+//   z_m  -> C_m, an integer multiple of 2^-T, T = 60 where |z| < 1,
+//   the sum of products exactly, in two limbs of 29 low bits and the rest,
+//   the sum rounded to 2^-61 of the stencil's scale, and once to a double.
+// A value within a factor of 16 of the stencil's largest is converted
+// without loss, so the sum carries the rounding of its weights (2^-61) and
+// the one to double: about half a unit in the last place of the result,
+// where 25 products and sums rounded in FP64 leave several.  Every step is
+// odd (the sum of the negated values is the negated sum, bit for bit) and
+// does not depend on the order of the terms, so mirror images stay mirror
+// images.
+// Plain C as well as CUDA, so that a host unit test can check it.
+#pragma once
+
+#include <stdint.h>
+#include <string.h>
+
+#ifdef __CUDACC__
+#define FXD_FN __host__ __device__ __forceinline__
+#else
+#define FXD_FN static inline
+#endif
+
+#define FXD_SPLIT 29     // bits of the low limbs
+#define FXD_EMIN 64      // smallest reference exponent (all-zero stencils)
+
+// the words of a double
+FXD_FN uint32_t fxd_hi(double x) {
+  uint64_t b;
+  memcpy(&b, &x, sizeof b);
+  return (uint32_t)(b >> 32);
+}
+FXD_FN uint32_t fxd_lo(double x) {
+  uint64_t b;
+  memcpy(&b, &x, sizeof b);
+  return (uint32_t)b;
+}
+
+// v >> s for 0 <= s, zero from 64 on
+FXD_FN uint64_t fxd_shr(uint64_t v, int s) {
+#ifdef __CUDA_ARCH__
+  uint64_t r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));  // PTX clamps the amount
+  return r;
+#else
+  return s > 63 ? 0 : v >> s;
+#endif
+}
+FXD_FN int fxd_clz(uint32_t v) {
+#ifdef __CUDA_ARCH__
+  return __clz((int)v);
+#else
+  return v ? __builtin_clz(v) : 32;
+#endif
+}
+
+// x as a multiple of 2^(E - 1079), E >= the biased exponent of x: 53
+// significant bits moved up by 4 and down by E - e, the magnitude cut off.
+// Zeros and subnormals (e = 0 < FXD_EMIN <= E) give zero.
+FXD_FN int64_t fxd_from_double(double x, int E) {
+  const uint32_t h = fxd_hi(x), l = fxd_lo(x);
+  const int e = (int)((h >> 20) & 0x7ffu);
+  const uint32_t mh = ((h << 4 | l >> 28) & 0x00ffffffu) | 0x01000000u;
+  const uint64_t m = fxd_shr((uint64_t)mh << 32 | (uint32_t)(l << 4), E - e);
+  const int64_t s = (int32_t)h >> 31;
+  return (int64_t)(m ^ (uint64_t)s) - s;
+}
+
+// the limbs of a stencil sum |s| < 2^60: s = hi 2^29 + lo, 0 <= lo < 2^29
+FXD_FN int32_t fxd_limb_hi(int64_t s) { return (int32_t)(s >> FXD_SPLIT); }
+FXD_FN int32_t fxd_limb_lo(int64_t s) { return (int32_t)s & ((1 << FXD_SPLIT) - 1); }
+
+// the limbs of a weight |c| 2^T < 2^60: C = hi 2^29 + lo, |lo| <= 2^28
+FXD_FN void fxd_weight(double c, int T, int32_t* hi, int32_t* lo) {
+  // c 2^T to the nearest integer; a product by a power of two is exact
+  const double f = c * (double)(1ll << T);
+  const int64_t C = (int64_t)(f < 0.0 ? f - 0.5 : f + 0.5);
+  const int64_t h = (C + (1ll << (FXD_SPLIT - 1))) >> FXD_SPLIT;
+  *hi = (int32_t)h;
+  *lo = (int32_t)(C - h * (1ll << FXD_SPLIT));
+}
+
+// the running sum of products: hh 2^58 + mid 2^29 + ll
+typedef struct {
+  int64_t hh, mid, ll;
+} fxd_acc;
+FXD_FN void fxd_mac(fxd_acc* a, int32_t ch, int32_t cl, int32_t sh, int32_t sl) {
+  a->hh += (int64_t)ch * sh;
+  a->mid += (int64_t)ch * sl;
+  a->mid += (int64_t)cl * sh;
+  a->ll += (int64_t)cl * sl;
+}
+// the sum over 2^56, to the nearest (halves away from zero: odd)
+FXD_FN int64_t fxd_round(fxd_acc a) {
+  const int64_t m = a.mid + (a.ll >> FXD_SPLIT);
+  const int64_t r = (m + (m >> 63) + (1ll << 26)) >> 27;
+  return (int64_t)((uint64_t)a.hh << 2) + r;
+}
+
+// the double nearest r 2^(E + off - 1086): off = 3 + 60 - T takes the sums of
+// fxd_round with weights of T bits and values of reference exponent E.
+// `special`: bits OR-ed into the high word (0x7ff80000: a NaN, for a stencil
+// that holds a NaN or an infinity; else 0).
+FXD_FN double fxd_to_double(int64_t r, int E, int off, uint32_t special) {
+  const uint64_t s = (uint64_t)(r >> 63);
+  const uint64_t m = ((uint64_t)r ^ s) - s;
+  uint32_t h = (uint32_t)(m >> 32), l = (uint32_t)m;
+  int e = E + off - 1;  // the leading one of the significand adds one
+  if (h == 0) {
+    h = l;
+    l = 0;
+    e -= 32;
+  }
+  const int z = fxd_clz(h);
+  const uint64_t n = z > 31 ? 0 : ((uint64_t)h << 32 | l) << z;
+  const uint64_t q = (n >> 11) + ((n >> 10) & 1u);  // halves away from zero
+  uint64_t b = q + ((uint64_t)(uint32_t)(e - z) << 52);
+  if (h == 0) b = 0;
+  b |= (s & 0x8000000000000000ull) | ((uint64_t)special << 32);
+  double x;
+  memcpy(&x, &b, sizeof b);
+  return x;
+}

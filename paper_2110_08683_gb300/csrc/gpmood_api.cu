@@ -680,6 +680,34 @@ namespace gpm {
 
 thread_local int g_pdl = 0;
 
+int fx_segments(int nx) { return (nx + 1 + kSegFaces - 1) / kSegFaces; }
+int fx_chunks(int ny, int nb) { return (ny + 1 + 4 * nb - 2) / (4 * nb - 1); }
+
+// bands a block: the FP64 pipe is each SM's own, so the time is that of the
+// SM with the most bands, ceil(blocks / SMs) blocks of nb bands; of equal
+// choices the longer block, which reconstructs fewer rows twice
+int fx_bands(int nprob, const int* nx, const int* ny) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      sms <= 0) {
+    cudaGetLastError();
+    sms = 152;
+  }
+  int best = 1;
+  long long best_cost = 0;
+  for (int nb = 1; nb <= 16; ++nb) {
+    long long blocks = 0;
+    for (int p = 0; p < nprob; ++p) blocks += (long long)fx_segments(nx[p]) * fx_chunks(ny[p], nb);
+    const long long cost = (blocks + sms - 1) / sms * nb;
+    if (nb == 1 || cost <= best_cost) {
+      best = nb;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 cudaError_t launch_fill(double* X, float* Xf, const Grid& g, const Scalars* sc, double tfrac,
                         cudaStream_t st) {
   long long n = (long long)g.ny * 2 * g.H + (long long)2 * g.H * (g.nx + 2 * g.H);

@@ -130,7 +130,8 @@ struct gpmood_batch_s {
   Scalars *psc, *gsc;  // device: per problem and global
   Scalars* hgsc;       // pinned host mirror of the global scalars
   Item *items_fx[2], *items_fy[2], *items_up, *items_dt;  // [fw 4, fw 8]
-  Item* items_xy;  // fused x+y face blocks: (problem, segment, band of 7 face rows)
+  Item* items_xy;  // fused x+y face blocks: (problem, segment, band of 7 face rows), or
+                   // FP64 (problem, segment, first row, bands)
   int n_fx[2], n_fy[2], n_up, n_dt, n_xy;
   ParityW<double> pw64;
   ParityW<float> pw32;
@@ -268,11 +269,11 @@ int launch_fill_batch(gpmood_batch_t b, int ix, int s, cudaStream_t st) {
 
 template <class Real>
 int launch_faces_batch(gpmood_batch_t b, int dir, const StageArgs<Real>& A,
-                       const ParityW<Real>& P, int fw, int blocks, cudaStream_t st) {
+                       const ParityW<Real>& P, int fw, cudaStream_t st) {
   const int k = fw == 4 ? 0 : 1;
   Item* items = dir == 0 ? b->items_fx[k] : b->items_fy[k];
   int n = dir == 0 ? b->n_fx[k] : b->n_fy[k];
-  return LaunchB<Real>::faces(b->top, dir, fw, A, b->probs, b->psc, items, n, blocks, P, st) ==
+  return LaunchB<Real>::faces(b->top, dir, fw, A, b->probs, b->psc, items, n, P, st) ==
                  cudaSuccess
              ? 0
              : GPMOOD_E_CUDA;
@@ -288,12 +289,12 @@ int faces_b(gpmood_batch_t b, const StageArgs<Real>& A, const ParityW<Real>& P,
                    cudaSuccess
                ? 0
                : GPMOOD_E_CUDA;
-  int rc = launch_faces_batch<Real>(b, 0, A, P, b->fw[0], b->blocks[0], st);
-  if (!rc) rc = launch_faces_batch<Real>(b, 1, A, P, b->fw[1], b->blocks[1], st);
+  int rc = launch_faces_batch<Real>(b, 0, A, P, b->fw[0], st);
+  if (!rc) rc = launch_faces_batch<Real>(b, 1, A, P, b->fw[1], st);
   return rc;
 }
 
-// the autotuner, on the first stage of the current state: the face kernels
+// the autotuner, on the first stage of the current state: the FP32 face kernels
 // (per sweep 4 or 8 warps, i.e. rows, per work item; or the fused x+y
 // kernel, one item per 31 x 7 faces of each direction) and the grid of the
 // update kernel (blocks walking the update items); each variant is timed as
@@ -324,32 +325,34 @@ int tune(gpmood_batch_t b, const ParityW<Real>& P, const DirectW<Real>& D) {
     }
     return ms_min;
   };
-  auto none = [] {};
-  float split = 0.f;
-  for (int dir = 0; dir < 2 && !rc; ++dir) {
-    float best = 1e30f;
-    for (int fw : {4, 8}) {
-      const float ms =
-          timed([&] { return launch_faces_batch<Real>(b, dir, A, P, fw, 0, b->stream); }, none);
-      if (!rc && ms < best) {
-        best = ms;
-        b->fw[dir] = fw;
-        b->blocks[dir] = dir == 0 ? b->n_fx[fw == 4 ? 0 : 1] : b->n_fy[fw == 4 ? 0 : 1];
+  if (sizeof(Real) == sizeof(float)) {  // FP64 has the fused kernel only
+    auto none = [] {};
+    float split = 0.f;
+    for (int dir = 0; dir < 2 && !rc; ++dir) {
+      float best = 1e30f;
+      for (int fw : {4, 8}) {
+        const float ms =
+            timed([&] { return launch_faces_batch<Real>(b, dir, A, P, fw, b->stream); }, none);
+        if (!rc && ms < best) {
+          best = ms;
+          b->fw[dir] = fw;
+          b->blocks[dir] = dir == 0 ? b->n_fx[fw == 4 ? 0 : 1] : b->n_fy[fw == 4 ? 0 : 1];
+        }
       }
+      split += best;
     }
-    split += best;
-  }
-  const float fused = timed(
-      [&] {
-        return LaunchB<Real>::faces_xy(b->top, A, b->probs, b->psc, b->items_xy, b->n_xy, P,
-                                       b->stream) == cudaSuccess
-                   ? 0
-                   : GPMOOD_E_CUDA;
-      },
-      none);
-  if (!rc && fused < split) {
-    b->fw[0] = b->fw[1] = 0;
-    b->blocks[0] = b->blocks[1] = b->n_xy;
+    const float fused = timed(
+        [&] {
+          return LaunchB<Real>::faces_xy(b->top, A, b->probs, b->psc, b->items_xy, b->n_xy, P,
+                                         b->stream) == cudaSuccess
+                     ? 0
+                     : GPMOOD_E_CUDA;
+        },
+        none);
+    if (!rc && fused < split) {
+      b->fw[0] = b->fw[1] = 0;
+      b->blocks[0] = b->blocks[1] = b->n_xy;
+    }
   }
   // the update kernel's grid; the queue and counters it fills are cleared
   // before every run
@@ -632,6 +635,16 @@ int gpmood_batch_create(const gpmood_grid* grids, int nprob, double gamma, int R
   const size_t fsz = sizeof(double);  // face fluxes are FP64 on both paths
   std::vector<Item> fx4, fx8, fy4, fy8, up, dtl, xy;
   long long max_ghost = 0;
+  const bool fp64 = b->precision != GPMOOD_FP32;
+  int bands = 1;
+  if (fp64) {
+    std::vector<int> nxs, nys;
+    for (int p = 0; p < nprob; ++p) {
+      nxs.push_back(grids[p].nx);
+      nys.push_back(grids[p].ny);
+    }
+    bands = fx_bands(nprob, nxs.data(), nys.data());
+  }
   for (int p = 0; p < nprob; ++p) {
     const gpmood_grid* gr = &grids[p];
     Prob& P = b->hprobs[p];
@@ -699,17 +712,20 @@ int gpmood_batch_create(const gpmood_grid* grids, int nprob, double gamma, int R
     fyo = (fyo + 31) / 32 * 32;
     coff += P.ncell;
     // work items
-    for (int fw : {4, 8}) {
-      auto& vx = fw == 4 ? fx4 : fx8;
-      auto& vy = fw == 4 ? fy4 : fy8;
-      const int sx = (g.nx + 1 + kSegFaces - 1) / kSegFaces, bx = (g.ny + fw - 1) / fw;
-      for (int b2 = 0; b2 < bx; ++b2)
-        for (int s2 = 0; s2 < sx; ++s2) vx.push_back(Item{p, s2, b2, 0});
-      const int sy = (g.ny + 1 + kSegFaces - 1) / kSegFaces, by = (g.nx + fw - 1) / fw;
-      for (int b2 = 0; b2 < by; ++b2)
-        for (int s2 = 0; s2 < sy; ++s2) vy.push_back(Item{p, s2, b2, 0});
-    }
-    {
+    if (fp64) {
+      for (int r0 = 0; r0 <= g.ny; r0 += 4 * bands - 1)
+        for (int s2 = 0; s2 < fx_segments(g.nx); ++s2) xy.push_back(Item{p, s2, r0, bands});
+    } else {
+      for (int fw : {4, 8}) {
+        auto& vx = fw == 4 ? fx4 : fx8;
+        auto& vy = fw == 4 ? fy4 : fy8;
+        const int sx = (g.nx + 1 + kSegFaces - 1) / kSegFaces, bx = (g.ny + fw - 1) / fw;
+        for (int b2 = 0; b2 < bx; ++b2)
+          for (int s2 = 0; s2 < sx; ++s2) vx.push_back(Item{p, s2, b2, 0});
+        const int sy = (g.ny + 1 + kSegFaces - 1) / kSegFaces, by = (g.nx + fw - 1) / fw;
+        for (int b2 = 0; b2 < by; ++b2)
+          for (int s2 = 0; s2 < sy; ++s2) vy.push_back(Item{p, s2, b2, 0});
+      }
       const int sx = (g.nx + 1 + kSegFaces - 1) / kSegFaces, bb = (g.ny + 1 + kXYBand - 1) / kXYBand;
       for (int b2 = 0; b2 < bb; ++b2)
         for (int s2 = 0; s2 < sx; ++s2) xy.push_back(Item{p, s2, b2, 0});
@@ -792,8 +808,9 @@ int gpmood_batch_create(const gpmood_grid* grids, int nprob, double gamma, int R
   }
   b->up_blocks = 152 * 8;
   b->dt_blocks = b->n_dt < 152 * 4 ? b->n_dt : 152 * 4;
-  b->fw[0] = b->fw[1] = 8;
-  b->blocks[0] = b->blocks[1] = 152 * 2;
+  // FP64: the fused kernel; FP32: until the tuner has chosen
+  b->fw[0] = b->fw[1] = fp64 ? 0 : 8;
+  b->blocks[0] = b->blocks[1] = fp64 ? b->n_xy : 152 * 2;
   b->stream = nullptr;
   *out = b;
   return GPMOOD_OK;

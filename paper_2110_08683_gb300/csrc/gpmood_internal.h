@@ -102,6 +102,15 @@ struct ParityW {
   Real cy[2][kMaxN];  // y faces (north-face weights)
   Real w[kMaxQ];      // Gauss weights of the rule of this radius
 };
+// FP64: the coefficients as the fixed-point limbs of fixed_dot.h (x high, y
+// low), T bits each
+template <>
+struct ParityW<double> {
+  int2 cx[2][kMaxN];
+  int2 cy[2][kMaxN];
+  int off;            // 63 - T
+  double w[kMaxQ];
+};
 
 // full prediction weights z[R][face][g][m] (face E, W, N, S), for the MOOD
 // recompute at any radius, stencil order: b = -R..R, a = -R..R, |a|+|b| <= R

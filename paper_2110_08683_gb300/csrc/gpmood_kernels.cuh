@@ -21,6 +21,7 @@
 #include <stdint.h>
 
 #include "gpmood_internal.h"
+#include "fixed_dot.h"
 #include "fp_bits.h"
 
 namespace gpm {
@@ -118,16 +119,99 @@ __device__ __forceinline__ void parity_sums(const Load& ld, Real* s) {
   }
 }
 
-// T[px][py] = sum over components of that parity of c[k] s[k]
+// the face states of one variable of one cell from its parity sums: sums()
+// takes the stencil in, dot() forms the sums T[px][py] over the components
+// of each parity, whose sums and differences (the butterflies) are the face
+// states, and out() turns one into a Real.  dead: no cell here, all sums zero.
 template <int R, class Real>
-__device__ __forceinline__ void parity_dot(const Real* c, const Real* s, Real T[2][2]) {
-  T[0][0] = T[0][1] = T[1][0] = T[1][1] = Real(0);
+struct Recon {
+  using T = Real;
+  Real s[stencil_n(R)];
+  template <class Load>
+  __device__ __forceinline__ void sums(const Load& ld, bool live) {
+    if (live) {
+      parity_sums<R, Real>(ld, s);
+    } else {
 #pragma unroll
-  for (int k = 0; k < stencil_n(R); ++k) {
-    const Comp cm = comp_at(R, k);
-    T[cm.px][cm.py] = fma(c[k], s[k], T[cm.px][cm.py]);
+      for (int k = 0; k < stencil_n(R); ++k) s[k] = Real(0);
+    }
   }
-}
+  // R = 0: the face states are the cell average itself
+  template <class Coef>
+  __device__ __forceinline__ void dot(const Coef* c, Real t[2][2]) const {
+    t[0][0] = t[0][1] = t[1][0] = t[1][1] = Real(0);
+    if (R == 0) {
+      t[0][0] = s[0];
+      return;
+    }
+    if constexpr (R > 0) {
+#pragma unroll
+      for (int k = 0; k < stencil_n(R); ++k) {
+        const Comp cm = comp_at(R, k);
+        t[cm.px][cm.py] = fma(c[k], s[k], t[cm.px][cm.py]);
+      }
+    }
+  }
+  __device__ __forceinline__ Real out(Real t, const ParityW<Real>&) const { return t; }
+};
+
+// FP64, R > 0: in fixed point on the integer pipes (fixed_dot.h), scaled by
+// the largest exponent of the cell's own stencil, so that a face state
+// depends on its stencil alone and not on the tile it was computed in.
+template <int R>
+struct ReconFixed {
+  using T = long long;
+  int2 s[stencil_n(R)];  // limbs of the parity sums (x high, y low)
+  int E;                 // reference exponent
+  uint32_t special;      // NaN bits: the stencil holds a NaN or an infinity
+  template <class Load>
+  __device__ __forceinline__ void sums(const Load& ld, bool live) {
+    double x[stencil_n(R)];
+    int k = 0;
+#pragma unroll
+    for (int b = -R; b <= R; ++b)
+#pragma unroll
+      for (int a = -R; a <= R; ++a)
+        if ((a < 0 ? -a : a) + (b < 0 ? -b : b) <= R) x[k++] = live ? ld(a, b) : 0.0;
+    uint32_t top = (uint32_t)FXD_EMIN << 20;
+#pragma unroll
+    for (int m = 0; m < stencil_n(R); ++m) top = max(top, fxd_hi(x[m]) & 0x7fffffffu);
+    E = (int)(top >> 20);
+    special = E == 0x7ff ? 0x7ff80000u : 0u;
+    long long X[stencil_n(R)], p[stencil_n(R)];
+#pragma unroll
+    for (int m = 0; m < stencil_n(R); ++m) X[m] = fxd_from_double(x[m], E);
+    auto at = [&](int a, int b) -> long long {
+      int m = 0;
+      for (int bb = -R; bb < b; ++bb) m += 2 * (R - (bb < 0 ? -bb : bb)) + 1;
+      return X[m + a + R - (b < 0 ? -b : b)];
+    };
+    parity_sums<R, long long>(at, p);
+#pragma unroll
+    for (int m = 0; m < stencil_n(R); ++m) s[m] = make_int2(fxd_limb_hi(p[m]), fxd_limb_lo(p[m]));
+  }
+  __device__ __forceinline__ void dot(const int2* c, long long t[2][2]) const {
+    fxd_acc acc[2][2] = {};
+#pragma unroll
+    for (int k = 0; k < stencil_n(R); ++k) {
+      const Comp cm = comp_at(R, k);
+      fxd_mac(&acc[cm.px][cm.py], c[k].x, c[k].y, s[k].x, s[k].y);
+    }
+#pragma unroll
+    for (int px = 0; px < 2; ++px)
+#pragma unroll
+      for (int py = 0; py < 2; ++py) t[px][py] = fxd_round(acc[px][py]);
+  }
+  __device__ __forceinline__ double out(long long t, const ParityW<double>& W) const {
+    return fxd_to_double(t, E, W.off, special);
+  }
+};
+template <>
+struct Recon<1, double> : ReconFixed<1> {};
+template <>
+struct Recon<2, double> : ReconFixed<2> {};
+template <>
+struct Recon<3, double> : ReconFixed<3> {};
 
 // ---------------------------------------------------------------------------
 // Euler equations (eq. euler_eqn) and HLLC (Toro et al. 1994) in Real
@@ -655,54 +739,34 @@ __device__ __forceinline__ void tile_face_states(const FaceTile<R, Real, FW>& T_
                                                  const ParityW<Real>& W, int fl, int sw,
                                                  bool live, Real (&SP)[rule_q(R)][4],
                                                  Real (&SM)[rule_q(R)][4]) {
-  constexpr int N = stencil_n(R);
   constexpr int Q = rule_q(R);
   constexpr int NS = (Q + 1) / 2;
   auto& tile = T_.t;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    Real s[N];
-    if (live) {
-      // (a, b): offsets along x and y
-      auto ld = [&](int a, int b) -> Real {
-        return DIR == 0 ? tile[v][sw + b][fl + a] : tile[v][sw + a][fl + b];
-      };
-      parity_sums<R, Real>(ld, s);
-    } else {
-#pragma unroll
-      for (int k = 0; k < N; ++k) s[k] = Real(0);
-    }
+    // (a, b): offsets along x and y
+    auto ld = [&](int a, int b) -> Real {
+      return DIR == 0 ? tile[v][sw + b][fl + a] : tile[v][sw + a][fl + b];
+    };
+    Recon<R, Real> rc;
+    rc.sums(ld, live);
 #pragma unroll
     for (int kk = 0; kk < NS; ++kk) {
-      Real T[2][2];
-      parity_dot<R, Real>(DIR == 0 ? W.cx[kk] : W.cy[kk], s, T);
+      typename Recon<R, Real>::T T[2][2];
+      rc.dot(DIR == 0 ? W.cx[kk] : W.cy[kk], T);
       const bool middle = (Q & 1) && kk == Q / 2;
-      if (DIR == 0) {
-        // east / west at +g and -g
-        if (middle) {
-          SP[kk][v] = T[0][0] + T[1][0];
-          SM[kk][v] = T[0][0] - T[1][0];
-        } else {
-          Real e = T[0][0] + T[0][1], o = T[1][0] + T[1][1];
-          Real e2 = T[0][0] - T[0][1], o2 = T[1][0] - T[1][1];
-          SP[kk][v] = e + o;            // E(+g)
-          SM[kk][v] = e - o;            // W(+g)
-          SP[Q - 1 - kk][v] = e2 + o2;  // E(-g)
-          SM[Q - 1 - kk][v] = e2 - o2;  // W(-g)
-        }
+      // DIR 0: e even, o odd along x (east / west); DIR 1: along y (north / south)
+      const auto t01 = DIR == 0 ? T[0][1] : T[1][0], t10 = DIR == 0 ? T[1][0] : T[0][1];
+      if (middle) {
+        SP[kk][v] = rc.out(T[0][0] + t10, W);
+        SM[kk][v] = rc.out(T[0][0] - t10, W);
       } else {
-        // north / south at +g and -g
-        if (middle) {
-          SP[kk][v] = T[0][0] + T[0][1];
-          SM[kk][v] = T[0][0] - T[0][1];
-        } else {
-          Real e = T[0][0] + T[1][0], o = T[0][1] + T[1][1];
-          Real e2 = T[0][0] - T[1][0], o2 = T[0][1] - T[1][1];
-          SP[kk][v] = e + o;            // N(+g)
-          SM[kk][v] = e - o;            // S(+g)
-          SP[Q - 1 - kk][v] = e2 + o2;  // N(-g)
-          SM[Q - 1 - kk][v] = e2 - o2;  // S(-g)
-        }
+        const auto e = T[0][0] + t01, o = t10 + T[1][1];
+        const auto e2 = T[0][0] - t01, o2 = t10 - T[1][1];
+        SP[kk][v] = rc.out(e + o, W);            // E or N (+g)
+        SM[kk][v] = rc.out(e - o, W);            // W or S (+g)
+        SP[Q - 1 - kk][v] = rc.out(e2 + o2, W);  // E or N (-g)
+        SM[Q - 1 - kk][v] = rc.out(e2 - o2, W);  // W or S (-g)
       }
     }
   }
@@ -836,7 +900,6 @@ template <int R, class Real>
 __device__ __forceinline__ void faces_xy_block(const StageArgs<Real>& A, const Grid& g,
                                                const ParityW<Real>& W, int seg, int band,
                                                XYShared<R, Real>& S) {
-  constexpr int N = stencil_n(R);
   constexpr int Q = rule_q(R);
   constexpr int NS = (Q + 1) / 2;
   const int lane = threadIdx.x, warp = threadIdx.y;
@@ -852,46 +915,40 @@ __device__ __forceinline__ void faces_xy_block(const StageArgs<Real>& A, const G
   const int fl = lane + R, sw = warp + R;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    Real s[N];
-    if (row_live) {
-      auto ld = [&](int a, int b) -> Real { return tile[v][sw + b][fl + a]; };
-      parity_sums<R, Real>(ld, s);
-    } else {
-#pragma unroll
-      for (int k = 0; k < N; ++k) s[k] = Real(0);
-    }
+    auto ld = [&](int a, int b) -> Real { return tile[v][sw + b][fl + a]; };
+    Recon<R, Real> rc;
+    rc.sums(ld, row_live);
 #pragma unroll
     for (int kk = 0; kk < NS; ++kk) {
       const bool middle = (Q & 1) && kk == Q / 2;
+      typename Recon<R, Real>::T T[2][2];
       if (xrow) {
         // east / west at +g and -g (the x sweep's butterflies)
-        Real T[2][2];
-        parity_dot<R, Real>(W.cx[kk], s, T);
+        rc.dot(W.cx[kk], T);
         if (middle) {
-          SP[kk][v] = T[0][0] + T[1][0];
-          SM[kk][v] = T[0][0] - T[1][0];
+          SP[kk][v] = rc.out(T[0][0] + T[1][0], W);
+          SM[kk][v] = rc.out(T[0][0] - T[1][0], W);
         } else {
-          Real e = T[0][0] + T[0][1], o = T[1][0] + T[1][1];
-          Real e2 = T[0][0] - T[0][1], o2 = T[1][0] - T[1][1];
-          SP[kk][v] = e + o;
-          SM[kk][v] = e - o;
-          SP[Q - 1 - kk][v] = e2 + o2;
-          SM[Q - 1 - kk][v] = e2 - o2;
+          const auto e = T[0][0] + T[0][1], o = T[1][0] + T[1][1];
+          const auto e2 = T[0][0] - T[0][1], o2 = T[1][0] - T[1][1];
+          SP[kk][v] = rc.out(e + o, W);
+          SM[kk][v] = rc.out(e - o, W);
+          SP[Q - 1 - kk][v] = rc.out(e2 + o2, W);
+          SM[Q - 1 - kk][v] = rc.out(e2 - o2, W);
         }
       }
       // north / south at +g and -g (the y sweep's butterflies), to shared memory
-      Real T[2][2];
-      parity_dot<R, Real>(W.cy[kk], s, T);
+      rc.dot(W.cy[kk], T);
       if (middle) {
-        S.ys[0][kk][v][warp][lane] = T[0][0] + T[0][1];
-        S.ys[1][kk][v][warp][lane] = T[0][0] - T[0][1];
+        S.ys[0][kk][v][warp][lane] = rc.out(T[0][0] + T[0][1], W);
+        S.ys[1][kk][v][warp][lane] = rc.out(T[0][0] - T[0][1], W);
       } else {
-        Real e = T[0][0] + T[1][0], o = T[0][1] + T[1][1];
-        Real e2 = T[0][0] - T[1][0], o2 = T[0][1] - T[1][1];
-        S.ys[0][kk][v][warp][lane] = e + o;
-        S.ys[1][kk][v][warp][lane] = e - o;
-        S.ys[0][Q - 1 - kk][v][warp][lane] = e2 + o2;
-        S.ys[1][Q - 1 - kk][v][warp][lane] = e2 - o2;
+        const auto e = T[0][0] + T[1][0], o = T[0][1] + T[1][1];
+        const auto e2 = T[0][0] - T[1][0], o2 = T[0][1] - T[1][1];
+        S.ys[0][kk][v][warp][lane] = rc.out(e + o, W);
+        S.ys[1][kk][v][warp][lane] = rc.out(e - o, W);
+        S.ys[0][Q - 1 - kk][v][warp][lane] = rc.out(e2 + o2, W);
+        S.ys[1][Q - 1 - kk][v][warp][lane] = rc.out(e2 - o2, W);
       }
     }
   }
@@ -992,12 +1049,10 @@ __device__ __forceinline__ void faces_xy_block(const StageArgs<Real>& A, const G
   }
 }
 
-// resident blocks of the fused face kernel: FP64 2 (128 registers), FP32 4
-template <class Real>
-constexpr int xy_min_blocks() { return sizeof(Real) == sizeof(double) ? 2 : 4; }
+constexpr int kXYBlocks = 4;  // resident blocks an SM of the fused FP32 face kernel
 
 template <int R, class Real>
-__global__ void __launch_bounds__(32 * kXYRows, xy_min_blocks<Real>()) k_faces_xy(StageArgs<Real> A, Grid g,
+__global__ void __launch_bounds__(32 * kXYRows, kXYBlocks) k_faces_xy(StageArgs<Real> A, Grid g,
                                                            const __grid_constant__ ParityW<Real> W) {
   pdl_wait();
   pdl_trigger();
@@ -2070,7 +2125,7 @@ __global__ void __launch_bounds__(32 * FW) k_faces_batch(StageArgs<Real> B, cons
 
 // the fused x+y face kernel over (problem, segment, band) work items
 template <int R, class Real>
-__global__ void __launch_bounds__(32 * kXYRows, xy_min_blocks<Real>()) k_faces_xy_batch(
+__global__ void __launch_bounds__(32 * kXYRows, kXYBlocks) k_faces_xy_batch(
     StageArgs<Real> B, const Prob* probs, const Scalars* psc, const Item* items,
     const __grid_constant__ ParityW<Real> W) {
   pdl_wait();

@@ -35,6 +35,12 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
   return launch_ks(kernel, grid, block, 0, st, args...);
 }
 
+// the FP64 face kernel's blocks: fx_bands() bands of 4 rows each, covering
+// 4 nb - 1 rows of faces (of ny + 1) of a segment of 31
+int fx_segments(int nx);
+int fx_chunks(int ny, int nb);
+int fx_bands(int nprob, const int* nx, const int* ny);
+
 template <class Real>
 struct Launch {
   // first pass: x (dir 0) or y (dir 1) faces at the top radius
@@ -78,12 +84,12 @@ struct LaunchA {
 // batched launchers: persistent grids walking work-item lists
 template <class Real>
 struct LaunchB {
+  // one direction, fw (4 or 8) warps a block (FP32 only)
   static cudaError_t faces(int top, int dir, int fw, const StageArgs<Real>& B, const Prob* probs,
-                           const Scalars* psc, const Item* items, int nitems, int blocks,
+                           const Scalars* psc, const Item* items, int nitems,
                            const ParityW<Real>& W, cudaStream_t st);
-  // max resident blocks per SM of a face kernel variant
-  static int faces_occupancy(int top, int dir, int fw);
-  // both directions in one kernel over (problem, segment, band) items
+  // both directions in one kernel over items: FP32 (problem, segment, band),
+  // FP64 (problem, segment, first row, bands)
   static cudaError_t faces_xy(int top, const StageArgs<Real>& B, const Prob* probs,
                               const Scalars* psc, const Item* items, int nitems,
                               const ParityW<Real>& W, cudaStream_t st);

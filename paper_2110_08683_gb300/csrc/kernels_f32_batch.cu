@@ -1,0 +1,4 @@
+// kernels_f32_batch.cu -- the batched kernels, FP32: reconstruction, Riemann solver and detection in float;
+// state, candidate and RK sums in double.
+#include "kernels_impl.cuh"
+template struct gpm::LaunchB<float>;

@@ -1,5 +1,3 @@
-// kernels_f64.cu -- FP64 instantiation of the stage kernels.
+// kernels_f64.cu -- the stage kernels, FP64.
 #include "kernels_impl.cuh"
 template struct gpm::Launch<double>;
-template struct gpm::LaunchB<double>;
-template struct gpm::LaunchA<double>;

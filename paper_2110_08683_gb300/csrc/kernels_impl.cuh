@@ -1,67 +1,92 @@
 // kernels_impl.cuh -- launcher bodies, instantiated once per precision.
 #pragma once
 
+#include <type_traits>
+
 #include "adjoint_kernels.cuh"
+#include "faces_fp64.cuh"
 #include "gpmood_kernels.cuh"
 #include "gpmood_launch.h"
 
 namespace gpm {
 
-template <int R, class Real>
-static cudaError_t faces_r(int dir, const StageArgs<Real>& A, const Grid& g,
-                           const ParityW<Real>& W, cudaStream_t st) {
+// calls f(std::integral_constant<int, R>) for the top radius
+template <class F>
+static cudaError_t with_radius(int top, F&& f) {
+  switch (top) {
+    case 0: return f(std::integral_constant<int, 0>());
+    case 1: return f(std::integral_constant<int, 1>());
+    case 2: return f(std::integral_constant<int, 2>());
+    default: return f(std::integral_constant<int, 3>());
+  }
+}
+
+// FP64 faces of the directions in dirs (1 x, 2 y, 3 both)
+template <class Real>  // double; a template, so that only its own files instantiate the kernels
+static cudaError_t faces_fx(int top, int dirs, const StageArgs<Real>& A, const Grid& g,
+                            const ParityW<Real>& W, cudaStream_t st) {
+  const int nseg = fx_segments(g.nx), nb = fx_bands(1, &g.nx, &g.ny);
+  const long long blocks = (long long)nseg * fx_chunks(g.ny, nb);
+  return with_radius(top, [&](auto r) {
+    constexpr int R = decltype(r)::value;
+    return launch_ks(k_faces_fx<R>, dim3((unsigned)blocks), dim3(32 * kFxRows),
+                     sizeof(FxShared<R>), st, A, g, W, nseg, nb, dirs);
+  });
+}
+
+template <int R>
+static cudaError_t faces_r(int dir, const StageArgs<float>& A, const Grid& g,
+                           const ParityW<float>& W, cudaStream_t st) {
   dim3 blk(32, kFaceWarps);
   if (dir == 0) {
     dim3 gx((g.nx + 1 + kSegFaces - 1) / kSegFaces, (g.ny + kFaceWarps - 1) / kFaceWarps);
-    return launch_k(k_faces<R, Real, 0, kFaceWarps>, gx, blk, st, A, g, W);
+    return launch_k(k_faces<R, float, 0, kFaceWarps>, gx, blk, st, A, g, W);
   }
   dim3 gy((g.nx + kFaceWarps - 1) / kFaceWarps, (g.ny + 1 + kSegFaces - 1) / kSegFaces);
-  return launch_k(k_faces<R, Real, 1, kFaceWarps>, gy, blk, st, A, g, W);
+  return launch_k(k_faces<R, float, 1, kFaceWarps>, gy, blk, st, A, g, W);
 }
 
 template <class Real>
 cudaError_t Launch<Real>::faces(int top, int dir, const StageArgs<Real>& A, const Grid& g,
                                 const ParityW<Real>& W, cudaStream_t st) {
-  switch (top) {
-    case 0: return faces_r<0, Real>(dir, A, g, W, st);
-    case 1: return faces_r<1, Real>(dir, A, g, W, st);
-    case 2: return faces_r<2, Real>(dir, A, g, W, st);
-    default: return faces_r<3, Real>(dir, A, g, W, st);
-  }
-}
-
-template <int R, class Real>
-static cudaError_t faces_xy_r(const StageArgs<Real>& A, const Grid& g, const ParityW<Real>& W,
-                              cudaStream_t st) {
-  dim3 grd((g.nx + 1 + kSegFaces - 1) / kSegFaces, (g.ny + 1 + kXYBand - 1) / kXYBand);
-  return launch_ks(k_faces_xy<R, Real>, grd, dim3(32, kXYRows), sizeof(XYShared<R, Real>), st,
-                   A, g, W);
+  if constexpr (sizeof(Real) == sizeof(double)) return faces_fx(top, 1 << dir, A, g, W, st);
+  else return with_radius(top, [&](auto r) { return faces_r<decltype(r)::value>(dir, A, g, W, st); });
 }
 
 template <class Real>
 cudaError_t Launch<Real>::faces_xy(int top, const StageArgs<Real>& A, const Grid& g,
                                    const ParityW<Real>& W, cudaStream_t st) {
-  switch (top) {
-    case 0: return faces_xy_r<0, Real>(A, g, W, st);
-    case 1: return faces_xy_r<1, Real>(A, g, W, st);
-    case 2: return faces_xy_r<2, Real>(A, g, W, st);
-    default: return faces_xy_r<3, Real>(A, g, W, st);
+  if constexpr (sizeof(Real) == sizeof(double)) {
+    return faces_fx(top, 3, A, g, W, st);
+  } else {
+    return with_radius(top, [&](auto r) {
+      constexpr int R = decltype(r)::value;
+      dim3 grd((g.nx + 1 + kSegFaces - 1) / kSegFaces, (g.ny + 1 + kXYBand - 1) / kXYBand);
+      return launch_ks(k_faces_xy<R, Real>, grd, dim3(32, kXYRows), sizeof(XYShared<R, Real>),
+                       st, A, g, W);
+    });
   }
 }
 
-template <int R, class Real>
-static cudaError_t xy_attr() {
-  return cudaFuncSetAttribute(k_faces_xy<R, Real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(XYShared<R, Real>));
+// the shared-memory limit of a face kernel of either precision
+template <class Kernel>
+static cudaError_t shared_limit(Kernel k, size_t bytes) {
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+template <class Real, class F>
+static cudaError_t every_radius(F&& f) {
+  cudaError_t e = cudaSuccess;
+  for (int r = 0; r <= 3 && e == cudaSuccess; ++r) e = with_radius(r, f);
+  return e;
 }
 
 template <class Real>
 cudaError_t Launch<Real>::prepare() {
-  cudaError_t e = xy_attr<0, Real>();
-  if (e == cudaSuccess) e = xy_attr<1, Real>();
-  if (e == cudaSuccess) e = xy_attr<2, Real>();
-  if (e == cudaSuccess) e = xy_attr<3, Real>();
-  return e;
+  return every_radius<Real>([](auto r) {
+    constexpr int R = decltype(r)::value;
+    if constexpr (sizeof(Real) == sizeof(double)) return shared_limit(k_faces_fx<R>, sizeof(FxShared<R>));
+    else return shared_limit(k_faces_xy<R, Real>, sizeof(XYShared<R, Real>));
+  });
 }
 
 template <class Real>
@@ -106,44 +131,27 @@ int Launch<Real>::mood_loop_blocks() {
   return sms * (occ < 2 ? occ : 2);
 }
 
-template <int R, class Real, int FW>
-static cudaError_t faces_batch_r(int dir, const StageArgs<Real>& B, const Prob* probs,
-                                 const Scalars* psc, const Item* items, int nitems, int blocks,
-                                 const ParityW<Real>& W, cudaStream_t st) {
-  dim3 blk(32, FW);
-  (void)blocks;  // one block per item
-  if (dir == 0) k_faces_batch<R, Real, 0, FW><<<nitems, blk, 0, st>>>(B, probs, psc, items, W);
-  else k_faces_batch<R, Real, 1, FW><<<nitems, blk, 0, st>>>(B, probs, psc, items, W);
-  return cudaGetLastError();
-}
-
-template <int R, class Real>
-static cudaError_t faces_batch_fw(int dir, int fw, const StageArgs<Real>& B, const Prob* probs,
-                                  const Scalars* psc, const Item* items, int nitems, int blocks,
-                                  const ParityW<Real>& W, cudaStream_t st) {
-  if (fw == 4) return faces_batch_r<R, Real, 4>(dir, B, probs, psc, items, nitems, blocks, W, st);
-  return faces_batch_r<R, Real, 8>(dir, B, probs, psc, items, nitems, blocks, W, st);
+template <int R, int FW>
+static void faces_batch_r(int dir, const StageArgs<float>& B, const Prob* probs,
+                          const Scalars* psc, const Item* items, int nitems,
+                          const ParityW<float>& W, cudaStream_t st) {
+  dim3 blk(32, FW);  // one block per item
+  if (dir == 0) k_faces_batch<R, float, 0, FW><<<nitems, blk, 0, st>>>(B, probs, psc, items, W);
+  else k_faces_batch<R, float, 1, FW><<<nitems, blk, 0, st>>>(B, probs, psc, items, W);
 }
 
 template <class Real>
 cudaError_t LaunchB<Real>::faces(int top, int dir, int fw, const StageArgs<Real>& B,
                                  const Prob* probs, const Scalars* psc, const Item* items,
-                                 int nitems, int blocks, const ParityW<Real>& W, cudaStream_t st) {
+                                 int nitems, const ParityW<Real>& W, cudaStream_t st) {
   if (nitems <= 0) return cudaSuccess;
-  switch (top) {
-    case 0: return faces_batch_fw<0, Real>(dir, fw, B, probs, psc, items, nitems, blocks, W, st);
-    case 1: return faces_batch_fw<1, Real>(dir, fw, B, probs, psc, items, nitems, blocks, W, st);
-    case 2: return faces_batch_fw<2, Real>(dir, fw, B, probs, psc, items, nitems, blocks, W, st);
-    default: return faces_batch_fw<3, Real>(dir, fw, B, probs, psc, items, nitems, blocks, W, st);
-  }
-}
-
-template <int R, class Real>
-static cudaError_t faces_xy_batch_r(const StageArgs<Real>& B, const Prob* probs,
-                                    const Scalars* psc, const Item* items, int nitems,
-                                    const ParityW<Real>& W, cudaStream_t st) {
-  return launch_ks(k_faces_xy_batch<R, Real>, dim3(nitems), dim3(32, kXYRows),
-                   sizeof(XYShared<R, Real>), st, B, probs, psc, items, W);
+  if constexpr (sizeof(Real) == sizeof(double)) return cudaErrorInvalidValue;  // FP64: faces_xy
+  else return with_radius(top, [&](auto r) {
+    constexpr int R = decltype(r)::value;
+    if (fw == 4) faces_batch_r<R, 4>(dir, B, probs, psc, items, nitems, W, st);
+    else faces_batch_r<R, 8>(dir, B, probs, psc, items, nitems, W, st);
+    return cudaGetLastError();
+  });
 }
 
 template <class Real>
@@ -151,51 +159,25 @@ cudaError_t LaunchB<Real>::faces_xy(int top, const StageArgs<Real>& B, const Pro
                                     const Scalars* psc, const Item* items, int nitems,
                                     const ParityW<Real>& W, cudaStream_t st) {
   if (nitems <= 0) return cudaSuccess;
-  switch (top) {
-    case 0: return faces_xy_batch_r<0, Real>(B, probs, psc, items, nitems, W, st);
-    case 1: return faces_xy_batch_r<1, Real>(B, probs, psc, items, nitems, W, st);
-    case 2: return faces_xy_batch_r<2, Real>(B, probs, psc, items, nitems, W, st);
-    default: return faces_xy_batch_r<3, Real>(B, probs, psc, items, nitems, W, st);
-  }
-}
-
-template <int R, class Real>
-static cudaError_t xy_batch_attr() {
-  return cudaFuncSetAttribute(k_faces_xy_batch<R, Real>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(XYShared<R, Real>));
+  return with_radius(top, [&](auto r) {
+    constexpr int R = decltype(r)::value;
+    if constexpr (sizeof(Real) == sizeof(double))
+      return launch_ks(k_faces_fx_batch<R>, dim3(nitems), dim3(32 * kFxRows), sizeof(FxShared<R>),
+                       st, B, probs, psc, items, W);
+    else
+      return launch_ks(k_faces_xy_batch<R, Real>, dim3(nitems), dim3(32, kXYRows),
+                       sizeof(XYShared<R, Real>), st, B, probs, psc, items, W);
+  });
 }
 
 template <class Real>
 cudaError_t LaunchB<Real>::prepare() {
-  cudaError_t e = xy_batch_attr<0, Real>();
-  if (e == cudaSuccess) e = xy_batch_attr<1, Real>();
-  if (e == cudaSuccess) e = xy_batch_attr<2, Real>();
-  if (e == cudaSuccess) e = xy_batch_attr<3, Real>();
-  return e;
-}
-
-template <int R, class Real>
-static int occ_r(int dir, int fw) {
-  int n = 0;
-  if (fw == 4) {
-    if (dir == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_faces_batch<R, Real, 0, 4>, 128, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_faces_batch<R, Real, 1, 4>, 128, 0);
-  } else {
-    if (dir == 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_faces_batch<R, Real, 0, 8>, 256, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_faces_batch<R, Real, 1, 8>, 256, 0);
-  }
-  return n > 0 ? n : 1;
-}
-
-template <class Real>
-int LaunchB<Real>::faces_occupancy(int top, int dir, int fw) {
-  switch (top) {
-    case 0: return occ_r<0, Real>(dir, fw);
-    case 1: return occ_r<1, Real>(dir, fw);
-    case 2: return occ_r<2, Real>(dir, fw);
-    default: return occ_r<3, Real>(dir, fw);
-  }
+  return every_radius<Real>([](auto r) {
+    constexpr int R = decltype(r)::value;
+    if constexpr (sizeof(Real) == sizeof(double))
+      return shared_limit(k_faces_fx_batch<R>, sizeof(FxShared<R>));
+    else return shared_limit(k_faces_xy_batch<R, Real>, sizeof(XYShared<R, Real>));
+  });
 }
 
 template <class Real>

@@ -3,8 +3,10 @@
 // coefficients of the top radius for the first pass.
 #pragma once
 
+#include <math.h>
 #include <string.h>
 
+#include "fixed_dot.h"
 #include "gp_weights.h"
 #include "gpmood_kernels.cuh"
 
@@ -16,6 +18,40 @@ int sidx(const gpw_radius& w, int a, int b) {
   for (int m = 0; m < w.n; ++m)
     if (w.da[m] == a && w.db[m] == b) return m;
   return -1;
+}
+
+// the parity coefficients cx, cy of the top radius, q points a face, in the
+// form the face kernels read
+void set_parity(int, int, const double (*cx)[kMaxN], const double (*cy)[kMaxN],
+                const gpw_radius&, ParityW<float>& P) {
+  for (int kk = 0; kk < 2; ++kk)
+    for (int c = 0; c < kMaxN; ++c) {
+      P.cx[kk][c] = (float)cx[kk][c];
+      P.cy[kk][c] = (float)cy[kk][c];
+    }
+}
+void set_parity(int q, int ns, const double (*cx)[kMaxN], const double (*cy)[kMaxN],
+                const gpw_radius& w, ParityW<double>& P) {
+  // T: every coefficient below one and every face state (at most the sum of
+  // |z| times the stencil's largest value) below four in fixed point
+  double big = 0.0, l1 = 0.0;
+  for (int kk = 0; kk < ns; ++kk)
+    for (int c = 0; c < kMaxN; ++c)
+      big = fmax(big, fmax(fabs(cx[kk][c]), fabs(cy[kk][c])));
+  for (int face = 0; face < 2; ++face)
+    for (int k = 0; k < q; ++k) {
+      double s = 0.0;
+      for (int m = 0; m < w.n; ++m) s += fabs(w.z[face][k][m]);
+      l1 = fmax(l1, s);
+    }
+  int T = 60;
+  while (T > 30 && (ldexp(big, T - 60) >= 1.0 - 0x1p-30 || ldexp(l1, T - 60) >= 3.9)) --T;
+  P.off = 63 - T;
+  for (int kk = 0; kk < 2; ++kk)
+    for (int c = 0; c < kMaxN; ++c) {
+      fxd_weight(cx[kk][c], T, &P.cx[kk][c].x, &P.cx[kk][c].y);
+      fxd_weight(cy[kk][c], T, &P.cy[kk][c].x, &P.cy[kk][c].y);
+    }
 }
 
 template <class Real>
@@ -51,11 +87,13 @@ void fill_weights(const gpw_radius* wr, int top, const double* d2x, const double
   }
   // parity coefficients of the top radius
   const int R = top;
-  if (R == 0) {
-    P.cx[0][0] = P.cy[0][0] = Real(1);
+  if (R == 0) {  // the face states are the cell averages
     P.w[0] = Real(1);
     return;
   }
+  double cx[2][kMaxN], cy[2][kMaxN];
+  memset(cx, 0, sizeof(cx));
+  memset(cy, 0, sizeof(cy));
   const gpw_radius& w = wr[R];
   const int q = w.q, ns = (q + 1) / 2;
   for (int k = 0; k < q; ++k) P.w[k] = (Real)w.w[k];
@@ -80,10 +118,11 @@ void fill_weights(const gpw_radius* wr, int top, const double* d2x, const double
       // at g = 0 the odd components across the face vanish exactly
       if (middle && cm.py) ex = 0.0;
       if (middle && cm.px) ny = 0.0;
-      P.cx[kk][c] = (Real)ex;
-      P.cy[kk][c] = (Real)ny;
+      cx[kk][c] = ex;
+      cy[kk][c] = ny;
     }
   }
+  set_parity(q, ns, cx, cy, w, P);
 }
 
 }  // namespace
