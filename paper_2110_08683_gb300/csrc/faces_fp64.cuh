@@ -4,9 +4,9 @@
 // sub-partition) in the Riemann solver, the integer pipes in the
 // reconstruction (fixed_dot.h).  Three blocks an SM keep both busy: while
 // one block solves, another reconstructs.  4096 x 1024 double Mach
-// reflection, R = 3: 6.0 ms a launch; with the reconstruction on the FP64
-// pipe (parity sums and products, 396 of 716 FP64 instructions a face) it
-// was 11.1 ms.
+// reflection, R = 3: 4.6 ms a launch.  It was 11.1 ms with everything on the
+// FP64 pipe (716 FP64 instructions a face) and 6.0 ms with the
+// reconstruction's 396 taken off it; the solver now takes 180 for 320.
 #pragma once
 
 #include "gpmood_kernels.cuh"

@@ -23,6 +23,7 @@
 #include "gpmood_internal.h"
 #include "fixed_dot.h"
 #include "fp_bits.h"
+#include "fp_newton.h"
 
 namespace gpm {
 
@@ -247,23 +248,9 @@ __device__ __forceinline__ float recip(float x) {
   return fmaf(r, fmaf(-x, r, 1.0f), r);
 }
 
-// square root of a sound-speed argument z > 0 (the Riemann solvers; outside
-// their domain the result is NaN, and so is their flux).  FP64: from the
-// hardware inverse square root y (rsqrt.approx.ftz.f64, relative error below
-// 2^-20 on this GPU), s = z y and two corrections s <- s + (y/2)(z - s^2),
-// each of which multiplies the relative error by about that of y: within
-// one unit in the last place, in six FP64 operations where the IEEE square
-// root takes the FP64 pipe about as long as seven and a half.  FP32: the
-// hardware approximation sqrt.approx.ftz.f32 (the FP32 path's reconstruction
-// and Riemann solver are FP32 arithmetic throughout).
-__device__ __forceinline__ double sqrt_r(double z) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(z));
-  const double h = __dmul_rn(0.5, y);
-  double s = __dmul_rn(z, y);
-  s = fma(h, fma(-s, s, z), s);
-  return fma(h, fma(-s, s, z), s);
-}
+// square root of a sound-speed argument z > 0, FP32: the hardware
+// approximation sqrt.approx.ftz.f32 (the FP32 path's reconstruction and
+// Riemann solver are FP32 arithmetic throughout)
 __device__ __forceinline__ float sqrt_r(float x) {
   float r;
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -428,12 +415,138 @@ __device__ __forceinline__ void hll_x(const Real* UL, const Real* UR, Real gam, 
   }
 }
 
+// ---------------------------------------------------------------------------
+// the same two solvers in FP64.  Every FP64 instruction of a warp costs a
+// sub-partition 64 cycles, so they are written for few of them: 41 an HLLC
+// point (76 as hllc_x above, whose reciprocals and roots took 24):
+//  - reciprocals and square roots on the integer pipes (fp_newton.h);
+//  - products rho u are the momenta themselves;
+//  - one flux formula f = (f0, f0 u + p, f0 v, u (E + p)) for the physical
+//    flux of a side, f0 = rho u, and for the star region, whose velocity is
+//    the contact's: u = S*, f0 = rho* S*, with p* = p_K + q_K (S* - u_K),
+//    E* = (d_K E_K + p* S* - p_K u_K) / (S_K - S*), rho* = q_K / (S_K - S*),
+//    d_K = S_K - u_K and q_K = rho_K d_K (Rankine-Hugoniot across S_K).
+// All products and sums are rounded one by one or explicit FMAs, so every
+// kernel gets the same flux bit for bit.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double recip_int(double x) {
+  float s;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(fpn_recip_arg(x)));
+  return fpn_recip_seeded(x, s);
+}
+__device__ __forceinline__ double sqrt_int(double z) {
+  float s;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(fpn_sqrt_arg(z)));
+  return fpn_sqrt_seeded(z, s);
+}
+// x / 2 for |x| >= 2^-1021 (its exponent reduced)
+__device__ __forceinline__ double half_of(double x) {
+  return __longlong_as_double(__double_as_longlong(x) - (1ll << 52));
+}
+// positive, finite and normal: the arguments recip_int and sqrt_int take
+__device__ __forceinline__ bool pos_normal(double x) {
+  const long long b = __double_as_longlong(x);
+  return b >= 0x0010000000000000ll && b < 0x7ff0000000000000ll;
+}
+
+// one side of a face: velocity along x, pressure, sound speed and 1/rho
+struct Side {
+  double u, p, c, ir;
+  bool ok;  // inside the solver's domain
+};
+__device__ __forceinline__ Side side_of(const double* U, double gam, double gm1) {
+  Side s;
+  s.ir = recip_int(U[0]);
+  s.u = __dmul_rn(U[1], s.ir);
+  const double m2 = fma(U[1], U[1], __dmul_rn(U[2], U[2]));
+  // a subnormal ir / 2 (rho beyond 2^1020) has no use here
+  s.p = __dmul_rn(gm1, fma(-half_of(s.ir), m2, U[3]));
+  s.ok = pos_normal(U[0]) && pos_normal(s.p);
+  s.c = sqrt_int(__dmul_rn(__dmul_rn(gam, s.p), s.ir));
+  // what the caller checks: outside the domain the pressure is not a number
+  if (!pos_normal(U[0])) qnan(s.p);
+  return s;
+}
+
+__device__ __forceinline__ void hllc_x_fp64(const double* UL, const double* UR, double gam,
+                                            double* F, double& pL, double& pR) {
+  const double gm1 = gam - 1.0;
+  const Side L = side_of(UL, gam, gm1), R = side_of(UR, gam, gm1);
+  pL = L.p;
+  pR = R.p;
+  const double SL = min_num(L.u - L.c, R.u - R.c);
+  const double SR = max_num(L.u + L.c, R.u + R.c);
+  const double dL = SL - L.u, dR = SR - R.u;
+  const double qL = __dmul_rn(UL[0], dL), qR = __dmul_rn(UR[0], dR);
+  const double num = fma(-R.u, qR, fma(L.u, qL, R.p - L.p));
+  const double Ss = __dmul_rn(num, recip_int(qL - qR));
+  const bool left = ge0_num(Ss);
+  const bool useL = ge0_num(SL);
+  const bool useS = left || gt0_num(SR);
+  const bool star = !useL && useS;
+  // the side the flux is taken on: of the contact, or of the wave that has
+  // passed the face
+  const bool sideL = useL || (useS && left);
+  const double uK = sideL ? L.u : R.u, pK = sideL ? L.p : R.p, EK = sideL ? UL[3] : UR[3];
+  const double mK = sideL ? UL[1] : UR[1];
+  const double vK = __dmul_rn(sideL ? UL[2] : UR[2], sideL ? L.ir : R.ir);
+  const double SK = sideL ? SL : SR, dK = sideL ? dL : dR, qK = sideL ? qL : qR;
+  const double iD = recip_int(SK - Ss);
+  const double ps = fma(qK, Ss - uK, pK);
+  const double Es = __dmul_rn(iD, fma(dK, EK, fma(ps, Ss, -__dmul_rn(pK, uK))));
+  const double fs = __dmul_rn(__dmul_rn(qK, iD), Ss);
+  const double u = star ? Ss : uK, p = star ? ps : pK, E = star ? Es : EK;
+  const double f = star ? fs : mK;
+  F[0] = f;
+  F[1] = fma(f, u, p);
+  F[2] = __dmul_rn(f, vK);
+  F[3] = __dmul_rn(u, E + p);
+  if (!(L.ok && R.ok)) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) qnan(F[v]);
+  }
+}
+
+__device__ __forceinline__ void hll_x_fp64(const double* UL, const double* UR, double gam,
+                                           double* F, double& pL, double& pR) {
+  const double gm1 = gam - 1.0;
+  const Side L = side_of(UL, gam, gm1), R = side_of(UR, gam, gm1);
+  pL = L.p;
+  pR = R.p;
+  const double SL = min_num(L.u - L.c, R.u - R.c);
+  const double SR = max_num(L.u + L.c, R.u + R.c);
+  // physical fluxes by the same rounded sequence on both sides
+  const double vL = __dmul_rn(UL[2], L.ir), vR = __dmul_rn(UR[2], R.ir);
+  const double FL[4] = {UL[1], fma(UL[1], L.u, L.p), __dmul_rn(UL[1], vL),
+                        __dmul_rn(L.u, UL[3] + L.p)};
+  const double FR[4] = {UR[1], fma(UR[1], R.u, R.p), __dmul_rn(UR[1], vR),
+                        __dmul_rn(R.u, UR[3] + R.p)};
+  const double iw = recip_int(SR - SL), SS = __dmul_rn(SL, SR);
+  const bool useL = ge0_num(SL), useR = !gt0_num(SR);
+  const bool dom = L.ok && R.ok;
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    // x-mirror: (L, R, S_L, S_R) -> (R', L', -S_R, -S_L) swaps the two
+    // products; each is rounded on its own so the mirror face negates exactly
+    const double a = __dmul_rn(SR, FL[v]), b = __dmul_rn(SL, FR[v]);
+    const double c = __dmul_rn(SS, UR[v] - UL[v]);
+    const double Fm = __dmul_rn(__dadd_rn(a - b, c), iw);
+    F[v] = useL ? FL[v] : (useR ? FR[v] : Fm);
+    if (!dom) qnan(F[v]);
+  }
+}
+
 // the Riemann solver of the grid (Grid::riemann: 0 HLLC, 1 HLL)
 template <class Real>
 __device__ __forceinline__ void riemann_x(int kind, const Real* UL, const Real* UR, Real gam,
                                           Real* F, Real& pL, Real& pR) {
-  if (kind == 1) hll_x<Real>(UL, UR, gam, F, pL, pR);
-  else hllc_x<Real>(UL, UR, gam, F, pL, pR);
+  if constexpr (sizeof(Real) == sizeof(double)) {
+    if (kind == 1) hll_x_fp64(UL, UR, gam, F, pL, pR);
+    else hllc_x_fp64(UL, UR, gam, F, pL, pR);
+  } else {
+    if (kind == 1) hll_x<Real>(UL, UR, gam, F, pL, pR);
+    else hllc_x<Real>(UL, UR, gam, F, pL, pR);
+  }
 }
 
 // ---------------------------------------------------------------------------
