@@ -253,8 +253,8 @@ __device__ void adj_face_at(const Real* X, const Grid& g, const DirectW<Real>& W
         UR[v] = __ldg(X + gidx(g, v, iR, jR));
       }
     } else {
-      recon_direct<K, Real, Real>(X, g, Wd.z[K][DIR == 0 ? 0 : 2][q], iL, jL, UL);
-      recon_direct<K, Real, Real>(X, g, Wd.z[K][DIR == 0 ? 1 : 3][q], iR, jR, UR);
+      recon_direct<K, Real>(X, g, Wd, DIR == 0 ? 0 : 2, q, iL, jL, UL);
+      recon_direct<K, Real>(X, g, Wd, DIR == 0 ? 1 : 3, q, iR, jR, UR);
     }
     adj_point<Real, DIR>(UL, UR, gam, Wd.w[K][q], a, q, AL, AR, f, nf);
   }
@@ -386,7 +386,7 @@ __device__ __forceinline__ int stencil_index(int K, int a, int b) {
 }
 
 template <class Real>
-__device__ __forceinline__ void gather_face(const DirectW<Real>& Wd, int face, int a, int b,
+__device__ __forceinline__ void gather_face(const GatherW<Real>& Wd, int face, int a, int b,
                                             int K, const Real* S, long long f, long long nf,
                                             Real* acc) {
   const int ab = (a < 0 ? -a : a) + (b < 0 ? -b : b);
@@ -408,7 +408,7 @@ __device__ __forceinline__ void gather_face(const DirectW<Real>& Wd, int face, i
 // pass 2: every cell of the ghosted grid collects from the faces whose
 // reconstruction stencils contain it
 template <class Real>
-__global__ void __launch_bounds__(256) k_adj_gather(Grid g, const __grid_constant__ DirectW<Real> Wd,
+__global__ void __launch_bounds__(256) k_adj_gather(Grid g, const __grid_constant__ GatherW<Real> Wd,
                                                     AdjFaces Ax, AdjFaces Ay, double* G) {
   const int gx = g.nx + 2 * g.H, gyy = g.ny + 2 * g.H;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;

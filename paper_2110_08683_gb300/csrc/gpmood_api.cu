@@ -40,6 +40,8 @@ struct gpmood_s {
   ParityW<float> pw32;
   DirectW<double> dw64;
   DirectW<float> dw32;
+  GatherW<double> gw64;
+  GatherW<float> gw32;
   int cur;         // buffer holding U^n
   int has_state;
   int launches;
@@ -198,6 +200,12 @@ void make_scheme(int rk, Scheme* S) {
   S->st[3].wa = e2;
   S->st[3].wb = e3;
   S->st[4] = {1, 0, 4, -1, -1, f4 / e4, 1.0, e4, 0.0, 0.0, c};
+}
+
+template <class Real>
+const GatherW<Real>& gather_w(gpmood_t h) {
+  if constexpr (sizeof(Real) == sizeof(float)) return h->gw32;
+  else return h->gw64;
 }
 
 // buffer holding slot `slot` of the scheme in rotation `rot`
@@ -898,6 +906,8 @@ int gpmood_create(const gpmood_grid* grid, double gamma, int R_max, double ell,
   }
   fill_weights<double>(wr, R_max, d2x, d2y, h->pw64, h->dw64);
   fill_weights<float>(wr, R_max, d2x, d2y, h->pw32, h->dw32);
+  fill_gather<double>(wr, R_max, h->gw64);
+  fill_gather<float>(wr, R_max, h->gw32);
 
   // device buffers
   const size_t ncell = (size_t)g.nx * g.ny;
@@ -1267,7 +1277,7 @@ int adj_stage(gpmood_t h, const double* X, const uint8_t* ords, double ts, doubl
   if (st) {
     // the recorded face states: no reconstruction, no ghosted copy of X
     CK(LaunchA<Real>::adj_faces_stored(st, v, ords, g, P, D, h->ax, h->ay, h->stream));
-    CK(LaunchA<Real>::adj_gather(g, D, h->ax, h->ay, h->aG, h->stream));
+    CK(LaunchA<Real>::adj_gather(g, gather_w<Real>(h), h->ax, h->ay, h->aG, h->stream));
     k_adj_fold_y<<<(g.nx + 2 * g.H + 127) / 128, 128, 0, h->stream>>>(h->aG, g);
     k_adj_fold_x<<<(g.ny + 127) / 128, 128, 0, h->stream>>>(h->aG, g);
     k_adj_stage_out<<<152 * 8, 256, 0, h->stream>>>(w, v, h->aG, g, dt);
@@ -1284,7 +1294,7 @@ int adj_stage(gpmood_t h, const double* X, const uint8_t* ords, double ts, doubl
   k_fill_ghosts_at<<<gb, 256, 0, h->stream>>>(h->aX, g, ts);
   CK(cudaGetLastError());
   CK(LaunchA<Real>::adj_faces(h->aX, h->aXr, v, ords, g, P, D, h->ax, h->ay, h->stream));
-  CK(LaunchA<Real>::adj_gather(g, D, h->ax, h->ay, h->aG, h->stream));
+  CK(LaunchA<Real>::adj_gather(g, gather_w<Real>(h), h->ax, h->ay, h->aG, h->stream));
   k_adj_fold_y<<<(g.nx + 2 * g.H + 127) / 128, 128, 0, h->stream>>>(h->aG, g);
   k_adj_fold_x<<<(g.ny + 127) / 128, 128, 0, h->stream>>>(h->aG, g);
   k_adj_stage_out<<<152 * 8, 256, 0, h->stream>>>(w, v, h->aG, g, dt);

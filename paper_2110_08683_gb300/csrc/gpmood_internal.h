@@ -62,9 +62,9 @@ struct Scalars {
   double dt;                    // current step
   unsigned long long rate_bits;  // running max of the CFL rate (|u|+c)/dx as ordered bits
   int err;                      // error bits (kErr*)
-  int count[2];                 // queue lengths (double buffered)
-  int slot;                     // queue holding the cells to work on
-  int go;                       // MOOD loop continues (mirrors the graph condition)
+  int count[2];                 // troubled cells of the first pass (the first entry)
+  unsigned int small_count;     // barrier among the first kSmallBlocks blocks of the MOOD
+  unsigned int small_gen;       // loop kernel: arrivals and generation
   unsigned int stamp_cur;       // stamp of the cells in the current queue
   int iters[5], nbad_first[5], nbad_total[5], nfog_pad[5];  // per RK stage
   long long nsteps;
@@ -74,6 +74,9 @@ struct Scalars {
   unsigned int bar_gen;         // and generation (count returns to 0 after each use)
   int rate_ready;               // rate_bits holds the CFL rate of the current state
   int rate_bad;                 // and that state had a cell with no admissible rate
+  int next[2][2];               // queue lengths of the MOOD loop's iterations, with the
+                                // whole grid and with the small group at work (count[0]
+                                // keeps the first pass's until the loop has ended)
 };
 
 // work the MOOD loop kernel of a stage does once its loop has ended, while its
@@ -112,6 +115,14 @@ struct ParityW<double> {
   double w[kMaxQ];
 };
 
+// slot of offset (a, b) in the radius-3 diamond, rows b = -3..3, in a row a
+// ascending
+__host__ __device__ constexpr int diamond3_slot(int a, int b) {
+  int m = a + 3 - (b < 0 ? -b : b);
+  for (int r = -3; r < b; ++r) m += 2 * (3 - (r < 0 ? -r : r)) + 1;
+  return m;
+}
+
 // full prediction weights z[R][face][g][m] (face E, W, N, S), for the MOOD
 // recompute at any radius, stencil order: b = -R..R, a = -R..R, |a|+|b| <= R
 template <class Real>
@@ -119,6 +130,25 @@ struct DirectW {
   Real z[4][4][kMaxQ][kMaxN];
   Real w[4][kMaxQ];     // Gauss weights per radius (index 0: FOG, one point)
   Real d2x[5], d2y[5];  // App. B second-derivative weights on the R=1 stencil
+  int top;
+};
+
+// FP64: as the fixed-point limbs of fixed_dot.h (x high, y low), every radius
+// in the slots of the radius-3 diamond (zero outside its own): one fixed set
+// of offsets serves every radius
+template <>
+struct DirectW<double> {
+  int2 z[4][4][kMaxQ][kMaxN];
+  int off;              // 63 - T
+  double w[4][kMaxQ];
+  double d2x[5], d2y[5];
+  int top;
+};
+
+// the same weights as plain numbers, for the adjoint's gather
+template <class Real>
+struct GatherW {
+  Real z[4][4][kMaxQ][kMaxN];
   int top;
 };
 
@@ -177,7 +207,9 @@ struct StageArgs {
   double* Fx;        // face-averaged fluxes, FP64 on both paths: each float flux is
   double* Fy;        // widened once, by the face kernel, not once per neighbour
   uint8_t* fbx;      // per x face: bit 0 its left, bit 1 its right state failed the
-  uint8_t* fby;      // face-state check (per y face: lower, upper), at the face's radius
+  uint8_t* fby;      // face-state check (per y face: lower, upper), at the face's radius;
+                     // bits 2-3 of an x face: what detection knows of the cell to its
+                     // right (kVerdict*)
   uint8_t* ord;      // radius per cell, this stage
   uint8_t* first;    // first-pass troubled map, this stage
   int* queue;        // troubled cells (first pass output)

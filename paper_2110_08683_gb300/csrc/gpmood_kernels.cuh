@@ -1200,11 +1200,29 @@ __device__ __forceinline__ Real xload(const Real* X, const Grid& g, int v, int i
   return __ldg(X + gidx(g, v, i, j));
 }
 
+// What Steps 6, 7 and 9 find depends on the stage input alone, not on the
+// candidate, so a cell detected again in the same stage need not repeat it.
+// What is known of a cell is kept in bits 2-3 of the byte of its W face:
+constexpr int kVerdictNone = 0;    // nothing yet
+constexpr int kVerdictAccept = 1;  // accepted by CSD, the plateau or u2
+constexpr int kVerdictDmp = 2;     // CSD and plateau failed, u2 not looked at
+constexpr int kVerdictDmpOnly = 3; // and u2 failed: accepted by the DMP or not at all
+constexpr int kVerdictBits = 12;
+// (the other bits of the byte change in other phases only)
+template <class Real>
+__device__ __forceinline__ void keep_verdict(const StageArgs<Real>& A, const Grid& g, int i,
+                                             int j, int verdict) {
+  uint8_t* b = A.fbx + (long long)j * (g.nx + 1) + i;
+  *b = (uint8_t)((*b & ~kVerdictBits) | verdict << 2);
+}
+
 // X(v, a, b): variable v of the ghosted stage input at (i + a, j + b), in
-// Real; every call below has constant offsets once the loops are unrolled
+// Real; every call below has constant offsets once the loops are unrolled.
+// verdict: what is known of the cell (kVerdict*), updated.
 template <class Real, class LX>
 __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const Detect& D,
-                                            const Real* d2x, const Real* d2y, const double* Yd) {
+                                            const Real* d2x, const Real* d2y, const double* Yd,
+                                            int& verdict) {
   const Real gm1 = det_c<Real>(D.gm1, D.gm1_f);
   Real Y[4] = {to_real<Real>(Yd[0]), to_real<Real>(Yd[1]), to_real<Real>(Yd[2]),
                to_real<Real>(Yd[3])};
@@ -1212,8 +1230,9 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
   Real p = gm1 * (Y[3] - Real(0.5) * (Y[1] * Y[1] + Y[2] * Y[2]) * recip(Y[0]));
   if (!finite_r(rho) || !finite_r(p)) return true;    // Step 4, CAD
   if (!gt0_num(rho) || !gt0_num(p)) return true;       // Step 5, PAD
+  if (verdict == kVerdictAccept) return false;
   const bool two = g.dim == 2;  // 1D: the x terms and the W/E neighbours only
-  if (D.csd_on) {                                      // Step 6, CSD
+  if (verdict == kVerdictNone && D.csd_on) {           // Step 6, CSD
     Real rE = X(0, 1, 0), rW = X(0, -1, 0);
     Real rN = X(0, 0, 1), rS = X(0, 0, -1);
     Real mxE = X(1, 1, 0), mxW = X(1, -1, 0);
@@ -1239,8 +1258,10 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
       gradP += fabs(pN - pS) * hy * recip(my_);
     }
     if (le_ieee(-det_c<Real>(D.sigma_v, D.sigma_v_f), divV) &&
-        le_ieee(gradP, det_c<Real>(D.sigma_p, D.sigma_p_f)))
+        le_ieee(gradP, det_c<Real>(D.sigma_p, D.sigma_p_f))) {
+      verdict = kVerdictAccept;
       return false;
+    }
   }
   Real r0 = X(0, 0, 0);
   Real rmin = r0, rmax = r0;
@@ -1253,8 +1274,15 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
     rmin = lt_ieee(r, rmin) ? r : rmin;
     rmax = lt_ieee(rmax, r) ? r : rmax;
   }
-  if (lt_ieee(rmax - rmin, det_c<Real>(D.plateau_thr, D.plateau_thr_f))) return false;  // Step 7
+  if (verdict == kVerdictNone) {
+    if (lt_ieee(rmax - rmin, det_c<Real>(D.plateau_thr, D.plateau_thr_f))) {  // Step 7
+      verdict = kVerdictAccept;
+      return false;
+    }
+    verdict = kVerdictDmp;
+  }
   if (le_ieee(rmin, rho) && le_ieee(rho, rmax)) return false;     // Step 8, DMP
+  if (verdict == kVerdictDmpOnly) return true;
   // Step 9, u2 with the App. B second-derivative weights (R=1 stencil in
   // the order b=-1: (0,-1); b=0: (-1,0),(0,0),(1,0); b=1: (0,1))
   const int ci[5] = {0, -1, 1, 0, 0}, cj[5] = {0, 0, 0, 1, -1};
@@ -1287,8 +1315,12 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
     // |Cmin|/|Cmax| >= 1/2 written without the division; equal for every
     // non-NaN input once (a) is taken into account
     bool ub = same && le_ieee(Real(0.5) * acmax, acmin);
-    if (!(ua || ub)) return true;
+    if (!(ua || ub)) {
+      verdict = kVerdictDmpOnly;
+      return true;
+    }
   }
+  verdict = kVerdictAccept;
   return false;
 }
 
@@ -1296,42 +1328,9 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
 // reach them (the first pass: many cells in flight hide their latency)
 template <class Real>
 __device__ bool troubled(const Real* X, const Grid& g, const Detect& D, const Real* d2x,
-                         const Real* d2y, int i, int j, const double* Yd) {
+                         const Real* d2y, int i, int j, const double* Yd, int& verdict) {
   auto lx = [&](int v, int a, int b) -> Real { return xload<Real>(X, g, v, i + a, j + b); };
-  return troubled_at<Real>(lx, g, D, d2x, d2y, Yd);
-}
-
-// slot of offset (a, b) in the diamond |a| + |b| <= 2 (13 cells)
-__host__ __device__ constexpr int diamond2_slot(int a, int b) {
-  return b == -2 ? 0 : b == -1 ? 2 + a : b == 0 ? 6 + a : b == 1 ? 10 + a : 12;
-}
-
-// the same tests with every value they may read loaded first, in one batch:
-// the densities of the diamond |a| + |b| <= 2 and the momenta and energies
-// of the four face neighbours.  For the MOOD loop, whose few cells per
-// iteration leave the latency of dependent loads exposed.
-template <class Real>
-__device__ bool troubled_prefetched(const Real* X, const Grid& g, const Detect& D,
-                                    const Real* d2x, const Real* d2y, int i, int j,
-                                    const double* Yd) {
-  Real r[13], m[3][4];
-#pragma unroll
-  for (int b = -2; b <= 2; ++b) {
-    const int hb = 2 - (b < 0 ? -b : b);
-#pragma unroll
-    for (int a = -hb; a <= hb; ++a) r[diamond2_slot(a, b)] = xload<Real>(X, g, 0, i + a, j + b);
-  }
-  const int fa[4] = {1, -1, 0, 0}, fb[4] = {0, 0, 1, -1};
-#pragma unroll
-  for (int v = 1; v < 4; ++v)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) m[v - 1][k] = xload<Real>(X, g, v, i + fa[k], j + fb[k]);
-  auto lx = [&](int v, int a, int b) -> Real {
-    if (v == 0) return r[diamond2_slot(a, b)];
-    const int k = a == 1 ? 0 : a == -1 ? 1 : b == 1 ? 2 : 3;
-    return m[v - 1][k];
-  };
-  return troubled_at<Real>(lx, g, D, d2x, d2y, Yd);
+  return troubled_at<Real>(lx, g, D, d2x, d2y, Yd, verdict);
 }
 
 // candidate of eq. fvm_discrete and the SSP-RK3 combination (eq. rk3) of cell (i,j)
@@ -1363,19 +1362,51 @@ __device__ __forceinline__ void candidate(const StageArgs<Real>& A, const Grid& 
   candidate<Real>(A, g, i, j, stage_coeffs<Real>(A, g, dt), Y);
 }
 
+// u0: U^n of the cell (read where ca is not zero)
 template <class Real>
 __device__ __forceinline__ void combine_store(const StageArgs<Real>& A, const Grid& g, int i,
-                                              int j, const double* Y) {
+                                              int j, const double* Y, const double* u0) {
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     long long k = gidx(g, v, i, j);
-    // the first stage's combination is the candidate itself (ca = 0, cb = 1)
-    const double o = A.ca != 0.0 ? fma(A.ca, A.U0[k], A.cb * Y[v])
-                                 : (A.cb == 1.0 ? Y[v] : A.cb * Y[v]);
+    // the first stage's combination is the candidate itself (ca = 0, cb = 1);
+    // compared as integers, an FP64 compare costs what a product does
+    const double o = __double_as_longlong(A.ca) != 0 ? fma(A.ca, u0[v], A.cb * Y[v])
+                     : __double_as_longlong(A.cb) == 0x3ff0000000000000ll ? Y[v]
+                                                                          : A.cb * Y[v];
     A.out[k] = o;
     if constexpr (sizeof(Real) == sizeof(float)) A.outr[k] = fpb_double_to_float_rn(o);
     if (A.out2) A.out2[k] = fma(A.wa, A.W[k], A.wb * Y[v]);
   }
+}
+template <class Real>
+__device__ __forceinline__ void combine_store(const StageArgs<Real>& A, const Grid& g, int i,
+                                              int j, const double* Y) {
+  double u0[4] = {0.0, 0.0, 0.0, 0.0};
+  if (__double_as_longlong(A.ca) != 0) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) u0[v] = A.U0[gidx(g, v, i, j)];
+  }
+  combine_store<Real>(A, g, i, j, Y, u0);
+}
+
+// a load issued where it stands: the MOOD loop's few cells an iteration leave
+// every memory latency exposed, and the compiler would move a load that only
+// a branch uses into it, behind the loads that decide the branch
+__device__ __forceinline__ double load_now(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ float load_now(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned load_now(const uint8_t* p) {
+  unsigned v;
+  asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
 }
 
 // append to a queue with one atomic per warp
@@ -1408,7 +1439,10 @@ __device__ __forceinline__ void update_cell_w(const StageArgs<Real>& A, const Gr
     candidate<Real>(A, g, i, j, k, Y);
     const int top = Wd.top;
     if (top != 0) {
-      bad = face_state_bad<Real>(A, g, i, j) || troubled<Real>(A.Xr, g, D, d2x, d2y, i, j, Y);
+      int verdict = kVerdictNone;
+      bad = face_state_bad<Real>(A, g, i, j) ||
+            troubled<Real>(A.Xr, g, D, d2x, d2y, i, j, Y, verdict);
+      if (verdict != kVerdictNone) keep_verdict<Real>(A, g, i, j, verdict);
     } else {
       Real y[4] = {(Real)Y[0], (Real)Y[1], (Real)Y[2], (Real)Y[3]};
       Real p = (Real)(g.gamma - 1.0) * (y[3] - Real(0.5) * (y[1] * y[1] + y[2] * y[2]) / y[0]);
@@ -1472,33 +1506,81 @@ __device__ __forceinline__ void radius_pair(const Grid& g, const uint8_t* ord, c
   before = stamp[c] == cur ? C.prev[now] : now;
 }
 
-// direct reconstruction of one face state at radius K (eq. gp_reconstructor)
-// T: storage type of the ghosted state (Real, or double read into Real)
-template <int K, class Real, class T = Real>
-__device__ __forceinline__ void recon_direct(const T* X, const Grid& g, const Real* z, int i,
-                                             int j, Real* S) {
-  // row by row, each row from its centre out in x-mirror pairs (a, -a) with
-  // every product rounded on its own: the x-mirror image of the problem,
-  // whose weights are the mirrored ones, gives the mirrored state bit for bit
+// one variable of a face state by the direct weights at a radius K <= KM
+// given at run time, in fixed point (fixed_dot.h): X points at the cell, z at
+// the weights in the slots of the radius-3 diamond.  All loads are issued
+// before the first use.
+template <int KM>
+__device__ __forceinline__ double fx_value(const double* X, int pitch, const int2* z, int K,
+                                           int off) {
+  double x[stencil_n(KM)];
+  int k = 0;
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const T* Xv = X + (long long)v * g.vstride + (long long)(j + g.H) * g.pitch + (i + g.H);
-    Real s = Real(0);
-    int row = 0;  // stencil index of the row's first cell
+  for (int b = -KM; b <= KM; ++b)
 #pragma unroll
-    for (int b = -K; b <= K; ++b) {
-      const int hb = K - (b < 0 ? -b : b);
-      const int mid = row + hb;  // (0, b)
-      const T* Xr = Xv + (long long)b * g.pitch;
-      Real t = mul_rn(z[mid], (Real)__ldg(Xr));
-#pragma unroll
-      for (int a = 1; a <= hb; ++a)
-        t = add_rn(t, add_rn(mul_rn(z[mid + a], (Real)__ldg(Xr + a)),
-                             mul_rn(z[mid - a], (Real)__ldg(Xr - a))));
-      s = add_rn(s, t);
-      row += 2 * hb + 1;
+    for (int a = -KM; a <= KM; ++a) {
+      const int ab = (a < 0 ? -a : a) + (b < 0 ? -b : b);
+      if (ab <= KM) x[k++] = ab <= K ? __ldg(X + (long long)b * pitch + a) : 0.0;
     }
-    S[v] = s;
+  uint32_t top = (uint32_t)FXD_EMIN << 20;
+#pragma unroll
+  for (int m = 0; m < stencil_n(KM); ++m) top = max(top, fxd_hi(x[m]) & 0x7fffffffu);
+  const int E = (int)(top >> 20);
+  fxd_acc acc = {0, 0, 0};
+  k = 0;
+#pragma unroll
+  for (int b = -KM; b <= KM; ++b)
+#pragma unroll
+    for (int a = -KM; a <= KM; ++a)
+      if ((a < 0 ? -a : a) + (b < 0 ? -b : b) <= KM) {
+        const int2 w = z[diamond3_slot(a, b)];
+        const long long v = fxd_from_double(x[k++], E);
+        fxd_mac(&acc, w.x, w.y, fxd_limb_hi(v), fxd_limb_lo(v));
+      }
+  return fxd_to_double(fxd_round(acc), E, off, E == 0x7ff ? 0x7ff80000u : 0u);
+}
+// out of line: the replay and reverse kernels call it for every variable of
+// every state
+static __device__ __noinline__ double fx_value_any(const double* X, int pitch, const int2* z,
+                                                   int K, int off) {
+  return fx_value<3>(X, pitch, z, K, off);
+}
+
+// direct reconstruction of one face state at radius K (eq.
+// gp_reconstructor): Gauss point q of face 0 E, 1 W, 2 N, 3 S of cell (i, j)
+template <int K, class Real>
+__device__ __forceinline__ void recon_direct(const Real* X, const Grid& g,
+                                             const DirectW<Real>& Wd, int face, int q, int i,
+                                             int j, Real* S) {
+  const Real* Xc = X + (long long)(j + g.H) * g.pitch + (i + g.H);
+  if constexpr (sizeof(Real) == sizeof(double)) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+      S[v] = fx_value_any(Xc + v * g.vstride, g.pitch, Wd.z[K][face][q], K, Wd.off);
+  } else {
+    // row by row, each row from its centre out in x-mirror pairs (a, -a) with
+    // every product rounded on its own: the x-mirror image of the problem,
+    // whose weights are the mirrored ones, gives the mirrored state bit for bit
+    const Real* z = Wd.z[K][face][q];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const Real* Xv = Xc + (long long)v * g.vstride;
+      Real s = Real(0);
+      int row = 0;  // stencil index of the row's first cell
+#pragma unroll
+      for (int b = -K; b <= K; ++b) {
+        const int hb = K - (b < 0 ? -b : b);
+        const int mid = row + hb;  // (0, b)
+        const Real* Xr = Xv + (long long)b * g.pitch;
+        Real t = mul_rn(z[mid], __ldg(Xr));
+#pragma unroll
+        for (int a = 1; a <= hb; ++a)
+          t = add_rn(t, add_rn(mul_rn(z[mid + a], __ldg(Xr + a)), mul_rn(z[mid - a], __ldg(Xr - a))));
+        s = add_rn(s, t);
+        row += 2 * hb + 1;
+      }
+      S[v] = s;
+    }
   }
 }
 
@@ -1520,9 +1602,8 @@ __device__ __forceinline__ void face_point(const Real* X, const Grid& g, const D
       UR[v] = __ldg(X + gidx(g, v, iR, jR));
     }
   } else {
-    // faces: 0 E, 1 W, 2 N, 3 S
-    recon_direct<K, Real>(X, g, Wd.z[K][DIR == 0 ? 0 : 2][q], iL, jL, UL);
-    recon_direct<K, Real>(X, g, Wd.z[K][DIR == 0 ? 1 : 3][q], iR, jR, UR);
+    recon_direct<K, Real>(X, g, Wd, DIR == 0 ? 0 : 2, q, iL, jL, UL);
+    recon_direct<K, Real>(X, g, Wd, DIR == 0 ? 1 : 3, q, iR, jR, UR);
   }
   Real pl, pr;
   if (DIR == 0) {
@@ -1579,12 +1660,13 @@ __device__ __forceinline__ void store_face(const StageArgs<Real>& A, const Grid&
     int f = iR;  // face index
 #pragma unroll
     for (int v = 0; v < 4; ++v) A.Fx[fxidx(g, v, f, jL)] = F[v];
-    A.fbx[(long long)jL * (g.nx + 1) + f] = bits;
+    uint8_t* fb = A.fbx + (long long)jL * (g.nx + 1);
+    fb[f] = (uint8_t)((fb[f] & kVerdictBits) | bits);
     if (g.periodic_x && (f == 0 || f == g.nx)) {
       int f2 = f == 0 ? g.nx : 0;
 #pragma unroll
       for (int v = 0; v < 4; ++v) A.Fx[fxidx(g, v, f2, jL)] = F[v];
-      A.fbx[(long long)jL * (g.nx + 1) + f2] = bits;
+      fb[f2] = (uint8_t)((fb[f2] & kVerdictBits) | bits);
     }
   } else {
     int f = jR;
@@ -1633,97 +1715,8 @@ __device__ __forceinline__ bool mood_face_plan(const StageArgs<Real>& A, const G
   return K != Kold;  // else the EDP1 order of this face is unchanged
 }
 
-// one Gauss point of a face recomputed by the MOOD loop, with the radius K
-// and the direction (0 x, 1 y) as run-time values: the lanes of one warp
-// hold faces of both directions and of several radii, and a compiled
-// variant per (K, direction) would run each variant present in the warp one
-// after the other, Riemann solver included.  One path for all: the stencil
-// rows beyond K are predicated off, and the y direction swaps the momenta
-// around the x solver by selects.  The arithmetic is that of
-// face_point<K, Real, DIR> (recon_direct's order, the same solver), so the
-// flux is the same bit for bit.  z: this point's weights of the left and
-// right states ([K][face][q][.] of DirectW, staged in shared memory).
-template <class Real>
-__device__ __forceinline__ void recon_rt(const Real* X, const Grid& g, const Real* zL,
-                                         const Real* zR, int K, int iL, int jL, int iR, int jR,
-                                         Real* UL, Real* UR) {
-  // the stencil rows and their mirror pairs as loops that run K deep, the
-  // eight (side, variable) sums of one term side by side; each sum sees the
-  // operations of recon_direct<K> in their order
-  const long long vs = g.vstride;
-  const Real* XL = X + (long long)(jL + g.H) * g.pitch + (iL + g.H);
-  const Real* XR = X + (long long)(jR + g.H) * g.pitch + (iR + g.H);
-  Real sL[4], sR[4];
-#pragma unroll
-  for (int v = 0; v < 4; ++v) sL[v] = sR[v] = Real(0);
-  int row = 0;  // stencil index of the row's first cell
-#pragma unroll 1
-  for (int b = -K; b <= K; ++b) {
-    const int hb = K - (b < 0 ? -b : b);
-    const int mid = row + hb;  // (0, b)
-    const Real* L0 = XL + (long long)b * g.pitch;
-    const Real* R0 = XR + (long long)b * g.pitch;
-    Real tL[4], tR[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      tL[v] = mul_rn(zL[mid], __ldg(L0 + v * vs));
-      tR[v] = mul_rn(zR[mid], __ldg(R0 + v * vs));
-    }
-#pragma unroll 1
-    for (int a = 1; a <= hb; ++a) {
-      const Real lp = zL[mid + a], lm = zL[mid - a], rp = zR[mid + a], rm = zR[mid - a];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        tL[v] = add_rn(tL[v], add_rn(mul_rn(lp, __ldg(L0 + v * vs + a)),
-                                     mul_rn(lm, __ldg(L0 + v * vs - a))));
-        tR[v] = add_rn(tR[v], add_rn(mul_rn(rp, __ldg(R0 + v * vs + a)),
-                                     mul_rn(rm, __ldg(R0 + v * vs - a))));
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      sL[v] = add_rn(sL[v], tL[v]);
-      sR[v] = add_rn(sR[v], tR[v]);
-    }
-    row += 2 * hb + 1;
-  }
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    UL[v] = K == 0 ? __ldg(XL + v * vs) : sL[v];
-    UR[v] = K == 0 ? __ldg(XR + v * vs) : sR[v];
-  }
-}
-
-template <class Real>
-__device__ __forceinline__ void face_point_rt(int K, int dir, const Real* X, const Grid& g,
-                                              const Real* zL, const Real* zR, int iL, int jL,
-                                              Real* f, bool& badL, bool& badR, Real* sUL,
-                                              Real* sUR) {
-  const int iR = iL + (dir == 0), jR = jL + (dir == 1);
-  Real UL[4], UR[4];
-  recon_rt<Real>(X, g, zL, zR, K, iL, jL, iR, jR, UL, UR);
-  const bool y = dir != 0;
-  const Real a[4] = {UL[0], y ? UL[2] : UL[1], y ? UL[1] : UL[2], UL[3]};
-  const Real b[4] = {UR[0], y ? UR[2] : UR[1], y ? UR[1] : UR[2], UR[3]};
-  Real h[4], pl, pr;
-  riemann_x<Real>(g.riemann, a, b, (Real)g.gamma, h, pl, pr);
-  f[0] = h[0];
-  f[1] = y ? h[2] : h[1];
-  f[2] = y ? h[1] : h[2];
-  f[3] = h[3];
-  badL |= !(pos_finite(UL[0]) && pos_finite(pl));
-  badR |= !(pos_finite(UR[0]) && pos_finite(pr));
-  if (sUL) {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      sUL[v] = UL[v];
-      sUR[v] = UR[v];
-    }
-  }
-}
-
-// the compiled variant of radius K (the FP32 path: its arithmetic is cheap
-// next to the run-time loops' overhead)
+// one Gauss point of a face recomputed by the MOOD loop on the FP32 path: the
+// compiled variant of radius K
 template <class Real, int DIR>
 __device__ __forceinline__ void face_point_k(int K, const Real* X, const Grid& g,
                                              const DirectW<Real>& Wd, int iL, int jL, int q,
@@ -1737,18 +1730,19 @@ __device__ __forceinline__ void face_point_k(int K, const Real* X, const Grid& g
   }
 }
 
-// DirectW's reconstruction weights, staged in shared memory by the FP64
-// MOOD kernel: the lanes of a warp read different radii, faces and points,
-// which a kernel parameter serves one address at a time
-template <class Real>
-struct MoodW {
-  Real z[4][4][kMaxQ][kMaxN];
+// what the FP64 MOOD kernel keeps in shared memory: the weights of the radii
+// below the top (1 and 2 at most), which the lanes of a warp read at
+// different radii, faces and points at once, and the states of each warp's
+// points
+struct MoodShared {
+  int2 z[2][4][3][kMaxN];
+  double st[8][32][8];  // [warp][point][left 0-3, right 4-7]
 };
-template <class Real>
-__device__ __forceinline__ void stage_mood_weights(const DirectW<Real>& Wd, MoodW<Real>& S) {
-  Real* zs = &S.z[0][0][0][0];
-  const Real* zd = &Wd.z[0][0][0][0];
-  for (int k = threadIdx.x; k < 4 * 4 * kMaxQ * kMaxN; k += blockDim.x) zs[k] = zd[k];
+__device__ __forceinline__ void stage_mood_weights(const DirectW<double>& Wd, MoodShared& S) {
+  for (int k = threadIdx.x; k < 2 * 4 * 3 * kMaxN; k += blockDim.x) {
+    const int m = k % kMaxN, q = k / kMaxN % 3, f = k / (3 * kMaxN) % 4, K = k / (12 * kMaxN);
+    S.z[K][f][q][m] = Wd.z[K + 1][f][q][m];
+  }
   __syncthreads();
 }
 
@@ -1779,23 +1773,46 @@ __device__ __forceinline__ bool mood_update_item(const StageArgs<Real>& A, const
       taken |= o >= 0 && stamp[o] == cur;
     }
   }
+  const long long wf = (long long)dj * (g.nx + 1) + di, sf = (long long)dj * g.nx + di;
+  const unsigned bw = load_now(A.fbx + wf), be = load_now(A.fbx + wf + 1);
+  const unsigned bs = load_now(A.fby + sf), bn = load_now(A.fby + sf + g.nx);
+  const int od = (int)load_now(A.ord + d);
+  const long long k0 = gidx(g, 0, di, dj);
+  const bool with_u0 = __double_as_longlong(A.ca) != 0;
+  double u0[4] = {0.0, 0.0, 0.0, 0.0};
+  if (with_u0) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) u0[v] = load_now(A.U0 + k0 + v * g.vstride);
+  }
+  const Real r0 = load_now(A.Xr + k0), rw = load_now(A.Xr + k0 - 1), re = load_now(A.Xr + k0 + 1);
+  const Real rs = load_now(A.Xr + k0 - g.pitch), rn = load_now(A.Xr + k0 + g.pitch);
   double Y[4];
   candidate<Real>(A, g, di, dj, A.sc->dt, Y);
-  const int od = A.ord[d];
   if (taken) {
     d = -1;
     return false;
   }
   bool flag = false;
   if (od != 0) {
-    flag = face_state_bad<Real>(A, g, di, dj) ||
-           troubled_prefetched<Real>(A.Xr, g, D, d2x, d2y, di, dj, Y);
+    const int known = (int)(bw & kVerdictBits) >> 2;
+    int verdict = known;
+    // face_state_bad; the y faces' bits are zero in 1D
+    flag = (((bw >> 1) | be | (bs >> 1) | bn) & 1) != 0;
+    if (!flag) {
+      auto lx = [&](int v, int a, int b) -> Real {
+        if (v == 0 && a * a + b * b <= 1)
+          return a < 0 ? rw : a > 0 ? re : b < 0 ? rs : b > 0 ? rn : r0;
+        return xload<Real>(A.Xr, g, v, di + a, dj + b);
+      };
+      flag = troubled_at<Real>(lx, g, D, d2x, d2y, Y, verdict);
+    }
+    if (verdict != known) keep_verdict<Real>(A, g, di, dj, verdict);
   } else {
     Real y[4] = {(Real)Y[0], (Real)Y[1], (Real)Y[2], (Real)Y[3]};
     Real p = (Real)(g.gamma - 1.0) * (y[3] - Real(0.5) * (y[1] * y[1] + y[2] * y[2]) / y[0]);
     if (!(y[0] > Real(0)) || !(p > Real(0))) atomicAdd(&A.scw->nfog_pad[A.stage], 1);
   }
-  combine_store<Real>(A, g, di, dj, Y);
+  combine_store<Real>(A, g, di, dj, Y, u0);
   return flag;
 }
 
@@ -1815,33 +1832,43 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// grid-wide barrier of a co-resident grid: the last block to arrive resets
+// barrier among `blocks` co-resident blocks: the last block to arrive resets
 // the count and opens the next generation.  A wait gives up after about a
-// second (or 2^26 polls), latches kErrSync and returns false; a block that
-// sees the error leaves the loop, so no wait can outlast the limit.
-__device__ __forceinline__ bool grid_barrier(Scalars* sc) {
+// second (or 2^26 polls) without a change of *alive (null: none to look at),
+// latches kErrSync and returns false; a block that sees the error leaves the
+// loop, so no wait can outlast the limit.
+__device__ __forceinline__ bool block_barrier(Scalars* sc, unsigned* bar_count,
+                                              unsigned* bar_gen, unsigned blocks,
+                                              unsigned* alive, unsigned pause) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned* gen = &sc->bar_gen;
+    volatile unsigned* gen = bar_gen;
+    volatile unsigned* life = alive;
     volatile int* err = &sc->err;
     const unsigned g0 = *gen;
     __threadfence();
     int good = 1;
-    if (atomicAdd(&sc->bar_count, 1u) == gridDim.x - 1) {
-      atomicExch(&sc->bar_count, 0u);
+    if (atomicAdd(bar_count, 1u) == blocks - 1) {
+      atomicExch(bar_count, 0u);
       __threadfence();
-      atomicAdd(&sc->bar_gen, 1u);
+      atomicAdd(bar_gen, 1u);
     } else {
-      const unsigned long long t0 = global_ns();
-      unsigned polls = 0;
+      unsigned long long t0 = global_ns();
+      unsigned polls = 0, seen = life ? *life : 0;
       while (*gen == g0) {
         if (++polls > (1u << 26) || global_ns() - t0 > 1000000000ull) {
-          atomicOr(&sc->err, kErrSync);
-          good = 0;
-          break;
+          const unsigned now = life ? *life : seen;
+          if (now == seen || (*err & kErrSync)) {
+            atomicOr(&sc->err, kErrSync);
+            good = 0;
+            break;
+          }
+          seen = now;
+          t0 = global_ns();
+          polls = 0;
         }
-        __nanosleep(32);
+        __nanosleep(pause);
       }
       __threadfence();
     }
@@ -1851,6 +1878,22 @@ __device__ __forceinline__ bool grid_barrier(Scalars* sc) {
   __syncthreads();
   return ok != 0;
 }
+// of the whole grid
+__device__ __forceinline__ bool grid_barrier(Scalars* sc) {
+  return block_barrier(sc, &sc->bar_count, &sc->bar_gen, gridDim.x, nullptr, 32);
+}
+
+// Once a queue is short, the first kSmallBlocks blocks (on as many SMs) go on
+// alone to the end of the loop, and once it is very short the first block:
+// the others wait for them (or leave, without a tail).  A barrier among 32
+// blocks takes 1.5-2 us, among all (about 300) 3-5; one block needs neither
+// it nor the L1 invalidation that comes with it, and finds in L1 what the
+// iteration before touched.  Chains of a few cells that walk along a
+// discontinuity for hundreds of iterations are common.  They do not come
+// back: a queue seldom grows, and stays correct if it does.
+constexpr int kSmallBlocks = 32;
+constexpr int kSmallQueue = 256;
+constexpr int kOneQueue64 = 10, kOneQueue32 = 24;  // FP64, FP32
 
 // the stamps of value v: two arrays, one per parity of v, so that an
 // iteration can mark the cells of the next queue (value v + 1) while its own
@@ -1873,91 +1916,203 @@ struct SingleSite {
   }
 };
 
-// lane index of a MOOD phase: the warps are ranked block-minor (warp 0 of
-// every block, then warp 1, ...), so the few warps of a short iteration land
-// on different SMs and FP64 sub-partitions instead of queueing on one
-__device__ __forceinline__ long long mood_lane() {
-  return ((long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+// lane index of a MOOD phase worked on by `blocks` blocks: the warps are
+// ranked block-minor (warp 0 of every block, then warp 1, ...), so the few
+// warps of a short iteration land on different SMs and FP64 sub-partitions
+// instead of queueing on one
+__device__ __forceinline__ long long mood_lane(unsigned blocks) {
+  return ((long long)(threadIdx.x >> 5) * blocks + blockIdx.x) * 32 + (threadIdx.x & 31);
 }
 
-// the MOOD face recompute with one lane per Gauss point: lane t covers
+// the flux of a recomputed face from its points' fluxes, lane by lane: the
+// four lanes of a face hold its points' fluxes fq and state checks bl, br;
+// the first forms the Gauss sum in the order of face_at (mirror pairs summed
+// first), so the flux is the same bit for bit.  Called by whole warps.
+template <class Real>
+__device__ __forceinline__ void gauss_sum(const DirectW<Real>& Wd, int K, const Real* fq, bool bl,
+                                          bool br, Real* F, uint8_t& bits) {
+  const int base = threadIdx.x & 28;
+  Real fp[4][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) fp[p][v] = __shfl_sync(0xffffffffu, fq[v], base + p);
+  const unsigned bbl = __ballot_sync(0xffffffffu, bl), bbr = __ballot_sync(0xffffffffu, br);
+  // face_at's loop over (g, -g) pairs, one path for every rule size:
+  // Q = 4: w1 (f1 + f2) + w0 (f0 + f3); Q = 3: w1 f1 + w0 (f0 + f2);
+  // Q = 2: w0 (f0 + f1); Q = 1: w0 (f0 + 0), which rounds as w0 f0
+  const int Q = rule_q(K);
+  const Real w0 = Wd.w[K][0], w1 = Wd.w[K][1];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const Real z = Real(0);
+    const Real last = Q == 4 ? fp[3][v] : Q == 3 ? fp[2][v] : Q == 2 ? fp[1][v] : z;
+    const Real inner = fma(w0, add_rn(fp[0][v], last), z);
+    const Real mid = Q == 4 ? add_rn(fp[1][v], fp[2][v]) : fp[1][v];
+    const Real outer = fma(w1, mid, inner);
+    F[v] = Q >= 3 ? outer : inner;
+  }
+  bits = (uint8_t)((((bbl >> base) & 0xFu) ? 1 : 0) | (((bbr >> base) & 0xFu) ? 2 : 0));
+}
+
+// the MOOD face recompute, FP32, with one lane per Gauss point: lane t covers
 // pooled cell queue[t / 16], face (t / 4) % 4, point t % 4.  Each lane
-// reconstructs its point's two states and solves its Riemann problem; the
-// group's first lane forms the Gauss sum in the order of face_at (mirror
-// pairs summed first), so the flux is the same bit for bit.  Called by whole
-// warps (the loop runs per warp: all 32 lanes take part in the shuffles).
-template <class Real, class Site>
+// reconstructs its point's two states and solves its Riemann problem.
+// Called by whole warps (the loop runs per warp: all 32 lanes take part in
+// the shuffles).
+template <class Site>
 __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArgs& M,
-                                                 const DirectW<Real>& Wd, const MoodW<Real>& MW,
+                                                 const DirectW<float>& Wd, MoodShared&,
                                                  const Cascade& C, uint32_t cur,
-                                                 const int* queue, int n) {
+                                                 const int* queue, int n, unsigned blocks) {
   const long long L = 16LL * n;
-  const long long stride = (long long)gridDim.x * blockDim.x;
+  const long long stride = (long long)blocks * blockDim.x;
   const int lane = threadIdx.x & 31;
-  const int base = lane & ~3;
   const uint32_t* stamp = stamp_of(M, cur);
-  for (long long t0 = mood_lane() - lane; t0 < L; t0 += stride) {
+  for (long long t0 = mood_lane(blocks) - lane; t0 < L; t0 += stride) {
     const long long t = t0 + lane;
     const int q = (int)(t & 3);
     const int f = (int)((t >> 2) & 3);
     const int gc = t < L ? queue[t >> 4] : 0;
     int iL = 0, jL = 0, K = 0;
     bool work = false;
-    Real fq[4] = {Real(0), Real(0), Real(0), Real(0)};
+    float fq[4] = {0.f, 0.f, 0.f, 0.f};
     bool bl = false, br = false;
     if (t < L)
-      site.with(gc, [&](const StageArgs<Real>& A, const Grid& g, const Detect&, const Real*,
-                        const Real*, int off) {
-        work = mood_face_plan<Real>(A, g, C, stamp + off, cur, gc - off, f, iL, jL, K);
+      site.with(gc, [&](const StageArgs<float>& A, const Grid& g, const Detect&, const float*,
+                        const float*, int off) {
+        work = mood_face_plan<float>(A, g, C, stamp + off, cur, gc - off, f, iL, jL, K);
         if (work && q < rule_q(K)) {
           // a recorded step keeps the states of the recomputed face
           const bool keep = A.sc->ctl.stape != nullptr;
-          Real UL[4], UR[4];
-          const int dir = f < 2 ? 0 : 1;
-          if constexpr (sizeof(Real) == sizeof(double))
-            face_point_rt<Real>(K, dir, A.Xr, g, MW.z[K][2 * dir][q], MW.z[K][2 * dir + 1][q],
-                                iL, jL, fq, bl, br, keep ? UL : nullptr, UR);
-          else if (dir == 0)
-            face_point_k<Real, 0>(K, A.Xr, g, Wd, iL, jL, q, fq, bl, br, keep ? UL : nullptr, UR);
+          float UL[4], UR[4];
+          if (f < 2)
+            face_point_k<float, 0>(K, A.Xr, g, Wd, iL, jL, q, fq, bl, br, keep ? UL : nullptr, UR);
           else
-            face_point_k<Real, 1>(K, A.Xr, g, Wd, iL, jL, q, fq, bl, br, keep ? UL : nullptr, UR);
+            face_point_k<float, 1>(K, A.Xr, g, Wd, iL, jL, q, fq, bl, br, keep ? UL : nullptr, UR);
           if (keep) {
             const int qt = rule_q(Wd.top);
-            if (f < 2) tape_face<Real, 0>(A, g, qt, iL, jL, q, UL, UR);
-            else tape_face<Real, 1>(A, g, qt, iL, jL, q, UL, UR);
+            if (f < 2) tape_face<float, 0>(A, g, qt, iL, jL, q, UL, UR);
+            else tape_face<float, 1>(A, g, qt, iL, jL, q, UL, UR);
           }
         }
       });
-    Real fp[4][4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p)
-#pragma unroll
-      for (int v = 0; v < 4; ++v) fp[p][v] = __shfl_sync(0xffffffffu, fq[v], base + p);
-    const unsigned bbl = __ballot_sync(0xffffffffu, bl), bbr = __ballot_sync(0xffffffffu, br);
-    if (work && q == 0) {
-      // face_at's loop over (g, -g) pairs, one path for every rule size:
-      // Q = 4: w1 (f1 + f2) + w0 (f0 + f3); Q = 3: w1 f1 + w0 (f0 + f2);
-      // Q = 2: w0 (f0 + f1); Q = 1: w0 (f0 + 0), which rounds as w0 f0
-      const int Q = rule_q(K);
-      const Real w0 = Wd.w[K][0], w1 = Wd.w[K][1];
-      Real F[4];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const Real z = Real(0);
-        const Real last = Q == 4 ? fp[3][v] : Q == 3 ? fp[2][v] : Q == 2 ? fp[1][v] : z;
-        const Real inner = fma(w0, add_rn(fp[0][v], last), z);
-        const Real mid = Q == 4 ? add_rn(fp[1][v], fp[2][v]) : fp[1][v];
-        const Real outer = fma(w1, mid, inner);
-        F[v] = Q >= 3 ? outer : inner;
-      }
-      const uint8_t bits = (uint8_t)((((bbl >> base) & 0xFu) ? 1 : 0) |
-                                     (((bbr >> base) & 0xFu) ? 2 : 0));
-      site.with(gc, [&](const StageArgs<Real>& A, const Grid& g, const Detect&, const Real*,
-                        const Real*, int) {
-        if (f < 2) store_face<Real, 0>(A, g, iL, jL, F, bits);
-        else store_face<Real, 1>(A, g, iL, jL, F, bits);
+    float F[4];
+    uint8_t bits;
+    gauss_sum<float>(Wd, K, fq, bl, br, F, bits);
+    if (work && q == 0)
+      site.with(gc, [&](const StageArgs<float>& A, const Grid& g, const Detect&, const float*,
+                        const float*, int) {
+        if (f < 2) store_face<float, 0>(A, g, iL, jL, F, bits);
+        else store_face<float, 1>(A, g, iL, jL, F, bits);
       });
+  }
+}
+
+// The same, FP64.  A warp takes P consecutive points (4, 8, 16 or 32, whole
+// faces): lane l < P plans point l, then the eight values of a point (two
+// sides, four variables) are reconstructed by eight lanes, four points at a
+// time, and lane l solves point l.  A point's chain is 8 times shorter than
+// with one lane a point, and the 32 lanes of an FP64 instruction cost what
+// one does, so P is the number that makes
+//   ceil(points / (P x sub-partitions)) x (a Riemann solve)
+//   + P / 4 x (a reconstruction)
+// smallest: short queues spread over the chip, long ones fill the lanes.
+template <class Site>
+__device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArgs& M,
+                                                 const DirectW<double>& Wd, MoodShared& S,
+                                                 const Cascade& C, uint32_t cur,
+                                                 const int* queue, int n, unsigned blocks) {
+  const long long L = 16LL * n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t* stamp = stamp_of(M, cur);
+  // (in units of 100 cycles; the whole grid has two blocks an SM, the small
+  // group one)
+  const int subs = (blocks == gridDim.x ? 2 : 4) * blocks;
+  int P = 4;
+  long long best = 0;
+#pragma unroll
+  for (int p = 4; p <= 32; p *= 2) {
+    const long long cost = (L + (long long)p * subs - 1) / ((long long)p * subs) * 28 + p / 4 * 6;
+    if (p == 4 || cost < best) {
+      best = cost;
+      P = p;
     }
+  }
+  const long long stride = (long long)blocks * (blockDim.x >> 5) * P;
+  double (*st)[8] = S.st[warp];
+  for (long long t0 = ((long long)warp * blocks + blockIdx.x) * P; t0 < L; t0 += stride) {
+    const long long t = t0 + lane;
+    const int q = (int)(t & 3);
+    const int f = (int)((t >> 2) & 3);
+    const bool mine = lane < P && t < L;
+    const int gc = mine ? queue[t >> 4] : 0;
+    int iL = 0, jL = 0, K = 0, pitch = 0;
+    bool work = false;
+    const double* X = nullptr;  // the left cell, variable 0
+    long long vs = 0;
+    if (mine)
+      site.with(gc, [&](const StageArgs<double>& A, const Grid& g, const Detect&, const double*,
+                        const double*, int off) {
+        work = mood_face_plan<double>(A, g, C, stamp + off, cur, gc - off, f, iL, jL, K);
+        pitch = g.pitch;
+        vs = g.vstride;
+        X = A.Xr + gidx(g, 0, iL, jL);
+      });
+    const bool solve = work && q < rule_q(K);
+    const int dir = f < 2 ? 0 : 1;
+    const int plan = solve ? 1 | K << 1 | dir << 3 | q << 4 : 0;
+    for (int p = 0; p < P; p += 4) {
+      const int src = p + (lane >> 3), v = lane & 3, right = (lane >> 2) & 1;
+      const int pl = __shfl_sync(0xffffffffu, plan, src);
+      const double* Xp = (const double*)__shfl_sync(0xffffffffu, (unsigned long long)X, src);
+      const long long vsp = __shfl_sync(0xffffffffu, vs, src);
+      const int pp = __shfl_sync(0xffffffffu, pitch, src);
+      if (pl) {
+        const int k = (pl >> 1) & 3, d = (pl >> 3) & 1;
+        Xp += v * vsp + (right ? (d ? pp : 1) : 0);
+        st[src][lane & 7] = k == 0 ? __ldg(Xp)
+                                   : fx_value<2>(Xp, pp, S.z[k - 1][2 * d + right][pl >> 4], k, Wd.off);
+      }
+    }
+    __syncwarp();
+    double fq[4] = {0.0, 0.0, 0.0, 0.0};
+    bool bl = false, br = false;
+    if (solve) {
+      // faces: 0 W, 1 E, 2 S, 3 N of the queued cell; the y direction swaps
+      // the momenta around the x solver
+      const int mn = 1 + dir, mt = 2 - dir;
+      const double* u = st[lane];
+      const double a[4] = {u[0], u[mn], u[mt], u[3]};
+      const double b[4] = {u[4], u[4 + mn], u[4 + mt], u[7]};
+      double h[4], pl, pr;
+      site.with(gc, [&](const StageArgs<double>& A, const Grid& g, const Detect&, const double*,
+                        const double*, int) {
+        riemann_x<double>(g.riemann, a, b, g.gamma, h, pl, pr);
+        // a recorded step keeps the states of the recomputed face
+        if (A.sc->ctl.stape != nullptr) {
+          const int qt = rule_q(Wd.top);
+          if (dir == 0) tape_face<double, 0>(A, g, qt, iL, jL, q, u, u + 4);
+          else tape_face<double, 1>(A, g, qt, iL, jL, q, u, u + 4);
+        }
+      });
+      fq[0] = h[0];
+      fq[1] = dir ? h[2] : h[1];
+      fq[2] = dir ? h[1] : h[2];
+      fq[3] = h[3];
+      bl = !(pos_finite(a[0]) && pos_finite(pl));
+      br = !(pos_finite(b[0]) && pos_finite(pr));
+    }
+    double F[4];
+    uint8_t bits;
+    gauss_sum<double>(Wd, K, fq, bl, br, F, bits);
+    if (work && q == 0)
+      site.with(gc, [&](const StageArgs<double>& A, const Grid& g, const Detect&, const double*,
+                        const double*, int) {
+        if (dir == 0) store_face<double, 0>(A, g, iL, jL, F, bits);
+        else store_face<double, 1>(A, g, iL, jL, F, bits);
+      });
+    __syncwarp();  // the states are read before the next points' are written
   }
 }
 
@@ -1968,11 +2123,12 @@ template <class Real, class Site>
 __device__ __forceinline__ void mood_update_phase(const Site& site, const MoodArgs& M,
                                                   const DirectW<Real>& Wd, const Cascade& C,
                                                   uint32_t cur, const int* queue, int n,
-                                                  int* next_queue, int* next_count) {
-  const long long stride = (long long)gridDim.x * blockDim.x;
+                                                  int* next_queue, int* next_count,
+                                                  unsigned blocks) {
+  const long long stride = (long long)blocks * blockDim.x;
   const uint32_t* stamp = stamp_of(M, cur);
   uint32_t* next_stamp = stamp_of(M, cur + 1);
-  for (long long t = mood_lane(); t < 5LL * n; t += stride) {
+  for (long long t = mood_lane(blocks); t < 5LL * n; t += stride) {
     const int gc = queue[t / 5];
     int dg = -1;
     bool flag = false;
@@ -1993,7 +2149,8 @@ __device__ __forceinline__ void mood_update_phase(const Site& site, const MoodAr
   }
 }
 
-// the loop itself, for one problem or a batch (Site).  The first-pass queue
+// the loop itself, for one problem or a batch (Site); tail: every block has
+// work to do after it, on the loop's results.  The first-pass queue
 // is lowered and marked in a prologue; then every iteration is
 //   recompute the faces whose EDP1 radius changed  | barrier
 //   re-update + re-detect, lowering and marking the troubled cells
@@ -2002,63 +2159,94 @@ __device__ __forceinline__ void mood_update_phase(const Site& site, const MoodAr
 template <class Real, class Site>
 __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs& M,
                                                const DirectW<Real>& Wd, const Cascade& C,
-                                               int stage) {
+                                               int stage, bool tail) {
   Scalars* sc = M.sc;
   const bool leader = blockIdx.x == 0 && threadIdx.x == 0;
-  const long long stride = (long long)gridDim.x * blockDim.x;
   // the first pass filled queue 0; queue 1 receives the first iteration's
-  // troubled cells (its count is cleared here, read after two barriers)
+  // troubled cells (the counts are cleared here, used after a barrier).  Each
+  // group of blocks has counts of its own, so a block that leaves the loop may
+  // still read the old ones.
+  __shared__ int one_next[2];
   int n = *(volatile int*)&sc->count[0];
   const int nfirst = n;
   int slot = 0, iters = 0, total = n;
   uint32_t cur = sc->stamp_cur + 1;  // stamp of the cells of the first queue
   const int cap = sc->ctl.max_iters;
-  if (leader) sc->count[1] = 0;
+  if (leader) sc->next[0][1] = sc->next[1][0] = sc->next[1][1] = 0;
+  if (threadIdx.x == 0) one_next[0] = one_next[1] = 0;
   bool ok = true;
-  __shared__ MoodW<Real> MW;
-  if (n > 0) {
-    // n is the same in every block; FP32 reads the kernel parameter
-    if constexpr (sizeof(Real) == sizeof(double)) stage_mood_weights<Real>(Wd, MW);
-    uint32_t* st = stamp_of(M, cur);
-    for (long long q = mood_lane(); q < n; q += stride) {
-      const int gc = M.queue[0][q];
-      site.with(gc, [&](const StageArgs<Real>& A, const Grid&, const Detect&, const Real*,
-                        const Real*, int off) {
-        A.ord[gc - off] = (uint8_t)C.next[A.ord[gc - off]];
-      });
-      st[gc] = cur;
+  unsigned blocks = gridDim.x;  // that work on the queue
+  int* next = sc->next[0];
+  auto barrier = [&]() {
+    if (blocks == 1) {
+      __syncthreads();
+      return true;
     }
-    ok = grid_barrier(sc);
+    return blocks == gridDim.x ? grid_barrier(sc)
+                               : block_barrier(sc, &sc->small_count, &sc->small_gen, blocks,
+                                               nullptr, 32);
+  };
+  // n decides who goes on; false: not this block
+  constexpr int kOneQueue = sizeof(Real) == sizeof(double) ? kOneQueue64 : kOneQueue32;
+  auto shrink = [&]() {
+    if (blocks > 1 && n <= kOneQueue) {
+      blocks = 1;
+      next = one_next;
+    } else if (blocks > (unsigned)kSmallBlocks && n <= kSmallQueue) {
+      blocks = kSmallBlocks;
+      next = sc->next[1];
+    }
+    return blockIdx.x < blocks;
+  };
+  __shared__ MoodShared MS;  // FP64 only
+  if (n > 0) {
+    ok = shrink();
+    if (ok) {
+      // n is the same in every block; FP32 reads the kernel parameter
+      if constexpr (sizeof(Real) == sizeof(double)) stage_mood_weights(Wd, MS);
+      uint32_t* st = stamp_of(M, cur);
+      for (long long q = mood_lane(blocks); q < n; q += (long long)blocks * blockDim.x) {
+        const int gc = M.queue[0][q];
+        site.with(gc, [&](const StageArgs<Real>& A, const Grid&, const Detect&, const Real*,
+                          const Real*, int off) {
+          A.ord[gc - off] = (uint8_t)C.next[A.ord[gc - off]];
+        });
+        st[gc] = cur;
+      }
+      ok = barrier();
+    }
   }
   while (ok && n > 0) {
     if (iters >= cap) {
       if (leader) atomicOr(&sc->err, kErrCap);
       break;
     }
+    if (!shrink()) break;
     const int* queue = M.queue[slot];
-    mood_faces_phase<Real>(site, M, Wd, MW, C, cur, queue, n);
-    if (!grid_barrier(sc)) break;
-    int* next_count = &sc->count[slot ^ 1];
-    mood_update_phase<Real>(site, M, Wd, C, cur, queue, n, M.queue[slot ^ 1], next_count);
-    if (!grid_barrier(sc)) break;
-    n = *(volatile int*)next_count;
+    mood_faces_phase(site, M, Wd, MS, C, cur, queue, n, blocks);
+    if (!barrier()) break;
+    mood_update_phase<Real>(site, M, Wd, C, cur, queue, n, M.queue[slot ^ 1], &next[slot ^ 1],
+                            blocks);
+    if (!barrier()) break;
+    n = *(volatile int*)&next[slot ^ 1];
     // the queue just worked on receives the next iteration's cells
-    if (leader) sc->count[slot] = 0;
+    if (leader) next[slot] = 0;
     total += n;
     iters += 1;
     slot ^= 1;
     cur += 1;
   }
+  // the waiting blocks look at the others' barrier, so a long loop is no
+  // timeout; the error flag of a failed wait also ends this one
+  if (blocks != gridDim.x && tail)
+    block_barrier(sc, &sc->bar_count, &sc->bar_gen, gridDim.x, &sc->small_gen, 256);
   if (leader) {
     sc->nbad_first[stage] = nfirst;
     sc->nbad_total[stage] = total;
     sc->iters[stage] = iters;
     sc->stamp_cur = cur;  // every value up to cur has been used
-    sc->slot = 0;
-    sc->go = 0;
-    // both queues empty for the next stage, also after a failed loop
+    // the queue is empty for the next stage, also after a failed loop
     sc->count[0] = 0;
-    sc->count[1] = 0;
   }
 }
 
@@ -2107,7 +2295,7 @@ __global__ void __launch_bounds__(256, 2) k_mood_loop(StageArgs<Real> A, MoodArg
                                                    Cascade C, int stage, LoopTail T) {
   pdl_wait();
   const SingleSite<Real> site{A, g, D, Wd.d2x, Wd.d2y};
-  mood_loop_body<Real>(site, M, Wd, C, stage);
+  mood_loop_body<Real>(site, M, Wd, C, stage, true);
   mood_loop_tail(g, M.sc, T);
 }
 
@@ -2297,12 +2485,19 @@ __global__ void __launch_bounds__(256) k_update_batch(StageArgs<Real> B, const P
   }
 }
 
+// the first cells of a batch's problems in shared memory, where there is room:
+// a search through the problems themselves is a chain of loads
+constexpr int kMaxStarts = 512;
+struct BatchStarts {
+  int first[kMaxStarts];
+};
 // problem of a pooled cell index (probs sorted by cell_off)
-__device__ __forceinline__ int problem_of(const Prob* probs, int nprob, int gc) {
+__device__ __forceinline__ int problem_of(const Prob* probs, const BatchStarts& S, int nprob,
+                                          int gc) {
   int lo = 0, hi = nprob - 1;
   while (lo < hi) {
     int mid = (lo + hi + 1) >> 1;
-    if (probs[mid].cell_off <= gc) lo = mid;
+    if ((nprob <= kMaxStarts ? S.first[mid] : probs[mid].cell_off) <= gc) lo = mid;
     else hi = mid - 1;
   }
   return lo;
@@ -2316,9 +2511,10 @@ struct BatchSite {
   const Prob* probs;
   const Scalars* psc;
   int nprob;
+  const BatchStarts& starts;
   template <class F>
   __device__ __forceinline__ void with(int gc, F&& f) const {
-    const int p = problem_of(probs, nprob, gc);
+    const int p = problem_of(probs, starts, nprob, gc);
     const Prob& P = probs[p];
     const StageArgs<Real> A = problem_args<Real>(B, P, psc, p);
     f(A, P.g, P.det, d2_of<Real>(P, 0), d2_of<Real>(P, 1), P.cell_off);
@@ -2331,8 +2527,12 @@ __global__ void __launch_bounds__(256, 2) k_mood_loop_batch(StageArgs<Real> B, M
                                                          int nprob,
                                                          const __grid_constant__ DirectW<Real> Wd,
                                                          Cascade C, int stage) {
-  const BatchSite<Real> site{B, probs, psc, nprob};
-  mood_loop_body<Real>(site, M, Wd, C, stage);
+  __shared__ BatchStarts starts;
+  for (int p = threadIdx.x; p < nprob && nprob <= kMaxStarts; p += blockDim.x)
+    starts.first[p] = probs[p].cell_off;
+  __syncthreads();
+  const BatchSite<Real> site{B, probs, psc, nprob, starts};
+  mood_loop_body<Real>(site, M, Wd, C, stage, false);
 }
 
 }  // namespace gpm

@@ -77,7 +77,7 @@ struct LaunchA {
                                       const Grid& g, const ParityW<Real>& W,
                                       const DirectW<Real>& Wd, const AdjFaces& Ax,
                                       const AdjFaces& Ay, cudaStream_t st_);
-  static cudaError_t adj_gather(const Grid& g, const DirectW<Real>& Wd, const AdjFaces& Ax,
+  static cudaError_t adj_gather(const Grid& g, const GatherW<Real>& Wd, const AdjFaces& Ax,
                                 const AdjFaces& Ay, double* G, cudaStream_t st);
 };
 

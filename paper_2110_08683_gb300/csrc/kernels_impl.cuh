@@ -282,7 +282,7 @@ cudaError_t LaunchA<Real>::adj_faces_stored(const void* st, const double* v, con
 }
 
 template <class Real>
-cudaError_t LaunchA<Real>::adj_gather(const Grid& g, const DirectW<Real>& Wd, const AdjFaces& Ax,
+cudaError_t LaunchA<Real>::adj_gather(const Grid& g, const GatherW<Real>& Wd, const AdjFaces& Ax,
                                       const AdjFaces& Ay, double* G, cudaStream_t st) {
   const long long n = (long long)(g.nx + 2 * g.H) * (g.ny + 2 * g.H);
   k_adj_gather<Real><<<(int)((n + 255) / 256), 256, 0, st>>>(g, Wd, Ax, Ay, G);

@@ -20,38 +20,95 @@ int sidx(const gpw_radius& w, int a, int b) {
   return -1;
 }
 
+// the prediction weight of stencil point (a, b) for face E, W, N, S and point
+// k, from the east / north solves at g >= 0 by the mirrors: E at -g is E at
+// g with b negated, W the x-mirror of E; N and S alike
+double direct_weight(const gpw_radius& w, int face, int k, int a, int b) {
+  const int kp = k < (w.q + 1) / 2 ? k : w.q - 1 - k;  // the +g point of the pair
+  if (k != kp) (face < 2 ? b : a) *= -1;
+  if (face == 1) a = -a;
+  if (face == 3) b = -b;
+  return w.z[face / 2][kp][sidx(w, a, b)];
+}
+
+// fixed-point bits T of a set of weights: the largest up to 60 that keeps
+// every weight below one and every sum of |weight| below four
+int weight_bits(double big, double l1) {
+  int T = 60;
+  while (T > 30 && (ldexp(big, T - 60) >= 1.0 - 0x1p-30 || ldexp(l1, T - 60) >= 3.9)) --T;
+  return T;
+}
+
 // the parity coefficients cx, cy of the top radius, q points a face, in the
 // form the face kernels read
-void set_parity(int, int, const double (*cx)[kMaxN], const double (*cy)[kMaxN],
-                const gpw_radius&, ParityW<float>& P) {
+void set_parity(const double (*cx)[kMaxN], const double (*cy)[kMaxN], const gpw_radius&,
+                ParityW<float>& P) {
   for (int kk = 0; kk < 2; ++kk)
     for (int c = 0; c < kMaxN; ++c) {
       P.cx[kk][c] = (float)cx[kk][c];
       P.cy[kk][c] = (float)cy[kk][c];
     }
 }
-void set_parity(int q, int ns, const double (*cx)[kMaxN], const double (*cy)[kMaxN],
-                const gpw_radius& w, ParityW<double>& P) {
-  // T: every coefficient below one and every face state (at most the sum of
-  // |z| times the stencil's largest value) below four in fixed point
+void set_parity(const double (*cx)[kMaxN], const double (*cy)[kMaxN], const gpw_radius& w,
+                ParityW<double>& P) {
   double big = 0.0, l1 = 0.0;
-  for (int kk = 0; kk < ns; ++kk)
+  for (int kk = 0; kk < 2; ++kk)
     for (int c = 0; c < kMaxN; ++c)
       big = fmax(big, fmax(fabs(cx[kk][c]), fabs(cy[kk][c])));
   for (int face = 0; face < 2; ++face)
-    for (int k = 0; k < q; ++k) {
+    for (int k = 0; k < w.q; ++k) {
       double s = 0.0;
       for (int m = 0; m < w.n; ++m) s += fabs(w.z[face][k][m]);
       l1 = fmax(l1, s);
     }
-  int T = 60;
-  while (T > 30 && (ldexp(big, T - 60) >= 1.0 - 0x1p-30 || ldexp(l1, T - 60) >= 3.9)) --T;
+  const int T = weight_bits(big, l1);
   P.off = 63 - T;
   for (int kk = 0; kk < 2; ++kk)
     for (int c = 0; c < kMaxN; ++c) {
       fxd_weight(cx[kk][c], T, &P.cx[kk][c].x, &P.cx[kk][c].y);
       fxd_weight(cy[kk][c], T, &P.cy[kk][c].x, &P.cy[kk][c].y);
     }
+}
+
+// the direct weights of every radius
+template <class Real, class Table>
+void plain_weights(const gpw_radius* wr, Table& D) {
+  for (int R = 1; R <= 3; ++R)
+    for (int face = 0; face < 4; ++face)
+      for (int k = 0; k < wr[R].q && wr[R].n; ++k)
+        for (int m = 0; m < wr[R].n; ++m)
+          D.z[R][face][k][m] = (Real)direct_weight(wr[R], face, k, wr[R].da[m], wr[R].db[m]);
+}
+void set_direct(const gpw_radius* wr, DirectW<float>& D) { plain_weights<float>(wr, D); }
+void set_direct(const gpw_radius* wr, DirectW<double>& D) {
+  double big = 0.0, l1 = 0.0;
+  for (int R = 1; R <= 3; ++R)
+    for (int face = 0; face < 2; ++face)
+      for (int k = 0; k < wr[R].q && wr[R].n; ++k) {
+        double s = 0.0;
+        for (int m = 0; m < wr[R].n; ++m) {
+          s += fabs(wr[R].z[face][k][m]);
+          big = fmax(big, fabs(wr[R].z[face][k][m]));
+        }
+        l1 = fmax(l1, s);
+      }
+  const int T = weight_bits(big, l1);
+  D.off = 63 - T;
+  for (int R = 1; R <= 3; ++R)
+    for (int face = 0; face < 4; ++face)
+      for (int k = 0; k < wr[R].q && wr[R].n; ++k)
+        for (int m = 0; m < wr[R].n; ++m) {
+          const int a = wr[R].da[m], b = wr[R].db[m];
+          int2& z = D.z[R][face][k][diamond3_slot(a, b)];
+          fxd_weight(direct_weight(wr[R], face, k, a, b), T, &z.x, &z.y);
+        }
+}
+
+template <class Real>
+void fill_gather(const gpw_radius* wr, int top, GatherW<Real>& G) {
+  memset(&G, 0, sizeof(G));
+  G.top = top;
+  plain_weights<Real>(wr, G);
 }
 
 template <class Real>
@@ -65,26 +122,9 @@ void fill_weights(const gpw_radius* wr, int top, const double* d2x, const double
     D.d2x[m] = (Real)d2x[m];
     D.d2y[m] = (Real)d2y[m];
   }
-  for (int R = 1; R <= 3; ++R) {
-    const gpw_radius& w = wr[R];
-    if (w.n == 0) continue;
-    const int q = w.q;
-    for (int k = 0; k < q; ++k) D.w[R][k] = (Real)w.w[k];
-    // direct weights from the east / north solves at g >= 0 by the mirrors
-    for (int k = 0; k < q; ++k) {
-      const int kp = k < (q + 1) / 2 ? k : q - 1 - k;  // the +g point of the pair
-      const bool neg = k != kp;
-      for (int m = 0; m < w.n; ++m) {
-        int a = w.da[m], b = w.db[m];
-        // E at g: z_E(g)(a,b); E at -g: z_E(g)(a,-b); W: x-mirror of E
-        D.z[R][0][k][m] = (Real)w.z[0][kp][sidx(w, a, neg ? -b : b)];
-        D.z[R][1][k][m] = (Real)w.z[0][kp][sidx(w, -a, neg ? -b : b)];
-        // N at g: z_N(g)(a,b); N at -g: z_N(g)(-a,b); S: y-mirror of N
-        D.z[R][2][k][m] = (Real)w.z[1][kp][sidx(w, neg ? -a : a, b)];
-        D.z[R][3][k][m] = (Real)w.z[1][kp][sidx(w, neg ? -a : a, -b)];
-      }
-    }
-  }
+  for (int R = 1; R <= 3; ++R)
+    for (int k = 0; k < wr[R].q && wr[R].n; ++k) D.w[R][k] = (Real)wr[R].w[k];
+  set_direct(wr, D);
   // parity coefficients of the top radius
   const int R = top;
   if (R == 0) {  // the face states are the cell averages
@@ -122,7 +162,7 @@ void fill_weights(const gpw_radius* wr, int top, const double* d2x, const double
       cy[kk][c] = ny;
     }
   }
-  set_parity(q, ns, cx, cy, w, P);
+  set_parity(cx, cy, w, P);
 }
 
 }  // namespace
