@@ -1208,6 +1208,8 @@ constexpr int kVerdictAccept = 1;  // accepted by CSD, the plateau or u2
 constexpr int kVerdictDmp = 2;     // CSD and plateau failed, u2 not looked at
 constexpr int kVerdictDmpOnly = 3; // and u2 failed: accepted by the DMP or not at all
 constexpr int kVerdictBits = 12;
+// (not kept: CAD and PAD passed and CSD failed, as quick_csd found)
+constexpr int kVerdictCsdFailed = 4;
 // (the other bits of the byte change in other phases only)
 template <class Real>
 __device__ __forceinline__ void keep_verdict(const StageArgs<Real>& A, const Grid& g, int i,
@@ -1227,9 +1229,11 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
   Real Y[4] = {to_real<Real>(Yd[0]), to_real<Real>(Yd[1]), to_real<Real>(Yd[2]),
                to_real<Real>(Yd[3])};
   Real rho = Y[0];
-  Real p = gm1 * (Y[3] - Real(0.5) * (Y[1] * Y[1] + Y[2] * Y[2]) * recip(Y[0]));
-  if (!finite_r(rho) || !finite_r(p)) return true;    // Step 4, CAD
-  if (!gt0_num(rho) || !gt0_num(p)) return true;       // Step 5, PAD
+  if (verdict != kVerdictCsdFailed) {
+    Real p = gm1 * (Y[3] - Real(0.5) * (Y[1] * Y[1] + Y[2] * Y[2]) * recip(Y[0]));
+    if (!finite_r(rho) || !finite_r(p)) return true;    // Step 4, CAD
+    if (!gt0_num(rho) || !gt0_num(p)) return true;       // Step 5, PAD
+  }
   if (verdict == kVerdictAccept) return false;
   const bool two = g.dim == 2;  // 1D: the x terms and the W/E neighbours only
   if (verdict == kVerdictNone && D.csd_on) {           // Step 6, CSD
@@ -1274,7 +1278,7 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
     rmin = lt_ieee(r, rmin) ? r : rmin;
     rmax = lt_ieee(rmax, r) ? r : rmax;
   }
-  if (verdict == kVerdictNone) {
+  if (verdict == kVerdictNone || verdict == kVerdictCsdFailed) {
     if (lt_ieee(rmax - rmin, det_c<Real>(D.plateau_thr, D.plateau_thr_f))) {  // Step 7
       verdict = kVerdictAccept;
       return false;
@@ -1422,6 +1426,70 @@ __device__ __forceinline__ void queue_push(bool flag, int cell, int* queue, int*
   if (flag) queue[base + __popc(m & ((1u << lane) - 1u))] = cell;
 }
 
+// Steps 4-6 of a cell in float, FP64 path, where the float values decide them
+// whatever the rounding: kVerdictAccept (CAD, PAD and CSD pass),
+// kVerdictCsdFailed (CAD and PAD pass, CSD fails) or kVerdictNone (too close
+// to a threshold, or CAD or PAD may fail).  Few cells are close, and an FP64
+// operation costs 64 times a float one: 0.26 ms a launch at 4096 x 1024 (the
+// candidate and the RK sums) for 0.78 with the tests in FP64.
+// The double -> float cut is below 2^-23 relative and so is every float
+// operation; |u|, K = |m|^2 / (2 rho) and E carry at most 8 such errors, so
+// 2^-19 of their magnitudes bounds each.  A NaN or an infinity fails every
+// comparison.
+struct QuickPrim {
+  float w, p, dp;  // normal velocity, pressure / (gamma - 1) and its error bound
+};
+__device__ __forceinline__ float cut_float(double x) {
+  // the leading 24 bits; below the float range zero, beyond it an infinity
+  const uint32_t h = fxd_hi(x), l = fxd_lo(x);
+  int t = (int)(h & 0x7fffffffu) - (896 << 20);
+  t = t < 0 ? 0 : t;
+  const uint32_t b = t >= (255 << 20) ? 0x7f800000u : ((uint32_t)t << 3 | (t ? l >> 29 : 0u));
+  return __int_as_float((int)(b | (h & 0x80000000u)));
+}
+__device__ __forceinline__ QuickPrim quick_prim(double r, double mn, double mt, double E) {
+  const float rf = cut_float(r), nf = cut_float(mn), tf = cut_float(mt), ef = cut_float(E);
+  const float ir = recip(rf);
+  const float K = 0.5f * (nf * nf + tf * tf) * ir;
+  QuickPrim q;
+  q.w = nf * ir;
+  q.p = rf > 0x1p-100f ? ef - K : -1.0f;
+  q.dp = 0x1p-19f * (fabsf(ef) + K);
+  return q;
+}
+template <class LX>
+__device__ __forceinline__ int quick_csd(const LX& X, const Grid& g, const Detect& D,
+                                         const double* Y) {
+  if (!D.csd_on) return kVerdictNone;
+  const QuickPrim y = quick_prim(Y[0], Y[1], Y[2], Y[3]);
+  const float r = cut_float(Y[0]);
+  bool sure = r > 0x1p-100f && r < 0x1p100f && y.p - y.dp > 0x1p-100f && y.p < 0x1p100f;
+  float div = 0.0f, ediv = 0.0f, most = 0.0f, least = 0.0f;  // bounds of the pressure gradient
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    if (d == 1 && g.dim != 2) break;
+    const int a = d == 0, b = d == 1;
+    const QuickPrim e = quick_prim(X(0, a, b), X(1 + d, a, b), X(2 - d, a, b), X(3, a, b));
+    const QuickPrim w = quick_prim(X(0, -a, -b), X(1 + d, -a, -b), X(2 - d, -a, -b), X(3, -a, -b));
+    const float h = d == 0 ? D.hx_f : D.hy_f;
+    div += (e.w - w.w) * h;
+    ediv += (fabsf(e.w) + fabsf(w.w)) * h;
+    const float low = fminf(e.p - e.dp, w.p - w.dp), high = fminf(e.p + e.dp, w.p + w.dp);
+    const float jump = fabsf(e.p - w.p), off = e.dp + w.dp;
+    sure = sure && low > 0x1p-100f && high < 0x1p100f;
+    most += (jump + off) * h * recip(low);
+    least += fmaxf(jump - off, 0.0f) * h * recip(high);
+  }
+  // 2^-18 of the sums of magnitudes covers the errors of the sums too
+  const float up = 1.0f + 0x1p-18f, down = 1.0f - 0x1p-18f;
+  if (!sure) return kVerdictNone;
+  if (div - 0x1p-18f * ediv >= -D.sigma_v_f * down && most * up <= D.sigma_p_f * down)
+    return kVerdictAccept;
+  if (div + 0x1p-18f * ediv < -D.sigma_v_f * up || least * down > D.sigma_p_f * up)
+    return kVerdictCsdFailed;
+  return kVerdictNone;
+}
+
 // first-pass update of cell (i,j) (if in range): candidate, detection,
 // RK combination; troubled cells go to the queue as cell_off + local index.
 // D and d2x/d2y are the detection constants and App. B weights of the grid.
@@ -1440,8 +1508,14 @@ __device__ __forceinline__ void update_cell_w(const StageArgs<Real>& A, const Gr
     const int top = Wd.top;
     if (top != 0) {
       int verdict = kVerdictNone;
-      bad = face_state_bad<Real>(A, g, i, j) ||
-            troubled<Real>(A.Xr, g, D, d2x, d2y, i, j, Y, verdict);
+      bad = face_state_bad<Real>(A, g, i, j);
+      if (!bad) {
+        if constexpr (sizeof(Real) == sizeof(double))
+          verdict = quick_csd(
+              [&](int v, int a, int b) { return xload<Real>(A.Xr, g, v, i + a, j + b); }, g, D, Y);
+        if (verdict != kVerdictAccept)
+          bad = troubled<Real>(A.Xr, g, D, d2x, d2y, i, j, Y, verdict);
+      }
       if (verdict != kVerdictNone) keep_verdict<Real>(A, g, i, j, verdict);
     } else {
       Real y[4] = {(Real)Y[0], (Real)Y[1], (Real)Y[2], (Real)Y[3]};

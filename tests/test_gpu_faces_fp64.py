@@ -50,3 +50,25 @@ def test_large_contrast_and_zero_momentum(R):
     Ug, Uo, og, oo, bg, bo = step_both(p, U)
     assert relerr(Ug, Uo) <= 1e-12
     assert (og == oo).all() and (bg == bo).all()
+
+
+@pytest.mark.parametrize("spread", [1e-3, 1e-5, 1e-7, 1e-9])
+def test_detection_near_the_csd_threshold(spread):
+    """first-pass flags where the normalised pressure gradient straddles its
+    threshold (5) by relative steps of `spread`: the FP64 path's float
+    pre-test may only decide what FP64 decides the same"""
+    nx, ny = 61, 40
+    p = I.uniform(nx, ny, R=2, state=(1.0, 0.0, 0.0, 1.0), bc="outflow", ell=0.2)
+    dx = 1.0 / nx
+    # p[i+1] / p[i-1] = 1 + 2 dx s[i], s around 5 (pW is the smaller side)
+    s = 5.0 * (1.0 + spread * (np.arange(nx) - nx // 2))
+    pr = np.ones(nx)
+    for i in range(1, nx - 1):
+        pr[i + 1] = pr[i - 1] * (1.0 + 2.0 * dx * s[i])
+    rho = 1.0 + 0.1 * np.random.default_rng(3).standard_normal((ny, nx))
+    U = np.zeros((4, ny, nx))
+    U[0] = rho
+    U[3] = pr[None, :] / 0.4
+    Ug, Uo, og, oo, bg, bo = step_both(p, U)
+    assert 0 < bo[0].sum() < bo[0].size
+    assert (bg[0] == bo[0]).all() and (og[0] == oo[0]).all()
