@@ -691,23 +691,34 @@ thread_local int g_pdl = 0;
 int fx_segments(int nx) { return (nx + 1 + kSegFaces - 1) / kSegFaces; }
 int fx_chunks(int ny, int nb) { return (ny + 1 + 4 * nb - 2) / (4 * nb - 1); }
 
-// bands a block: the FP64 pipe is each SM's own, so the time is that of the
-// SM with the most bands, ceil(blocks / SMs) blocks of nb bands; of equal
-// choices the longer block, which reconstructs fewer rows twice
-int fx_bands(int nprob, const int* nx, const int* ny) {
+static int sm_count() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       sms <= 0) {
     cudaGetLastError();
-    sms = 152;
+    return 152;
   }
+  return sms;
+}
+
+int fx_grid(int units) {
+  const int sms = sm_count();
+  return units < sms ? units : sms;
+}
+
+// bands a unit: the time is that of the SM with the most bands,
+// ceil(units / SMs) units of nb bands (the first of which leaves a quarter of
+// its faces out); of equal choices the longer unit, which reconstructs fewer
+// rows twice
+int fx_bands(int nprob, const int* nx, const int* ny) {
+  const int sms = sm_count();
   int best = 1;
   long long best_cost = 0;
   for (int nb = 1; nb <= 16; ++nb) {
-    long long blocks = 0;
-    for (int p = 0; p < nprob; ++p) blocks += (long long)fx_segments(nx[p]) * fx_chunks(ny[p], nb);
-    const long long cost = (blocks + sms - 1) / sms * nb;
+    long long units = 0;
+    for (int p = 0; p < nprob; ++p) units += (long long)fx_segments(nx[p]) * fx_chunks(ny[p], nb);
+    const long long cost = (units + sms - 1) / sms * nb;
     if (nb == 1 || cost <= best_cost) {
       best = nb;
       best_cost = cost;

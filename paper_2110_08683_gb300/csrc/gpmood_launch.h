@@ -35,11 +35,13 @@ inline cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
   return launch_ks(kernel, grid, block, 0, st, args...);
 }
 
-// the FP64 face kernel's blocks: fx_bands() bands of 4 rows each, covering
-// 4 nb - 1 rows of faces (of ny + 1) of a segment of 31
+// the FP64 face kernel's units of work: fx_bands() bands of 4 rows each,
+// covering 4 nb - 1 rows of faces (of ny + 1) of a segment of 31; its grid
+// (one block an SM walks the units)
 int fx_segments(int nx);
 int fx_chunks(int ny, int nb);
 int fx_bands(int nprob, const int* nx, const int* ny);
+int fx_grid(int units);
 
 template <class Real>
 struct Launch {

@@ -26,11 +26,11 @@ template <class Real>  // double; a template, so that only its own files instant
 static cudaError_t faces_fx(int top, int dirs, const StageArgs<Real>& A, const Grid& g,
                             const ParityW<Real>& W, cudaStream_t st) {
   const int nseg = fx_segments(g.nx), nb = fx_bands(1, &g.nx, &g.ny);
-  const long long blocks = (long long)nseg * fx_chunks(g.ny, nb);
+  const int units = nseg * fx_chunks(g.ny, nb);
   return with_radius(top, [&](auto r) {
     constexpr int R = decltype(r)::value;
-    return launch_ks(k_faces_fx<R>, dim3((unsigned)blocks), dim3(32 * kFxRows),
-                     sizeof(FxShared<R>), st, A, g, W, nseg, nb, dirs);
+    return launch_ks(k_faces_fx<R>, dim3(fx_grid(units)), dim3(kFxThreads), sizeof(FxShared<R>),
+                     st, A, g, W, nseg, nb, units, dirs);
   });
 }
 
@@ -84,8 +84,11 @@ template <class Real>
 cudaError_t Launch<Real>::prepare() {
   return every_radius<Real>([](auto r) {
     constexpr int R = decltype(r)::value;
-    if constexpr (sizeof(Real) == sizeof(double)) return shared_limit(k_faces_fx<R>, sizeof(FxShared<R>));
-    else return shared_limit(k_faces_xy<R, Real>, sizeof(XYShared<R, Real>));
+    if constexpr (sizeof(Real) == sizeof(double)) {
+      return shared_limit(k_faces_fx<R>, sizeof(FxShared<R>));
+    } else {
+      return shared_limit(k_faces_xy<R, Real>, sizeof(XYShared<R, Real>));
+    }
   });
 }
 
@@ -162,8 +165,8 @@ cudaError_t LaunchB<Real>::faces_xy(int top, const StageArgs<Real>& B, const Pro
   return with_radius(top, [&](auto r) {
     constexpr int R = decltype(r)::value;
     if constexpr (sizeof(Real) == sizeof(double))
-      return launch_ks(k_faces_fx_batch<R>, dim3(nitems), dim3(32 * kFxRows), sizeof(FxShared<R>),
-                       st, B, probs, psc, items, W);
+      return launch_ks(k_faces_fx_batch<R>, dim3(fx_grid(nitems)), dim3(kFxThreads),
+                       sizeof(FxShared<R>), st, B, probs, psc, items, nitems, W);
     else
       return launch_ks(k_faces_xy_batch<R, Real>, dim3(nitems), dim3(32, kXYRows),
                        sizeof(XYShared<R, Real>), st, B, probs, psc, items, W);
