@@ -62,6 +62,7 @@ struct gpmood_s {
   // steps can be queued without reading anything back; the host settles its
   // buffer rotation from the device's step count when it next synchronises
   int gated_ok;              // 0 not yet known, 1 plain graphs gated, -1 gating unavailable
+  int one_block;             // 1: 1D steps by the one-block kernel where they need no graph
   int pdl;                   // 1: programmatic dependent launch between step kernels
   int pend;                  // steps queued since the last settle
   int sync_cur;              // rotation at the last settle
@@ -322,6 +323,7 @@ int step_base_launches(int nstages, int face_kernels, int gated) {
 // first-pass face kernels a stage: 1 (fused, or 1D), 2 (split 2D)
 int face_kernels(const gpmood_t h) { return (h->g.dim == 2 && h->split_faces) ? 2 : 1; }
 int step_launches(const gpmood_t h, int gated) {
+  if (gated && h->one_block) return 1;
   return step_base_launches(h->sch.nstages, face_kernels(h), gated);
 }
 
@@ -339,6 +341,7 @@ MoodArgs mood_args(gpmood_t h) {
   M.queue[1] = h->queue[1];
   M.stamp = h->stamp;
   M.stamp_stride = (long long)h->g.nx * h->g.ny;
+  M.count = &h->sc->count[0];
   M.sc = h->sc;
   return M;
 }
@@ -613,6 +616,28 @@ int capture_step(gpmood_t h, int cur, int prof, int record, cudaGraphExec_t* out
   return rc;
 }
 
+// `steps` steps of a short 1D problem in one launch (each gated like a queued
+// step of the graphs)
+int launch_steps_1d(gpmood_t h, int steps) {
+  Steps1D S;
+  for (int k = 0; k < 5; ++k) S.U[k] = h->U[k];
+  S.Fx = (double*)h->Fx;
+  S.Fy = (double*)h->Fy;
+  S.fb = h->fb;
+  S.ord = h->ord;
+  S.first = h->first;
+  S.stamp = h->stamp;
+  S.queue[0] = h->queue[0];
+  S.queue[1] = h->queue[1];
+  S.sc = h->sc;
+  S.sch = h->sch;
+  S.rot = h->cur;
+  S.nsteps = steps;
+  g_pdl = 0;
+  CK(Launch<double>::steps_1d(h->cas.top, S, h->g, h->det, h->pw64, h->dw64, h->cas, h->stream));
+  return GPMOOD_OK;
+}
+
 int graph_step(gpmood_t h, double cfl, double fixed_dt, int clip, double t_end,
                double* tape = nullptr, uint8_t* otape = nullptr, void* stape = nullptr) {
   if (!h->has_state) return set_err(h, GPMOOD_E_NOSTATE);
@@ -621,16 +646,22 @@ int graph_step(gpmood_t h, double cfl, double fixed_dt, int clip, double t_end,
   if (h->eager) return do_step(h, cfl, fixed_dt, clip, t_end, tape, otape, stape);
   const int record = tape ? 1 : 0;
   const int prof = (h->prof_on && !record) ? 1 : 0;
+  const int one_block = h->one_block && !record && !prof;
   cudaGraphExec_t& ge = h->gexec[h->cur][record ? 2 : prof];
-  if (!ge) {
+  if (!ge && !one_block) {
     rc = capture_step(h, h->cur, prof, record, &ge);
     if (rc) return rc;
   }
-  const int gated = !record && !prof && h->gated_ok == 1;
+  const int gated = !record && !prof && (one_block || h->gated_ok == 1);
   write_control(h, cfl, fixed_dt, clip, t_end, tape, otape, stape);
   rc = push_control(h);
   if (rc) return rc;
-  CK(cudaGraphLaunch(ge, h->stream));
+  if (one_block) {
+    rc = launch_steps_1d(h, 1);
+    if (rc) return rc;
+  } else {
+    CK(cudaGraphLaunch(ge, h->stream));
+  }
   rc = pull_scalars(h);
   if (rc) return rc;
   if (prof) {
@@ -660,8 +691,18 @@ int graph_step(gpmood_t h, double cfl, double fixed_dt, int clip, double t_end,
 // queue one step without waiting (plain gated graphs).  Eager handles,
 // profiled steps and handles whose driver refused the gate step
 // synchronously instead.
-int graph_step_async(gpmood_t h, double cfl, double fixed_dt, int clip, double t_end) {
+int graph_step_async(gpmood_t h, double cfl, double fixed_dt, int clip, double t_end,
+                     int steps = 1) {
   if (!h->has_state) return set_err(h, GPMOOD_E_NOSTATE);
+  if (h->one_block && !h->eager && !h->prof_on) {
+    write_control(h, cfl, fixed_dt, clip, t_end);
+    int rc = push_control_if_changed(h);
+    if (!rc) rc = launch_steps_1d(h, steps);
+    if (rc) return rc;
+    h->cur = (h->cur + steps * h->sch.advance) % h->sch.nbuf;
+    h->pend += steps;
+    return GPMOOD_OK;
+  }
   if (h->eager || h->prof_on || h->gated_ok < 0) return graph_step(h, cfl, fixed_dt, clip, t_end);
   cudaGraphExec_t& ge = h->gexec[h->cur][0];
   if (!ge) {
@@ -877,6 +918,7 @@ int gpmood_create(const gpmood_grid* grid, double gamma, int R_max, double ell,
     delete h;
     return GPMOOD_E_CUDA;
   }
+  h->one_block = one_d && h->precision == GPMOOD_FP64 && g.nx <= kMaxCells1D && !h->split_faces;
   h->coop = 1;
   h->mood_blocks = h->precision == GPMOOD_FP32 ? Launch<float>::mood_loop_blocks()
                                                : Launch<double>::mood_loop_blocks();
@@ -1112,8 +1154,9 @@ int gpmood_run(gpmood_t h, double t_end, double cfl, long long* nsteps_out) {
     long long est = 1;
     if (dt > 0.0 && isfinite(dt)) est = (long long)ceil((t_end - t) / dt) + 1;
     const int chunk = (int)(est < 1 ? 1 : (est > 64 ? 64 : est));
-    for (int k = 0; k < chunk; ++k) {
-      rc = graph_step_async(h, cfl, 0.0, 1, t_end);
+    const int each = h->one_block && !h->eager && !h->prof_on ? chunk : 1;  // steps a launch
+    for (int k = 0; k < chunk; k += each) {
+      rc = graph_step_async(h, cfl, 0.0, 1, t_end, each);
       if (rc) return rc;
       // a step taken synchronously (eager or profiled handles) has updated
       // the host scalars: stop at t_end as the device gate would

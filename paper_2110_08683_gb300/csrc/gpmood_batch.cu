@@ -398,6 +398,7 @@ int mood_loop_b(gpmood_batch_t b, const StageArgs<Real>& A, int s, const DirectW
   M.queue[1] = b->queue[1];
   M.stamp = b->stamp;
   M.stamp_stride = b->total_cells;
+  M.count = &b->gsc->count[0];
   M.sc = b->gsc;
   cudaError_t e = LaunchB<Real>::mood_loop(A, M, b->probs, b->psc, b->nprob, D, b->cas, s,
                                            b->mood_blocks, b->coop, st);

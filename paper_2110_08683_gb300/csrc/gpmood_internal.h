@@ -234,7 +234,22 @@ struct MoodArgs {
   int* queue[2];
   uint32_t* stamp;
   long long stamp_stride;
+  int* count;        // troubled cells of the first pass
   Scalars* sc;
+};
+
+// a one-dimensional handle as the one-block step kernel sees it: its buffers,
+// the RK scheme, the buffer rotation and the steps to take
+constexpr int kMaxCells1D = 1024;
+struct Steps1D {
+  double* U[5];
+  double *Fx, *Fy;
+  uint8_t *fb, *ord, *first;
+  uint32_t* stamp;
+  int* queue[2];
+  Scalars* sc;
+  Scheme sch;
+  int rot, nsteps;
 };
 
 // state adjoints of the faces, [v][g][face]; faces of one direction

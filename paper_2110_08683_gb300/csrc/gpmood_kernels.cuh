@@ -566,10 +566,11 @@ __device__ __forceinline__ void load_cell(const double* X, const Grid& g, int i,
 // needs one reciprocal and no division).  False: no admissible step (the
 // rate NaN, infinite or zero; p / rho < 0 gives NaN).
 __device__ __forceinline__ bool cell_rate(const double* S, const Grid& g, double& rate) {
-  const double ir = recip(S[0]);
+  const double ir = pos_normal(S[0]) ? recip_int(S[0]) : recip(S[0]);
   const double u = S[1] * ir, v = S[2] * ir;
   const double p = (g.gamma - 1.0) * (S[3] - 0.5 * (S[1] * u + S[2] * v));
-  const double cs = sqrt(g.gamma * p * ir);
+  const double z = g.gamma * p * ir;
+  const double cs = pos_normal(z) ? sqrt_int(z) : sqrt(z);
   const double ax = (fabs(u) + cs) * g.inv_dx, ay = (fabs(v) + cs) * g.inv_dy;
   rate = (g.dim == 1 || lt_ieee(ay, ax)) ? ax : ay;  // a NaN state makes both rates NaN
   return pos_finite(rate);
@@ -1197,7 +1198,7 @@ __device__ __forceinline__ float to_real<float>(double x) { return fpb_double_to
 
 template <class Real>
 __device__ __forceinline__ Real xload(const Real* X, const Grid& g, int v, int i, int j) {
-  return __ldg(X + gidx(g, v, i, j));
+  return X[gidx(g, v, i, j)];  // not __ldg: the 1D step kernel has written X itself
 }
 
 // What Steps 6, 7 and 9 find depends on the stage input alone, not on the
@@ -1594,7 +1595,7 @@ __device__ __forceinline__ double fx_value(const double* X, int pitch, const int
 #pragma unroll
     for (int a = -KM; a <= KM; ++a) {
       const int ab = (a < 0 ? -a : a) + (b < 0 ? -b : b);
-      if (ab <= KM) x[k++] = ab <= K ? __ldg(X + (long long)b * pitch + a) : 0.0;
+      if (ab <= KM) x[k++] = ab <= K ? X[(long long)b * pitch + a] : 0.0;
     }
   uint32_t top = (uint32_t)FXD_EMIN << 20;
 #pragma unroll
@@ -2102,7 +2103,7 @@ __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArg
   const uint32_t* stamp = stamp_of(M, cur);
   // (in units of 100 cycles; the whole grid has two blocks an SM, the small
   // group one)
-  const int subs = (blocks == gridDim.x ? 2 : 4) * blocks;
+  const int subs = (blocks == gridDim.x && blocks > 1 ? 2 : 4) * blocks;
   int P = 4;
   long long best = 0;
 #pragma unroll
@@ -2145,7 +2146,7 @@ __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArg
       if (pl) {
         const int k = (pl >> 1) & 3, d = (pl >> 3) & 1;
         Xp += v * vsp + (right ? (d ? pp : 1) : 0);
-        st[src][lane & 7] = k == 0 ? __ldg(Xp)
+        st[src][lane & 7] = k == 0 ? *Xp
                                    : fx_value<2>(Xp, pp, S.z[k - 1][2 * d + right][pl >> 4], k, Wd.off);
       }
     }
@@ -2241,7 +2242,7 @@ __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs&
   // group of blocks has counts of its own, so a block that leaves the loop may
   // still read the old ones.
   __shared__ int one_next[2];
-  int n = *(volatile int*)&sc->count[0];
+  int n = *(volatile int*)M.count;
   const int nfirst = n;
   int slot = 0, iters = 0, total = n;
   uint32_t cur = sc->stamp_cur + 1;  // stamp of the cells of the first queue
@@ -2250,7 +2251,7 @@ __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs&
   if (threadIdx.x == 0) one_next[0] = one_next[1] = 0;
   bool ok = true;
   unsigned blocks = gridDim.x;  // that work on the queue
-  int* next = sc->next[0];
+  int* next = gridDim.x == 1 ? one_next : sc->next[0];
   auto barrier = [&]() {
     if (blocks == 1) {
       __syncthreads();
@@ -2320,7 +2321,7 @@ __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs&
     sc->iters[stage] = iters;
     sc->stamp_cur = cur;  // every value up to cur has been used
     // the queue is empty for the next stage, also after a failed loop
-    sc->count[0] = 0;
+    *M.count = 0;
   }
 }
 

@@ -51,6 +51,11 @@ struct Launch {
   // first pass: x and y faces in one launch (two-dimensional grids)
   static cudaError_t faces_xy(int top, const StageArgs<Real>& A, const Grid& g,
                               const ParityW<Real>& W, cudaStream_t st);
+  // S.nsteps whole steps of a 1D problem of at most kMaxCells1D cells in one
+  // block (FP64 only)
+  static cudaError_t steps_1d(int top, const Steps1D& S, const Grid& g, const Detect& D,
+                              const ParityW<Real>& W, const DirectW<Real>& Wd, const Cascade& C,
+                              cudaStream_t st);
   // once per process and device: kernel attributes (shared-memory limits)
   static cudaError_t prepare();
   static cudaError_t update_first(const StageArgs<Real>& A, const Grid& g, const Detect& D,

@@ -7,6 +7,7 @@
 #include "faces_fp64.cuh"
 #include "gpmood_kernels.cuh"
 #include "gpmood_launch.h"
+#include "steps_1d.cuh"
 
 namespace gpm {
 
@@ -81,11 +82,25 @@ static cudaError_t every_radius(F&& f) {
 }
 
 template <class Real>
+cudaError_t Launch<Real>::steps_1d(int top, const Steps1D& S, const Grid& g, const Detect& D,
+                                   const ParityW<Real>& W, const DirectW<Real>& Wd,
+                                   const Cascade& C, cudaStream_t st) {
+  if constexpr (sizeof(Real) == sizeof(double))
+    return with_radius(top, [&](auto r) {
+      constexpr int R = decltype(r)::value;
+      return launch_ks(k_steps_1d<R>, dim3(1), dim3(256), 8 * sizeof(double) * (g.nx + 2), st, S, g,
+                       D, W, Wd, C);
+    });
+  else return cudaErrorInvalidValue;
+}
+
+template <class Real>
 cudaError_t Launch<Real>::prepare() {
   return every_radius<Real>([](auto r) {
     constexpr int R = decltype(r)::value;
     if constexpr (sizeof(Real) == sizeof(double)) {
-      return shared_limit(k_faces_fx<R>, sizeof(FxShared<R>));
+      cudaError_t e = shared_limit(k_faces_fx<R>, sizeof(FxShared<R>));
+      return e != cudaSuccess ? e : shared_limit(k_steps_1d<R>, 8 * sizeof(double) * (kMaxCells1D + 2));
     } else {
       return shared_limit(k_faces_xy<R, Real>, sizeof(XYShared<R, Real>));
     }
