@@ -521,16 +521,18 @@ __device__ __forceinline__ void hll_x_fp64(const double* UL, const double* UR, d
                         __dmul_rn(L.u, UL[3] + L.p)};
   const double FR[4] = {UR[1], fma(UR[1], R.u, R.p), __dmul_rn(UR[1], vR),
                         __dmul_rn(R.u, UR[3] + R.p)};
-  const double iw = recip_int(SR - SL), SS = __dmul_rn(SL, SR);
+  // F = a F_L - b F_R + c (U_R - U_L), a = S_R / w, b = S_L / w, c = S_L S_R / w,
+  // w = S_R - S_L
+  const double iw = recip_int(SR - SL);
+  const double a = __dmul_rn(SR, iw), b = __dmul_rn(SL, iw), c = __dmul_rn(__dmul_rn(SL, SR), iw);
   const bool useL = ge0_num(SL), useR = !gt0_num(SR);
   const bool dom = L.ok && R.ok;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    // x-mirror: (L, R, S_L, S_R) -> (R', L', -S_R, -S_L) swaps the two
-    // products; each is rounded on its own so the mirror face negates exactly
-    const double a = __dmul_rn(SR, FL[v]), b = __dmul_rn(SL, FR[v]);
-    const double c = __dmul_rn(SS, UR[v] - UL[v]);
-    const double Fm = __dmul_rn(__dadd_rn(a - b, c), iw);
+    // x-mirror: (L, R, a, b, c) -> (R', L', -b, -a, c) swaps the two products;
+    // each is rounded on its own so the mirror face negates exactly
+    const double d = __dmul_rn(a, FL[v]) - __dmul_rn(b, FR[v]);
+    const double Fm = fma(c, UR[v] - UL[v], d);
     F[v] = useL ? FL[v] : (useR ? FR[v] : Fm);
     if (!dom) qnan(F[v]);
   }
