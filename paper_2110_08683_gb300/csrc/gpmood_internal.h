@@ -63,15 +63,13 @@ struct Scalars {
   unsigned long long rate_bits;  // running max of the CFL rate (|u|+c)/dx as ordered bits
   int err;                      // error bits (kErr*)
   int count[2];                 // troubled cells of the first pass (the first entry)
-  unsigned int small_count;     // barrier among the first kSmallBlocks blocks of the MOOD
-  unsigned int small_gen;       // loop kernel: arrivals and generation
   unsigned int stamp_cur;       // stamp of the cells in the current queue
   int iters[5], nbad_first[5], nbad_total[5], nfog_pad[5];  // per RK stage
   long long nsteps;
   long long launches;           // kernels launched by graph steps since the state was set
   int nactive;                  // batches: problems still advancing in this step
-  unsigned int bar_count;       // grid barrier of the MOOD loop kernel: arrivals
-  unsigned int bar_gen;         // and generation (count returns to 0 after each use)
+  unsigned long long bar_all;   // arrivals so far at the grid barrier of the MOOD loop kernel
+  unsigned long long bar_small; // and at the barrier of its first kSmallBlocks blocks
   int rate_ready;               // rate_bits holds the CFL rate of the current state
   int rate_bad;                 // and that state had a cell with no admissible rate
   int next[2][2];               // queue lengths of the MOOD loop's iterations, with the

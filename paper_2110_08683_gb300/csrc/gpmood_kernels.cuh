@@ -1211,14 +1211,127 @@ constexpr int kVerdictAccept = 1;  // accepted by CSD, the plateau or u2
 constexpr int kVerdictDmp = 2;     // CSD and plateau failed, u2 not looked at
 constexpr int kVerdictDmpOnly = 3; // and u2 failed: accepted by the DMP or not at all
 constexpr int kVerdictBits = 12;
-// (not kept: CAD and PAD passed and CSD failed, as quick_csd found)
-constexpr int kVerdictCsdFailed = 4;
+constexpr int kVerdictCsdFailed = 4;  // (not kept, see quick_csd)
 // (the other bits of the byte change in other phases only)
 template <class Real>
 __device__ __forceinline__ void keep_verdict(const StageArgs<Real>& A, const Grid& g, int i,
                                              int j, int verdict) {
   uint8_t* b = A.fbx + (long long)j * (g.nx + 1) + i;
   *b = (uint8_t)((*b & ~kVerdictBits) | verdict << 2);
+}
+
+// Detection in float, FP64 path, where the float values decide a test whatever
+// the rounding.  quick_csd: kVerdictAccept (CAD, PAD and CSD pass),
+// kVerdictCsdFailed (CAD and PAD pass, CSD fails) or kVerdictNone (too close
+// to a threshold, or CAD or PAD may fail).  Few cells are close, and an FP64
+// operation costs 64 times a float one: 0.26 ms a launch at 4096 x 1024 (the
+// candidate and the RK sums) for 0.78 with the tests in FP64.
+// The double -> float cut is below 2^-23 relative and so is every float
+// operation; |u|, K = |m|^2 / (2 rho) and E carry at most 8 such errors, so
+// 2^-19 of their magnitudes bounds each.  A NaN or an infinity fails every
+// comparison.
+struct QuickPrim {
+  float w, p, dp;  // normal velocity, pressure / (gamma - 1) and its error bound
+};
+__device__ __forceinline__ float cut_float(double x) {
+  // the leading 24 bits; below the float range zero, beyond it an infinity
+  const uint32_t h = fxd_hi(x), l = fxd_lo(x);
+  int t = (int)(h & 0x7fffffffu) - (896 << 20);
+  t = t < 0 ? 0 : t;
+  const uint32_t b = t >= (255 << 20) ? 0x7f800000u : ((uint32_t)t << 3 | (t ? l >> 29 : 0u));
+  return __int_as_float((int)(b | (h & 0x80000000u)));
+}
+__device__ __forceinline__ QuickPrim quick_prim(double r, double mn, double mt, double E) {
+  const float rf = cut_float(r), nf = cut_float(mn), tf = cut_float(mt), ef = cut_float(E);
+  const float ir = recip(rf);
+  const float K = 0.5f * (nf * nf + tf * tf) * ir;
+  QuickPrim q;
+  q.w = nf * ir;
+  q.p = rf > 0x1p-100f ? ef - K : -1.0f;
+  q.dp = 0x1p-19f * (fabsf(ef) + K);
+  return q;
+}
+// CAD and PAD pass
+__device__ __forceinline__ bool quick_pad(const double* Y) {
+  const QuickPrim y = quick_prim(Y[0], Y[1], Y[2], Y[3]);
+  const float r = cut_float(Y[0]);
+  return r > 0x1p-100f && r < 0x1p100f && y.p - y.dp > 0x1p-100f && y.p < 0x1p100f;
+}
+template <class LX>
+__device__ __forceinline__ int quick_csd(const LX& X, const Grid& g, const Detect& D,
+                                         const double* Y) {
+  if (!D.csd_on) return kVerdictNone;
+  bool sure = quick_pad(Y);
+  float div = 0.0f, ediv = 0.0f, most = 0.0f, least = 0.0f;  // bounds of the pressure gradient
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    if (d == 1 && g.dim != 2) break;
+    const int a = d == 0, b = d == 1;
+    const QuickPrim e = quick_prim(X(0, a, b), X(1 + d, a, b), X(2 - d, a, b), X(3, a, b));
+    const QuickPrim w = quick_prim(X(0, -a, -b), X(1 + d, -a, -b), X(2 - d, -a, -b), X(3, -a, -b));
+    const float h = d == 0 ? D.hx_f : D.hy_f;
+    div += (e.w - w.w) * h;
+    ediv += (fabsf(e.w) + fabsf(w.w)) * h;
+    const float low = fminf(e.p - e.dp, w.p - w.dp), high = fminf(e.p + e.dp, w.p + w.dp);
+    const float jump = fabsf(e.p - w.p), off = e.dp + w.dp;
+    sure = sure && low > 0x1p-100f && high < 0x1p100f;
+    most += (jump + off) * h * recip(low);
+    least += fmaxf(jump - off, 0.0f) * h * recip(high);
+  }
+  // 2^-18 of the sums of magnitudes covers the errors of the sums too
+  const float up = 1.0f + 0x1p-18f, down = 1.0f - 0x1p-18f;
+  if (!sure) return kVerdictNone;
+  if (div - 0x1p-18f * ediv >= -D.sigma_v_f * down && most * up <= D.sigma_p_f * down)
+    return kVerdictAccept;
+  if (div + 0x1p-18f * ediv < -D.sigma_v_f * up || least * down > D.sigma_p_f * up)
+    return kVerdictCsdFailed;
+  return kVerdictNone;
+}
+
+// u2: 1 passes, 0 fails, -1 too close.  With S the sum of |w| |rho| of a
+// curvature (the largest of the five) a float curvature is within 2^-21 S:
+// cuts of 2^-23 in both factors, a rounded product, four rounded sums.
+template <class LX>
+__device__ __forceinline__ int quick_u2(const LX& X, const Grid& g, const Detect& D,
+                                        const double* d2x, const double* d2y) {
+  const bool two = g.dim == 2;
+  const int ci[5] = {0, -1, 1, 0, 0}, cj[5] = {0, 0, 0, 1, -1};
+  const float lowd = D.delta_f * (1.0f - 0x1p-18f), highd = D.delta_f * (1.0f + 0x1p-18f);
+  const float up = 1.0f + 0x1p-18f, down = 1.0f - 0x1p-18f;
+  int pass = 1;
+#pragma unroll
+  for (int d = 0; d < 2; ++d) {
+    if (d == 1 && !two) break;
+    float w[5];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) w[m] = cut_float((d == 0 ? d2x : d2y)[m]);
+    float cmin = 0.0f, cmax = 0.0f, S = 0.0f;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+      if (m >= 3 && !two) break;
+      const int a = ci[m], b = cj[m];
+      const float t[5] = {w[0] * cut_float(X(0, a, b - 1)), w[1] * cut_float(X(0, a - 1, b)),
+                          w[2] * cut_float(X(0, a, b)), w[3] * cut_float(X(0, a + 1, b)),
+                          w[4] * cut_float(X(0, a, b + 1))};
+      const float k = ((t[0] + t[4]) + (t[1] + t[3])) + t[2];
+      S = fmaxf(S, fabsf(t[0]) + fabsf(t[1]) + fabsf(t[2]) + fabsf(t[3]) + fabsf(t[4]));
+      cmin = m == 0 ? k : fminf(cmin, k);
+      cmax = m == 0 ? k : fmaxf(cmax, k);
+    }
+    const float e = 0x1p-20f * S;
+    if (!(S < 0x1p60f)) return -1;  // also a NaN
+    // the product over the intervals of cmin and cmax
+    const float p1 = (cmin - e) * (cmax - e), p2 = (cmin - e) * (cmax + e);
+    const float p3 = (cmin + e) * (cmax - e), p4 = (cmin + e) * (cmax + e);
+    const float plo = fminf(fminf(p1, p2), fminf(p3, p4)), phi = fmaxf(fmaxf(p1, p2), fmaxf(p3, p4));
+    const bool same = plo > 0.0f || -plo < lowd, apart = phi < 0.0f && -phi > highd;
+    const float amin = fabsf(cmin), amax = fabsf(cmax), big = fmaxf(amin, amax);
+    const bool ua = big + e < lowd, not_ua = big - e > highd;
+    const bool ub = amin - e > 0.5f * (amax + e) * up, not_ub = amin + e < 0.5f * (amax - e) * down;
+    if (apart || (not_ua && not_ub)) return 0;
+    if (!(same && (ua || ub))) pass = -1;
+  }
+  return pass;
 }
 
 // X(v, a, b): variable v of the ghosted stage input at (i + a, j + b), in
@@ -1232,14 +1345,27 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
   Real Y[4] = {to_real<Real>(Yd[0]), to_real<Real>(Yd[1]), to_real<Real>(Yd[2]),
                to_real<Real>(Yd[3])};
   Real rho = Y[0];
-  if (verdict != kVerdictCsdFailed) {
+  bool sure = false, csd_failed = false;  // CAD and PAD passed; CSD failed
+  if constexpr (sizeof(Real) == sizeof(double)) {
+    if (verdict == kVerdictNone) {
+      const int q = quick_csd(X, g, D, Yd);
+      if (q == kVerdictAccept) {
+        verdict = kVerdictAccept;
+        return false;
+      }
+      sure = csd_failed = q == kVerdictCsdFailed;
+    } else {
+      sure = quick_pad(Yd);
+    }
+  }
+  if (!sure) {
     Real p = gm1 * (Y[3] - Real(0.5) * (Y[1] * Y[1] + Y[2] * Y[2]) * recip(Y[0]));
     if (!finite_r(rho) || !finite_r(p)) return true;    // Step 4, CAD
     if (!gt0_num(rho) || !gt0_num(p)) return true;       // Step 5, PAD
   }
   if (verdict == kVerdictAccept) return false;
   const bool two = g.dim == 2;  // 1D: the x terms and the W/E neighbours only
-  if (verdict == kVerdictNone && D.csd_on) {           // Step 6, CSD
+  if (verdict == kVerdictNone && !csd_failed && D.csd_on) {  // Step 6, CSD
     Real rE = X(0, 1, 0), rW = X(0, -1, 0);
     Real rN = X(0, 0, 1), rS = X(0, 0, -1);
     Real mxE = X(1, 1, 0), mxW = X(1, -1, 0);
@@ -1281,7 +1407,7 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
     rmin = lt_ieee(r, rmin) ? r : rmin;
     rmax = lt_ieee(rmax, r) ? r : rmax;
   }
-  if (verdict == kVerdictNone || verdict == kVerdictCsdFailed) {
+  if (verdict == kVerdictNone) {
     if (lt_ieee(rmax - rmin, det_c<Real>(D.plateau_thr, D.plateau_thr_f))) {  // Step 7
       verdict = kVerdictAccept;
       return false;
@@ -1290,6 +1416,13 @@ __device__ __forceinline__ bool troubled_at(const LX& X, const Grid& g, const De
   }
   if (le_ieee(rmin, rho) && le_ieee(rho, rmax)) return false;     // Step 8, DMP
   if (verdict == kVerdictDmpOnly) return true;
+  if constexpr (sizeof(Real) == sizeof(double)) {
+    const int q = quick_u2(X, g, D, d2x, d2y);
+    if (q >= 0) {
+      verdict = q ? kVerdictAccept : kVerdictDmpOnly;
+      return q == 0;
+    }
+  }
   // Step 9, u2 with the App. B second-derivative weights (R=1 stencil in
   // the order b=-1: (0,-1); b=0: (-1,0),(0,0),(1,0); b=1: (0,1))
   const int ci[5] = {0, -1, 1, 0, 0}, cj[5] = {0, 0, 0, 1, -1};
@@ -1352,39 +1485,33 @@ __device__ __forceinline__ StageC stage_coeffs(const StageArgs<Real>& A, const G
   return StageC{hdt * g.inv_dx, hdt * g.inv_dy};
 }
 
-// per variable two differences and two fmas
-template <class Real>
+// per variable two differences and two fmas: NV variables from v0 on
+template <int NV, class Real>
 __device__ __forceinline__ void candidate(const StageArgs<Real>& A, const Grid& g, int i, int j,
-                                          StageC k, double* Y) {
+                                          int v0, StageC k, double* Y) {
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
+  for (int n = 0; n < NV; ++n) {
+    const int v = v0 + n;
     double fe = A.Fx[fxidx(g, v, i + 1, j)], fw = A.Fx[fxidx(g, v, i, j)];
     double gn = A.Fy[fyidx(g, v, i, j + 1)], gs = A.Fy[fyidx(g, v, i, j)];
-    Y[v] = fma(-k.cx, fe - fw, fma(-k.cy, gn - gs, A.X[gidx(g, v, i, j)]));
+    Y[n] = fma(-k.cx, fe - fw, fma(-k.cy, gn - gs, A.X[gidx(g, v, i, j)]));
   }
-}
-template <class Real>
-__device__ __forceinline__ void candidate(const StageArgs<Real>& A, const Grid& g, int i, int j,
-                                          double dt, double* Y) {
-  candidate<Real>(A, g, i, j, stage_coeffs<Real>(A, g, dt), Y);
 }
 
-// u0: U^n of the cell (read where ca is not zero)
+// the SSP-RK combination of the candidate
+// one value of it, at index k: Y the candidate, u0 U^n (read where ca is not
+// zero)
 template <class Real>
-__device__ __forceinline__ void combine_store(const StageArgs<Real>& A, const Grid& g, int i,
-                                              int j, const double* Y, const double* u0) {
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    long long k = gidx(g, v, i, j);
-    // the first stage's combination is the candidate itself (ca = 0, cb = 1);
-    // compared as integers, an FP64 compare costs what a product does
-    const double o = __double_as_longlong(A.ca) != 0 ? fma(A.ca, u0[v], A.cb * Y[v])
-                     : __double_as_longlong(A.cb) == 0x3ff0000000000000ll ? Y[v]
-                                                                          : A.cb * Y[v];
-    A.out[k] = o;
-    if constexpr (sizeof(Real) == sizeof(float)) A.outr[k] = fpb_double_to_float_rn(o);
-    if (A.out2) A.out2[k] = fma(A.wa, A.W[k], A.wb * Y[v]);
-  }
+__device__ __forceinline__ void combine_one(const StageArgs<Real>& A, long long k, double Y,
+                                            double u0) {
+  // the first stage's combination is the candidate itself (ca = 0, cb = 1);
+  // compared as integers, an FP64 compare costs what a product does
+  const double o = __double_as_longlong(A.ca) != 0 ? fma(A.ca, u0, A.cb * Y)
+                   : __double_as_longlong(A.cb) == 0x3ff0000000000000ll ? Y
+                                                                        : A.cb * Y;
+  A.out[k] = o;
+  if constexpr (sizeof(Real) == sizeof(float)) A.outr[k] = fpb_double_to_float_rn(o);
+  if (A.out2) A.out2[k] = fma(A.wa, A.W[k], A.wb * Y);
 }
 template <class Real>
 __device__ __forceinline__ void combine_store(const StageArgs<Real>& A, const Grid& g, int i,
@@ -1394,7 +1521,8 @@ __device__ __forceinline__ void combine_store(const StageArgs<Real>& A, const Gr
 #pragma unroll
     for (int v = 0; v < 4; ++v) u0[v] = A.U0[gidx(g, v, i, j)];
   }
-  combine_store<Real>(A, g, i, j, Y, u0);
+#pragma unroll
+  for (int v = 0; v < 4; ++v) combine_one<Real>(A, gidx(g, v, i, j), Y[v], u0[v]);
 }
 
 // a load issued where it stands: the MOOD loop's few cells an iteration leave
@@ -1429,70 +1557,6 @@ __device__ __forceinline__ void queue_push(bool flag, int cell, int* queue, int*
   if (flag) queue[base + __popc(m & ((1u << lane) - 1u))] = cell;
 }
 
-// Steps 4-6 of a cell in float, FP64 path, where the float values decide them
-// whatever the rounding: kVerdictAccept (CAD, PAD and CSD pass),
-// kVerdictCsdFailed (CAD and PAD pass, CSD fails) or kVerdictNone (too close
-// to a threshold, or CAD or PAD may fail).  Few cells are close, and an FP64
-// operation costs 64 times a float one: 0.26 ms a launch at 4096 x 1024 (the
-// candidate and the RK sums) for 0.78 with the tests in FP64.
-// The double -> float cut is below 2^-23 relative and so is every float
-// operation; |u|, K = |m|^2 / (2 rho) and E carry at most 8 such errors, so
-// 2^-19 of their magnitudes bounds each.  A NaN or an infinity fails every
-// comparison.
-struct QuickPrim {
-  float w, p, dp;  // normal velocity, pressure / (gamma - 1) and its error bound
-};
-__device__ __forceinline__ float cut_float(double x) {
-  // the leading 24 bits; below the float range zero, beyond it an infinity
-  const uint32_t h = fxd_hi(x), l = fxd_lo(x);
-  int t = (int)(h & 0x7fffffffu) - (896 << 20);
-  t = t < 0 ? 0 : t;
-  const uint32_t b = t >= (255 << 20) ? 0x7f800000u : ((uint32_t)t << 3 | (t ? l >> 29 : 0u));
-  return __int_as_float((int)(b | (h & 0x80000000u)));
-}
-__device__ __forceinline__ QuickPrim quick_prim(double r, double mn, double mt, double E) {
-  const float rf = cut_float(r), nf = cut_float(mn), tf = cut_float(mt), ef = cut_float(E);
-  const float ir = recip(rf);
-  const float K = 0.5f * (nf * nf + tf * tf) * ir;
-  QuickPrim q;
-  q.w = nf * ir;
-  q.p = rf > 0x1p-100f ? ef - K : -1.0f;
-  q.dp = 0x1p-19f * (fabsf(ef) + K);
-  return q;
-}
-template <class LX>
-__device__ __forceinline__ int quick_csd(const LX& X, const Grid& g, const Detect& D,
-                                         const double* Y) {
-  if (!D.csd_on) return kVerdictNone;
-  const QuickPrim y = quick_prim(Y[0], Y[1], Y[2], Y[3]);
-  const float r = cut_float(Y[0]);
-  bool sure = r > 0x1p-100f && r < 0x1p100f && y.p - y.dp > 0x1p-100f && y.p < 0x1p100f;
-  float div = 0.0f, ediv = 0.0f, most = 0.0f, least = 0.0f;  // bounds of the pressure gradient
-#pragma unroll
-  for (int d = 0; d < 2; ++d) {
-    if (d == 1 && g.dim != 2) break;
-    const int a = d == 0, b = d == 1;
-    const QuickPrim e = quick_prim(X(0, a, b), X(1 + d, a, b), X(2 - d, a, b), X(3, a, b));
-    const QuickPrim w = quick_prim(X(0, -a, -b), X(1 + d, -a, -b), X(2 - d, -a, -b), X(3, -a, -b));
-    const float h = d == 0 ? D.hx_f : D.hy_f;
-    div += (e.w - w.w) * h;
-    ediv += (fabsf(e.w) + fabsf(w.w)) * h;
-    const float low = fminf(e.p - e.dp, w.p - w.dp), high = fminf(e.p + e.dp, w.p + w.dp);
-    const float jump = fabsf(e.p - w.p), off = e.dp + w.dp;
-    sure = sure && low > 0x1p-100f && high < 0x1p100f;
-    most += (jump + off) * h * recip(low);
-    least += fmaxf(jump - off, 0.0f) * h * recip(high);
-  }
-  // 2^-18 of the sums of magnitudes covers the errors of the sums too
-  const float up = 1.0f + 0x1p-18f, down = 1.0f - 0x1p-18f;
-  if (!sure) return kVerdictNone;
-  if (div - 0x1p-18f * ediv >= -D.sigma_v_f * down && most * up <= D.sigma_p_f * down)
-    return kVerdictAccept;
-  if (div + 0x1p-18f * ediv < -D.sigma_v_f * up || least * down > D.sigma_p_f * up)
-    return kVerdictCsdFailed;
-  return kVerdictNone;
-}
-
 // first-pass update of cell (i,j) (if in range): candidate, detection,
 // RK combination; troubled cells go to the queue as cell_off + local index.
 // D and d2x/d2y are the detection constants and App. B weights of the grid.
@@ -1507,18 +1571,12 @@ __device__ __forceinline__ void update_cell_w(const StageArgs<Real>& A, const Gr
   if (in) {
     c = cidx(g, i, j);
     double Y[4];
-    candidate<Real>(A, g, i, j, k, Y);
+    candidate<4, Real>(A, g, i, j, 0, k, Y);
     const int top = Wd.top;
     if (top != 0) {
       int verdict = kVerdictNone;
-      bad = face_state_bad<Real>(A, g, i, j);
-      if (!bad) {
-        if constexpr (sizeof(Real) == sizeof(double))
-          verdict = quick_csd(
-              [&](int v, int a, int b) { return xload<Real>(A.Xr, g, v, i + a, j + b); }, g, D, Y);
-        if (verdict != kVerdictAccept)
-          bad = troubled<Real>(A.Xr, g, D, d2x, d2y, i, j, Y, verdict);
-      }
+      bad = face_state_bad<Real>(A, g, i, j) ||
+            troubled<Real>(A.Xr, g, D, d2x, d2y, i, j, Y, verdict);
       if (verdict != kVerdictNone) keep_verdict<Real>(A, g, i, j, verdict);
     } else {
       Real y[4] = {(Real)Y[0], (Real)Y[1], (Real)Y[2], (Real)Y[3]};
@@ -1532,8 +1590,9 @@ __device__ __forceinline__ void update_cell_w(const StageArgs<Real>& A, const Gr
   queue_push(bad, cell_off + c, A.queue, A.qcount);
 }
 
+// resident blocks an SM: the registers that leaves hold the FP64 tests
 template <class Real>
-__global__ void __launch_bounds__(256) k_update_first(StageArgs<Real> A, Grid g, Detect D,
+__global__ void __launch_bounds__(256, sizeof(Real) == sizeof(double) ? 3 : 5) k_update_first(StageArgs<Real> A, Grid g, Detect D,
                                                       const __grid_constant__ DirectW<Real> Wd) {
   pdl_wait();
   pdl_trigger();
@@ -1826,13 +1885,17 @@ __device__ __forceinline__ void stage_mood_weights(const DirectW<double>& Wd, Mo
 // entry k (0 itself, 1 W, 2 E, 3 S, 4 N) of queued cell c's neighbourhood:
 // if c is the first queued cell of that cell's own list (itself, W, E, S,
 // N), re-update it, re-detect it and return whether it is troubled; d gets
-// the cell's index (or -1)
-template <class Real>
+// the cell's index (or -1).  VL = 4: the four lanes of an aligned quad share
+// an item, one variable each (6 FP64 instructions in a row for 24); the first
+// detects and has the result.
+template <int VL, class Real>
 __device__ __forceinline__ bool mood_update_item(const StageArgs<Real>& A, const Grid& g,
-                                                 const Detect& D, const DirectW<Real>& Wd,
-                                                 const Real* d2x, const Real* d2y,
+                                                 const Detect& D, const Real* d2x,
+                                                 const Real* d2y, StageC coef,
                                                  const uint32_t* stamp, uint32_t cur, int c,
                                                  int k, int& d) {
+  const int v0 = VL == 4 ? threadIdx.x & 3 : 0;
+  constexpr int NV = 4 / VL;
   const int i = c % g.nx, j = c / g.nx;
   d = k == 0 ? c : neighbour(g, i, j, k - 1);
   if (d < 0) return false;
@@ -1856,40 +1919,50 @@ __device__ __forceinline__ bool mood_update_item(const StageArgs<Real>& A, const
   const int od = (int)load_now(A.ord + d);
   const long long k0 = gidx(g, 0, di, dj);
   const bool with_u0 = __double_as_longlong(A.ca) != 0;
-  double u0[4] = {0.0, 0.0, 0.0, 0.0};
-  if (with_u0) {
+  double u0[NV];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) u0[v] = load_now(A.U0 + k0 + v * g.vstride);
-  }
+  for (int v = 0; v < NV; ++v) u0[v] = with_u0 ? load_now(A.U0 + k0 + (v0 + v) * g.vstride) : 0.0;
   const Real r0 = load_now(A.Xr + k0), rw = load_now(A.Xr + k0 - 1), re = load_now(A.Xr + k0 + 1);
   const Real rs = load_now(A.Xr + k0 - g.pitch), rn = load_now(A.Xr + k0 + g.pitch);
-  double Y[4];
-  candidate<Real>(A, g, di, dj, A.sc->dt, Y);
-  if (taken) {
+  double y[NV];
+  candidate<NV, Real>(A, g, di, dj, v0, coef, y);
+  if (taken) {  // the same in all lanes of a quad
     d = -1;
     return false;
   }
-  bool flag = false;
-  if (od != 0) {
-    const int known = (int)(bw & kVerdictBits) >> 2;
-    int verdict = known;
-    // face_state_bad; the y faces' bits are zero in 1D
-    flag = (((bw >> 1) | be | (bs >> 1) | bn) & 1) != 0;
-    if (!flag) {
-      auto lx = [&](int v, int a, int b) -> Real {
-        if (v == 0 && a * a + b * b <= 1)
-          return a < 0 ? rw : a > 0 ? re : b < 0 ? rs : b > 0 ? rn : r0;
-        return xload<Real>(A.Xr, g, v, di + a, dj + b);
-      };
-      flag = troubled_at<Real>(lx, g, D, d2x, d2y, Y, verdict);
-    }
-    if (verdict != known) keep_verdict<Real>(A, g, di, dj, verdict);
+  double Y[4];
+  if constexpr (VL == 4) {
+    const int lane = threadIdx.x & 31, base = lane & 28;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) Y[v] = __shfl_sync(0xfu << base, y[0], base + v);
   } else {
-    Real y[4] = {(Real)Y[0], (Real)Y[1], (Real)Y[2], (Real)Y[3]};
-    Real p = (Real)(g.gamma - 1.0) * (y[3] - Real(0.5) * (y[1] * y[1] + y[2] * y[2]) / y[0]);
-    if (!(y[0] > Real(0)) || !(p > Real(0))) atomicAdd(&A.scw->nfog_pad[A.stage], 1);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) Y[v] = y[v % NV];
   }
-  combine_store<Real>(A, g, di, dj, Y, u0);
+  bool flag = false;
+  if (v0 == 0) {
+    if (od != 0) {
+      const int known = (int)(bw & kVerdictBits) >> 2;
+      int verdict = known;
+      // face_state_bad; the y faces' bits are zero in 1D
+      flag = (((bw >> 1) | be | (bs >> 1) | bn) & 1) != 0;
+      if (!flag) {
+        auto lx = [&](int v, int a, int b) -> Real {
+          if (v == 0 && a * a + b * b <= 1)
+            return a < 0 ? rw : a > 0 ? re : b < 0 ? rs : b > 0 ? rn : r0;
+          return xload<Real>(A.Xr, g, v, di + a, dj + b);
+        };
+        flag = troubled_at<Real>(lx, g, D, d2x, d2y, Y, verdict);
+      }
+      if (verdict != known) keep_verdict<Real>(A, g, di, dj, verdict);
+    } else {
+      Real f[4] = {(Real)Y[0], (Real)Y[1], (Real)Y[2], (Real)Y[3]};
+      Real p = (Real)(g.gamma - 1.0) * (f[3] - Real(0.5) * (f[1] * f[1] + f[2] * f[2]) / f[0]);
+      if (!(f[0] > Real(0)) || !(p > Real(0))) atomicAdd(&A.scw->nfog_pad[A.stage], 1);
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) combine_one<Real>(A, k0 + (v0 + v) * g.vstride, y[v], u0[v]);
   return flag;
 }
 
@@ -1909,45 +1982,43 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// barrier among `blocks` co-resident blocks: the last block to arrive resets
-// the count and opens the next generation.  A wait gives up after about a
-// second (or 2^26 polls) without a change of *alive (null: none to look at),
-// latches kErrSync and returns false; a block that sees the error leaves the
-// loop, so no wait can outlast the limit.
-__device__ __forceinline__ bool block_barrier(Scalars* sc, unsigned* bar_count,
-                                              unsigned* bar_gen, unsigned blocks,
-                                              unsigned* alive, unsigned pause) {
+// barrier among `blocks` co-resident blocks on a running count of arrivals
+// (never reset: the count at rest is a multiple of `blocks`): one atomic to
+// arrive, and everyone polls for the count that completes the round.  A wait
+// gives up after about a second (or 2^26 polls) without a change of *alive
+// (null: none to look at), latches kErrSync and returns false; a block that
+// sees the error leaves the loop, so no wait can outlast the limit.
+__device__ __forceinline__ unsigned long long load_acquire(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ bool block_barrier(Scalars* sc, unsigned long long* count,
+                                              unsigned blocks, const unsigned long long* alive,
+                                              unsigned pause) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned* gen = bar_gen;
-    volatile unsigned* life = alive;
     volatile int* err = &sc->err;
-    const unsigned g0 = *gen;
-    __threadfence();
+    unsigned long long old;
+    asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(old) : "l"(count) : "memory");
+    const unsigned long long target = (old / blocks + 1) * blocks;
     int good = 1;
-    if (atomicAdd(bar_count, 1u) == blocks - 1) {
-      atomicExch(bar_count, 0u);
-      __threadfence();
-      atomicAdd(bar_gen, 1u);
-    } else {
-      unsigned long long t0 = global_ns();
-      unsigned polls = 0, seen = life ? *life : 0;
-      while (*gen == g0) {
-        if (++polls > (1u << 26) || global_ns() - t0 > 1000000000ull) {
-          const unsigned now = life ? *life : seen;
-          if (now == seen || (*err & kErrSync)) {
-            atomicOr(&sc->err, kErrSync);
-            good = 0;
-            break;
-          }
-          seen = now;
-          t0 = global_ns();
-          polls = 0;
+    unsigned long long t0 = 0, seen = 0;
+    for (unsigned polls = 0; load_acquire(count) < target; ++polls) {
+      if (polls == 0) {
+        t0 = global_ns();
+        seen = alive ? load_acquire(alive) : 0;
+      } else if (polls > (1u << 26) || global_ns() - t0 > 1000000000ull) {
+        const unsigned long long now = alive ? load_acquire(alive) : seen;
+        if (now == seen || (*err & kErrSync)) {
+          atomicOr(&sc->err, kErrSync);
+          good = 0;
+          break;
         }
-        __nanosleep(pause);
+        polls = 0;
       }
-      __threadfence();
+      __nanosleep(pause);
     }
     if (*err & kErrSync) good = 0;
     ok = good;
@@ -1957,7 +2028,7 @@ __device__ __forceinline__ bool block_barrier(Scalars* sc, unsigned* bar_count,
 }
 // of the whole grid
 __device__ __forceinline__ bool grid_barrier(Scalars* sc) {
-  return block_barrier(sc, &sc->bar_count, &sc->bar_gen, gridDim.x, nullptr, 32);
+  return block_barrier(sc, &sc->bar_all, gridDim.x, nullptr, 20);
 }
 
 // Once a queue is short, the first kSmallBlocks blocks (on as many SMs) go on
@@ -1987,6 +2058,11 @@ struct SingleSite {
   const Detect& D;
   const Real* d2x;
   const Real* d2y;
+  StageC* k;  // shared: the stage coefficients, three FP64 products for every item
+  __device__ __forceinline__ void prepare() const {
+    if (threadIdx.x == 0) *k = stage_coeffs<Real>(A, g, A.sc->dt);
+  }
+  __device__ __forceinline__ StageC coeffs(const StageArgs<Real>&, const Grid&) const { return *k; }
   template <class F>
   __device__ __forceinline__ void with(int gc, F&& f) const {
     f(A, g, D, d2x, d2y, 0);
@@ -2194,26 +2270,27 @@ __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArg
 }
 
 // re-update + re-detect: item t is entry t % 5 (itself, W, E, S, N) of
-// pooled cell queue[t / 5]; a cell found troubled is lowered one cascade
-// level at once, marked with the next stamp and appended to the next queue
-template <class Real, class Site>
-__device__ __forceinline__ void mood_update_phase(const Site& site, const MoodArgs& M,
-                                                  const DirectW<Real>& Wd, const Cascade& C,
-                                                  uint32_t cur, const int* queue, int n,
-                                                  int* next_queue, int* next_count,
-                                                  unsigned blocks) {
+// pooled cell queue[t / 5], VL lanes each; a cell found troubled is lowered
+// one cascade level at once, marked with the next stamp and appended to the
+// next queue
+template <int VL, class Real, class Site>
+__device__ __forceinline__ void mood_update_items(const Site& site, const MoodArgs& M,
+                                                  const Cascade& C, uint32_t cur,
+                                                  const int* queue, int n, int* next_queue,
+                                                  int* next_count, unsigned blocks) {
   const long long stride = (long long)blocks * blockDim.x;
   const uint32_t* stamp = stamp_of(M, cur);
   uint32_t* next_stamp = stamp_of(M, cur + 1);
-  for (long long t = mood_lane(blocks); t < 5LL * n; t += stride) {
+  for (long long l = mood_lane(blocks); l < 5LL * VL * n; l += stride) {
+    const int t = (int)(l / VL);
     const int gc = queue[t / 5];
     int dg = -1;
     bool flag = false;
     site.with(gc, [&](const StageArgs<Real>& A, const Grid& g, const Detect& D, const Real* d2x,
                       const Real* d2y, int off) {
       int d = -1;
-      flag = mood_update_item<Real>(A, g, D, Wd, d2x, d2y, stamp + off, cur, gc - off,
-                                    (int)(t % 5), d);
+      flag = mood_update_item<VL, Real>(A, g, D, d2x, d2y, site.coeffs(A, g), stamp + off, cur,
+                                        gc - off, t % 5, d);
       if (flag) {
         // only this item updates cell d in this iteration: its radius and
         // its next stamp are written by no one else
@@ -2224,6 +2301,18 @@ __device__ __forceinline__ void mood_update_phase(const Site& site, const MoodAr
     });
     queue_push(flag, dg, next_queue, next_count);
   }
+}
+// four lanes an item where all find a thread at once, else one: the same FP64
+// work, but detection on a quarter of the lanes
+template <class Real, class Site>
+__device__ __forceinline__ void mood_update_phase(const Site& site, const MoodArgs& M,
+                                                  const Cascade& C, uint32_t cur,
+                                                  const int* queue, int n, int* next_queue,
+                                                  int* next_count, unsigned blocks) {
+  if (20LL * n <= (long long)blocks * blockDim.x)
+    mood_update_items<4, Real>(site, M, C, cur, queue, n, next_queue, next_count, blocks);
+  else
+    mood_update_items<1, Real>(site, M, C, cur, queue, n, next_queue, next_count, blocks);
 }
 
 // the loop itself, for one problem or a batch (Site); tail: every block has
@@ -2260,8 +2349,7 @@ __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs&
       return true;
     }
     return blocks == gridDim.x ? grid_barrier(sc)
-                               : block_barrier(sc, &sc->small_count, &sc->small_gen, blocks,
-                                               nullptr, 32);
+                               : block_barrier(sc, &sc->bar_small, blocks, nullptr, 20);
   };
   // n decides who goes on; false: not this block
   constexpr int kOneQueue = sizeof(Real) == sizeof(double) ? kOneQueue64 : kOneQueue32;
@@ -2280,6 +2368,7 @@ __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs&
     ok = shrink();
     if (ok) {
       // n is the same in every block; FP32 reads the kernel parameter
+      site.prepare();  // for all threads after the barrier
       if constexpr (sizeof(Real) == sizeof(double)) stage_mood_weights(Wd, MS);
       uint32_t* st = stamp_of(M, cur);
       for (long long q = mood_lane(blocks); q < n; q += (long long)blocks * blockDim.x) {
@@ -2302,7 +2391,7 @@ __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs&
     const int* queue = M.queue[slot];
     mood_faces_phase(site, M, Wd, MS, C, cur, queue, n, blocks);
     if (!barrier()) break;
-    mood_update_phase<Real>(site, M, Wd, C, cur, queue, n, M.queue[slot ^ 1], &next[slot ^ 1],
+    mood_update_phase<Real>(site, M, C, cur, queue, n, M.queue[slot ^ 1], &next[slot ^ 1],
                             blocks);
     if (!barrier()) break;
     n = *(volatile int*)&next[slot ^ 1];
@@ -2316,7 +2405,7 @@ __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs&
   // the waiting blocks look at the others' barrier, so a long loop is no
   // timeout; the error flag of a failed wait also ends this one
   if (blocks != gridDim.x && tail)
-    block_barrier(sc, &sc->bar_count, &sc->bar_gen, gridDim.x, &sc->small_gen, 256);
+    block_barrier(sc, &sc->bar_all, gridDim.x, &sc->bar_small, 256);
   if (leader) {
     sc->nbad_first[stage] = nfirst;
     sc->nbad_total[stage] = total;
@@ -2371,7 +2460,8 @@ __global__ void __launch_bounds__(256, 2) k_mood_loop(StageArgs<Real> A, MoodArg
                                                    const __grid_constant__ DirectW<Real> Wd,
                                                    Cascade C, int stage, LoopTail T) {
   pdl_wait();
-  const SingleSite<Real> site{A, g, D, Wd.d2x, Wd.d2y};
+  __shared__ StageC coef;
+  const SingleSite<Real> site{A, g, D, Wd.d2x, Wd.d2y, &coef};
   mood_loop_body<Real>(site, M, Wd, C, stage, true);
   mood_loop_tail(g, M.sc, T);
 }
@@ -2429,7 +2519,7 @@ __global__ void __launch_bounds__(256) k_update_frozen(StageArgs<Real> A, Grid g
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= g.nx || j >= g.ny) return;
   double Y[4];
-  candidate<Real>(A, g, i, j, A.sc->dt, Y);
+  candidate<4, Real>(A, g, i, j, 0, stage_coeffs<Real>(A, g, A.sc->dt), Y);
   combine_store<Real>(A, g, i, j, Y);
 }
 
@@ -2589,6 +2679,10 @@ struct BatchSite {
   const Scalars* psc;
   int nprob;
   const BatchStarts& starts;
+  __device__ __forceinline__ void prepare() const {}
+  __device__ __forceinline__ StageC coeffs(const StageArgs<Real>& A, const Grid& g) const {
+    return stage_coeffs<Real>(A, g, A.sc->dt);
+  }
   template <class F>
   __device__ __forceinline__ void with(int gc, F&& f) const {
     const int p = problem_of(probs, starts, nprob, gc);

@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(256) k_steps_1d(const __grid_constant__ Steps1
       M.stamp_stride = g.nx;
       M.count = &queued;
       M.sc = sc;
-      const SingleSite<double> site{A, g, D, Wd.d2x, Wd.d2y};
+      const SingleSite<double> site{A, g, D, Wd.d2x, Wd.d2y, &coef};
       mood_loop_body<double>(site, M, Wd, C, s, false);
       __syncthreads();
     }
