@@ -510,7 +510,7 @@ __device__ __forceinline__ void gather_face(const GatherW<Real>& Wd, int face, i
 }
 
 // pass 2: every cell of the ghosted grid collects from the faces whose
-// reconstruction stencils contain it
+// reconstruction stencils contain it (FP32; k_adj_gather_fx is FP64's)
 template <class Real>
 __global__ void __launch_bounds__(256) k_adj_gather(Grid g, const __grid_constant__ GatherW<Real> Wd,
                                                     AdjFaces Ax, AdjFaces Ay, double* G) {
@@ -553,6 +553,137 @@ __global__ void __launch_bounds__(256) k_adj_gather(Grid g, const __grid_constan
   }
 #pragma unroll
   for (int v = 0; v < 4; ++v) G[gidx(g, v, ci, cj)] = (double)acc[v];
+}
+
+// the same, FP64, in fixed point (fixed_dot.h): on the FP64 pipe its 4 x 156
+// (R = 2) products a cell take 40000 cycles a warp, 1.11 ms at 1024^2; this
+// takes about a quarter.  A block covers 32 x 8 cells of the ghosted grid; a
+// variable at a time, the state adjoints of the cells n whose faces reach them
+// are staged as integers with one exponent a cell n (the largest of its up to
+// 4 q values), each output cell sums its neighbours' products exactly and
+// rounds each sum to 2^-57 of n's scale, and the sums are added at the largest
+// scale of the neighbourhood.
+template <int R>
+struct GatherShared {
+  static constexpr int TX = 32 + 2 * R, TY = 8 + 2 * R, NV = 4 * rule_q(R);
+  long long X[NV][TY * TX];  // [face E, W, N, S][point] of cell n
+  int E[TY * TX];
+  uint32_t K[TY * TX];       // the four faces' radii, a byte each (0xff: no face)
+};
+
+// the radius-independent part of a face: its index, or -1 beyond the grid
+__device__ __forceinline__ long long gather_face_index(const Grid& g, int face, int i, int j) {
+  if (face < 2) {
+    const int f = i + (face == 0);  // E: x face i + 1, W: x face i
+    return (j >= 0 && j < g.ny && f >= 0 && f <= g.nx) ? (long long)j * (g.nx + 1) + f : -1;
+  }
+  const int f = j + (face == 2);  // N: y face j + 1, S: y face j
+  return (i >= 0 && i < g.nx && f >= 0 && f <= g.ny) ? (long long)f * g.nx + i : -1;
+}
+
+// the sum over the neighbours of one output cell (tile position lx, ly);
+// UNI: every face is at the top radius, so the weights are known constants
+template <int R, bool UNI>
+__device__ __forceinline__ double gather_sum(const GatherW<double>& W, const GatherShared<R>& S,
+                                             int lx, int ly) {
+  constexpr int Q = rule_q(R), TX = GatherShared<R>::TX;
+  int E = FXD_EMIN;
+#pragma unroll
+  for (int b = -R; b <= R; ++b)
+#pragma unroll
+    for (int a = -R; a <= R; ++a)
+      if ((a < 0 ? -a : a) + (b < 0 ? -b : b) <= R) E = max(E, S.E[(ly + R - b) * TX + lx + R - a]);
+  long long sum = 0;
+  auto neighbour = [&](int a, int b) {
+    const int t = (ly + R - b) * TX + lx + R - a, slot = diamond3_slot(a, b);
+    fxd_acc acc = {0, 0, 0};
+#pragma unroll
+    for (int face = 0; face < 4; ++face) {
+      const int K = UNI ? R : (S.K[t] >> (8 * face)) & 3;  // no face: the values are zero
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int2 z = W.z[K][face][q][slot];
+        const long long x = S.X[face * Q + q][t];
+        fxd_mac(&acc, z.x, z.y, fxd_limb_hi(x), fxd_limb_lo(x));
+      }
+    }
+    const long long m = acc.mid + (acc.ll >> FXD_SPLIT);
+    const long long r = acc.hh + ((m + (1ll << (FXD_SPLIT - 1))) >> FXD_SPLIT);
+    const int d = E - S.E[t];
+    sum += d > 62 ? 0 : r >> d;
+  };
+  if constexpr (UNI) {
+#pragma unroll
+    for (int b = -R; b <= R; ++b)
+#pragma unroll
+      for (int a = -R; a <= R; ++a)
+        if ((a < 0 ? -a : a) + (b < 0 ? -b : b) <= R) neighbour(a, b);
+  } else {
+#pragma unroll 1
+    for (int b = -R; b <= R; ++b) {
+      const int hb = R - (b < 0 ? -b : b);
+#pragma unroll 1
+      for (int a = -hb; a <= hb; ++a) neighbour(a, b);
+    }
+  }
+  return fxd_to_double(sum, E, W.off, E == 0x7ff ? 0x7ff80000u : 0u);
+}
+
+template <int R>
+__global__ void __launch_bounds__(256) k_adj_gather_fx(Grid g,
+                                                       const __grid_constant__ GatherW<double> W,
+                                                       AdjFaces Ax, AdjFaces Ay, double* G) {
+  constexpr int Q = rule_q(R), TX = GatherShared<R>::TX, TY = GatherShared<R>::TY;
+  extern __shared__ __align__(16) unsigned char gather_smem[];
+  GatherShared<R>& S = *reinterpret_cast<GatherShared<R>*>(gather_smem);
+  const int i0 = blockIdx.x * 32 - g.H, j0 = blockIdx.y * 8 - g.H;  // first output cell
+  bool top = true;
+  for (int t = threadIdx.x; t < TX * TY; t += 256) {
+    const int i = i0 - R + t % TX, j = j0 - R + t / TX;
+    uint32_t k4 = 0;
+    for (int face = 0; face < 4; ++face) {
+      const long long f = gather_face_index(g, face, i, j);
+      const uint32_t k = f < 0 ? 0xffu : (face < 2 ? Ax.K : Ay.K)[f];
+      top = top && (f < 0 || k == R);
+      k4 |= k << (8 * face);
+    }
+    S.K[t] = k4;
+  }
+  const bool uni = __syncthreads_and(top);
+  const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
+  const bool out = i0 + lx < g.nx + g.H && j0 + ly < g.ny + g.H;
+#pragma unroll 1
+  for (int v = 0; v < 4; ++v) {
+    for (int t = threadIdx.x; t < TX * TY; t += 256) {
+      const int i = i0 - R + t % TX, j = j0 - R + t / TX;
+      double x[4 * Q];
+      uint32_t most = (uint32_t)FXD_EMIN << 20;
+#pragma unroll
+      for (int face = 0; face < 4; ++face) {
+        const uint32_t K = (S.K[t] >> (8 * face)) & 0xffu;
+        const AdjFaces& F = face < 2 ? Ax : Ay;
+        const double* s = (const double*)((face & 1) ? F.R : F.L);
+        const long long f = gather_face_index(g, face, i, j);
+        const int n = K == 0xffu ? 0 : rule_q((int)K);  // the points in use
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const double u = q < n ? s[((long long)v * kMaxQ + q) * F.nf + f] : 0.0;
+          x[face * Q + q] = u;
+          most = max(most, fxd_hi(u) & 0x7fffffffu);
+        }
+      }
+      const int E = (int)(most >> 20);
+#pragma unroll
+      for (int k = 0; k < 4 * Q; ++k) S.X[k][t] = fxd_from_double(x[k], E);
+      S.E[t] = E;
+    }
+    __syncthreads();
+    if (out) {
+      const double r = uni ? gather_sum<R, true>(W, S, lx, ly) : gather_sum<R, false>(W, S, lx, ly);
+      G[gidx(g, v, i0 + lx, j0 + ly)] = r;
+    }
+    __syncthreads();
+  }
 }
 
 }  // namespace gpm

@@ -959,8 +959,8 @@ int gpmood_create(const gpmood_grid* grid, double gamma, int R_max, double ell,
   }
   fill_weights<double>(wr, R_max, d2x, d2y, h->pw64, h->dw64);
   fill_weights<float>(wr, R_max, d2x, d2y, h->pw32, h->dw32);
-  fill_gather<double>(wr, R_max, h->gw64);
-  fill_gather<float>(wr, R_max, h->gw32);
+  fill_gather(wr, R_max, h->gw64);
+  fill_gather(wr, R_max, h->gw32);
 
   // device buffers
   const size_t ncell = (size_t)g.nx * g.ny;

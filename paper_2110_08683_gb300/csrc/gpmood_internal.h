@@ -143,10 +143,19 @@ struct DirectW<double> {
   int top;
 };
 
-// the same weights as plain numbers, for the adjoint's gather
+// the same weights for the adjoint's gather: plain numbers (radius 0 is not
+// in the table)
 template <class Real>
 struct GatherW {
   Real z[4][4][kMaxQ][kMaxN];
+  int top;
+};
+// FP64: fixed-point limbs of T <= 58 bits in the slots of the radius-3
+// diamond, zero where a radius has no such point, radius 0 included
+template <>
+struct GatherW<double> {
+  int2 z[4][4][kMaxQ][kMaxN];
+  int off;  // 65 - T
   int top;
 };
 

@@ -302,9 +302,20 @@ cudaError_t LaunchA<Real>::adj_faces_stored(const void* st, const double* v, con
 template <class Real>
 cudaError_t LaunchA<Real>::adj_gather(const Grid& g, const GatherW<Real>& Wd, const AdjFaces& Ax,
                                       const AdjFaces& Ay, double* G, cudaStream_t st) {
-  const long long n = (long long)(g.nx + 2 * g.H) * (g.ny + 2 * g.H);
-  k_adj_gather<Real><<<(int)((n + 255) / 256), 256, 0, st>>>(g, Wd, Ax, Ay, G);
-  return cudaGetLastError();
+  if constexpr (sizeof(Real) == sizeof(double)) {
+    return with_radius(Wd.top, [&](auto r) {
+      constexpr int R = decltype(r)::value;
+      cudaError_t e = shared_limit(k_adj_gather_fx<R>, sizeof(GatherShared<R>));
+      if (e != cudaSuccess) return e;
+      dim3 grd((g.nx + 2 * g.H + 31) / 32, (g.ny + 2 * g.H + 7) / 8);
+      k_adj_gather_fx<R><<<grd, 256, sizeof(GatherShared<R>), st>>>(g, Wd, Ax, Ay, G);
+      return cudaGetLastError();
+    });
+  } else {
+    const long long n = (long long)(g.nx + 2 * g.H) * (g.ny + 2 * g.H);
+    k_adj_gather<Real><<<(int)((n + 255) / 256), 256, 0, st>>>(g, Wd, Ax, Ay, G);
+    return cudaGetLastError();
+  }
 }
 
 }  // namespace gpm

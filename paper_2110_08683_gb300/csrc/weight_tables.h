@@ -79,9 +79,8 @@ void plain_weights(const gpw_radius* wr, Table& D) {
         for (int m = 0; m < wr[R].n; ++m)
           D.z[R][face][k][m] = (Real)direct_weight(wr[R], face, k, wr[R].da[m], wr[R].db[m]);
 }
-void set_direct(const gpw_radius* wr, DirectW<float>& D) { plain_weights<float>(wr, D); }
-void set_direct(const gpw_radius* wr, DirectW<double>& D) {
-  double big = 0.0, l1 = 0.0;
+// the largest weight of any radius and the largest sum of |weight| of a point
+void largest_weights(const gpw_radius* wr, double& big, double& l1) {
   for (int R = 1; R <= 3; ++R)
     for (int face = 0; face < 2; ++face)
       for (int k = 0; k < wr[R].q && wr[R].n; ++k) {
@@ -92,6 +91,11 @@ void set_direct(const gpw_radius* wr, DirectW<double>& D) {
         }
         l1 = fmax(l1, s);
       }
+}
+void set_direct(const gpw_radius* wr, DirectW<float>& D) { plain_weights<float>(wr, D); }
+void set_direct(const gpw_radius* wr, DirectW<double>& D) {
+  double big = 0.0, l1 = 0.0;
+  largest_weights(wr, big, l1);
   const int T = weight_bits(big, l1);
   D.off = 63 - T;
   for (int R = 1; R <= 3; ++R)
@@ -104,11 +108,31 @@ void set_direct(const gpw_radius* wr, DirectW<double>& D) {
         }
 }
 
-template <class Real>
-void fill_gather(const gpw_radius* wr, int top, GatherW<Real>& G) {
+void fill_gather(const gpw_radius* wr, int top, GatherW<float>& G) {
   memset(&G, 0, sizeof(G));
   G.top = top;
-  plain_weights<Real>(wr, G);
+  plain_weights<float>(wr, G);
+}
+void fill_gather(const gpw_radius* wr, int top, GatherW<double>& G) {
+  memset(&G, 0, sizeof(G));
+  G.top = top;
+  double big = 0.0, l1 = 1.0;
+  largest_weights(wr, big, l1);
+  int T = 58;
+  while (T > 30 && (ldexp(big, T - 58) > 1.0 || ldexp(l1, T - 58) >= 3.9)) --T;
+  G.off = 65 - T;
+  for (int face = 0; face < 4; ++face) {
+    int2& c = G.z[0][face][0][diamond3_slot(0, 0)];
+    fxd_weight(1.0, T, &c.x, &c.y);
+  }
+  for (int R = 1; R <= 3; ++R)
+    for (int face = 0; face < 4; ++face)
+      for (int k = 0; k < wr[R].q && wr[R].n; ++k)
+        for (int m = 0; m < wr[R].n; ++m) {
+          const int a = wr[R].da[m], b = wr[R].db[m];
+          int2& z = G.z[R][face][k][diamond3_slot(a, b)];
+          fxd_weight(direct_weight(wr[R], face, k, a, b), T, &z.x, &z.y);
+        }
 }
 
 template <class Real>
