@@ -1851,35 +1851,77 @@ __device__ __forceinline__ bool mood_face_plan(const StageArgs<Real>& A, const G
   return K != Kold;  // else the EDP1 order of this face is unchanged
 }
 
-// one Gauss point of a face recomputed by the MOOD loop on the FP32 path: the
-// compiled variant of radius K
-template <class Real, int DIR>
-__device__ __forceinline__ void face_point_k(int K, const Real* X, const Grid& g,
-                                             const DirectW<Real>& Wd, int iL, int jL, int q,
-                                             Real* f, bool& bl, bool& br, Real* sUL,
-                                             Real* sUR) {
-  switch (K) {
-    case 0: face_point<0, Real, DIR>(X, g, Wd, iL, jL, q, f, bl, br, sUL, sUR); break;
-    case 1: face_point<1, Real, DIR>(X, g, Wd, iL, jL, q, f, bl, br, sUL, sUR); break;
-    case 2: face_point<2, Real, DIR>(X, g, Wd, iL, jL, q, f, bl, br, sUL, sUR); break;
-    default: face_point<3, Real, DIR>(X, g, Wd, iL, jL, q, f, bl, br, sUL, sUR); break;
-  }
-}
-
-// what the FP64 MOOD kernel keeps in shared memory: the weights of the radii
-// below the top (1 and 2 at most), which the lanes of a warp read at
-// different radii, faces and points at once, and the states of each warp's
-// points
+// what the MOOD kernel keeps in shared memory: the weights of the radii below
+// the top (1 and 2 at most), which the lanes of a warp read at different
+// radii, faces and points at once, in the slots of the radius-3 diamond (zero
+// where a radius has no such point), and the states of each warp's points
+template <class Real>
 struct MoodShared {
-  int2 z[2][4][3][kMaxN];
-  double st[8][32][8];  // [warp][point][left 0-3, right 4-7]
+  using Z = Real;
+  Z z[2][4][3][kMaxN];
+  Real st[8][32][8];  // [warp][point][left 0-3, right 4-7]
 };
-__device__ __forceinline__ void stage_mood_weights(const DirectW<double>& Wd, MoodShared& S) {
+template <>
+struct MoodShared<double> {
+  using Z = int2;
+  Z z[2][4][3][kMaxN];
+  double st[8][32][8];
+};
+__device__ __forceinline__ void stage_mood_weights(const DirectW<double>& Wd, MoodShared<double>& S) {
   for (int k = threadIdx.x; k < 2 * 4 * 3 * kMaxN; k += blockDim.x) {
     const int m = k % kMaxN, q = k / kMaxN % 3, f = k / (3 * kMaxN) % 4, K = k / (12 * kMaxN);
     S.z[K][f][q][m] = Wd.z[K + 1][f][q][m];
   }
   __syncthreads();
+}
+__device__ __forceinline__ void stage_mood_weights(const DirectW<float>& Wd, MoodShared<float>& S) {
+  for (int k = threadIdx.x; k < 2 * 4 * 3 * kMaxN; k += blockDim.x) {
+    const int m = k % kMaxN, q = k / kMaxN % 3, f = k / (3 * kMaxN) % 4, K = k / (12 * kMaxN) + 1;
+    // offset (a, b) of slot m: row starts 0, 1, 4, 9, 16, 21, 24
+    const int b = m < 1 ? -3 : m < 4 ? -2 : m < 9 ? -1 : m < 16 ? 0 : m < 21 ? 1 : m < 24 ? 2 : 3;
+    const int a = m - (b == -3 ? 0 : b == -2 ? 2 : b == -1 ? 6 : b == 0 ? 12 : b == 1 ? 18 : b == 2 ? 22 : 24);
+    const int ab = (a < 0 ? -a : a) + (b < 0 ? -b : b);
+    // the table's own order: rows b = -K..K
+    int i = a + K - (b < 0 ? -b : b);
+    for (int r = -K; r < b; ++r) i += 2 * (K - (r < 0 ? -r : r)) + 1;
+    S.z[K - 1][f][q][m] = ab <= K ? Wd.z[K][f][q][i] : 0.0f;
+  }
+  __syncthreads();
+}
+
+// one variable of a face state at radius K <= 2 given at run time, from the
+// weights in shared memory; all loads are issued before the first use.  FP32:
+// recon_direct's sum, to which the points a radius lacks add zeros.
+__device__ __forceinline__ double mood_value(const double* X, int pitch, const int2* z, int K,
+                                             int off) {
+  return fx_value<2>(X, pitch, z, K, off);
+}
+__device__ __forceinline__ float mood_value(const float* X, int pitch, const float* z, int K,
+                                            int) {
+  float x[stencil_n(2)];
+  int k = 0;
+#pragma unroll
+  for (int b = -2; b <= 2; ++b)
+#pragma unroll
+    for (int a = -2; a <= 2; ++a) {
+      const int ab = (a < 0 ? -a : a) + (b < 0 ? -b : b);
+      if (ab <= 2) x[k++] = ab <= K ? X[(long long)b * pitch + a] : 0.0f;
+    }
+  float s = 0.0f;
+  k = 0;
+#pragma unroll
+  for (int b = -2; b <= 2; ++b) {
+    const int hb = 2 - (b < 0 ? -b : b), mid = k + hb;
+    float t = mul_rn(z[diamond3_slot(0, b)], x[mid]);
+#pragma unroll
+    for (int a = 1; a <= 2; ++a)
+      if (a <= hb)
+        t = add_rn(t, add_rn(mul_rn(z[diamond3_slot(a, b)], x[mid + a]),
+                             mul_rn(z[diamond3_slot(-a, b)], x[mid - a])));
+    s = add_rn(s, t);
+    k += 2 * hb + 1;
+  }
+  return s;
 }
 
 // entry k (0 itself, 1 W, 2 E, 3 S, 4 N) of queued cell c's neighbourhood:
@@ -2108,74 +2150,22 @@ __device__ __forceinline__ void gauss_sum(const DirectW<Real>& Wd, int K, const 
   bits = (uint8_t)((((bbl >> base) & 0xFu) ? 1 : 0) | (((bbr >> base) & 0xFu) ? 2 : 0));
 }
 
-// the MOOD face recompute, FP32, with one lane per Gauss point: lane t covers
-// pooled cell queue[t / 16], face (t / 4) % 4, point t % 4.  Each lane
-// reconstructs its point's two states and solves its Riemann problem.
-// Called by whole warps (the loop runs per warp: all 32 lanes take part in
-// the shuffles).
-template <class Site>
-__device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArgs& M,
-                                                 const DirectW<float>& Wd, MoodShared&,
-                                                 const Cascade& C, uint32_t cur,
-                                                 const int* queue, int n, unsigned blocks) {
-  const long long L = 16LL * n;
-  const long long stride = (long long)blocks * blockDim.x;
-  const int lane = threadIdx.x & 31;
-  const uint32_t* stamp = stamp_of(M, cur);
-  for (long long t0 = mood_lane(blocks) - lane; t0 < L; t0 += stride) {
-    const long long t = t0 + lane;
-    const int q = (int)(t & 3);
-    const int f = (int)((t >> 2) & 3);
-    const int gc = t < L ? queue[t >> 4] : 0;
-    int iL = 0, jL = 0, K = 0;
-    bool work = false;
-    float fq[4] = {0.f, 0.f, 0.f, 0.f};
-    bool bl = false, br = false;
-    if (t < L)
-      site.with(gc, [&](const StageArgs<float>& A, const Grid& g, const Detect&, const float*,
-                        const float*, int off) {
-        work = mood_face_plan<float>(A, g, C, stamp + off, cur, gc - off, f, iL, jL, K);
-        if (work && q < rule_q(K)) {
-          // a recorded step keeps the states of the recomputed face
-          const bool keep = A.sc->ctl.stape != nullptr;
-          float UL[4], UR[4];
-          if (f < 2)
-            face_point_k<float, 0>(K, A.Xr, g, Wd, iL, jL, q, fq, bl, br, keep ? UL : nullptr, UR);
-          else
-            face_point_k<float, 1>(K, A.Xr, g, Wd, iL, jL, q, fq, bl, br, keep ? UL : nullptr, UR);
-          if (keep) {
-            const int qt = rule_q(Wd.top);
-            if (f < 2) tape_face<float, 0>(A, g, qt, iL, jL, q, UL, UR);
-            else tape_face<float, 1>(A, g, qt, iL, jL, q, UL, UR);
-          }
-        }
-      });
-    float F[4];
-    uint8_t bits;
-    gauss_sum<float>(Wd, K, fq, bl, br, F, bits);
-    if (work && q == 0)
-      site.with(gc, [&](const StageArgs<float>& A, const Grid& g, const Detect&, const float*,
-                        const float*, int) {
-        if (f < 2) store_face<float, 0>(A, g, iL, jL, F, bits);
-        else store_face<float, 1>(A, g, iL, jL, F, bits);
-      });
-  }
-}
-
-// The same, FP64.  A warp takes P consecutive points (4, 8, 16 or 32, whole
-// faces): lane l < P plans point l, then the eight values of a point (two
-// sides, four variables) are reconstructed by eight lanes, four points at a
-// time, and lane l solves point l.  A point's chain is 8 times shorter than
-// with one lane a point, and the 32 lanes of an FP64 instruction cost what
-// one does, so P is the number that makes
+// The MOOD face recompute.  Point t of 16 n is point t % 4 of face (t / 4) % 4 of
+// pooled cell queue[t / 16].  A warp takes P consecutive points (4, 8, 16 or
+// 32, whole faces): lane l < P plans point l, then the eight values of a point
+// (two sides, four variables) are reconstructed by eight lanes, four points at
+// a time and every radius and direction alike, and lane l solves point l.  A
+// point's chain is 8 times shorter than with one lane a point, and the 32
+// lanes of an instruction cost what one does, so P is the number that makes
 //   ceil(points / (P x sub-partitions)) x (a Riemann solve)
 //   + P / 4 x (a reconstruction)
 // smallest: short queues spread over the chip, long ones fill the lanes.
-template <class Site>
+template <class Real, class Site>
 __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArgs& M,
-                                                 const DirectW<double>& Wd, MoodShared& S,
+                                                 const DirectW<Real>& Wd, MoodShared<Real>& S,
                                                  const Cascade& C, uint32_t cur,
                                                  const int* queue, int n, unsigned blocks) {
+  constexpr bool F64 = sizeof(Real) == sizeof(double);
   const long long L = 16LL * n;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t* stamp = stamp_of(M, cur);
@@ -2184,16 +2174,19 @@ __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArg
   const int subs = (blocks == gridDim.x && blocks > 1 ? 2 : 4) * blocks;
   int P = 4;
   long long best = 0;
-#pragma unroll
+#pragma unroll 1
   for (int p = 4; p <= 32; p *= 2) {
-    const long long cost = (L + (long long)p * subs - 1) / ((long long)p * subs) * 28 + p / 4 * 6;
+    const long long cost =
+        (L + (long long)p * subs - 1) / ((long long)p * subs) * (F64 ? 28 : 5) + p / 4 * (F64 ? 6 : 3);
     if (p == 4 || cost < best) {
       best = cost;
       P = p;
     }
   }
+  int off = 0;
+  if constexpr (F64) off = Wd.off;
   const long long stride = (long long)blocks * (blockDim.x >> 5) * P;
-  double (*st)[8] = S.st[warp];
+  Real (*st)[8] = S.st[warp];
   for (long long t0 = ((long long)warp * blocks + blockIdx.x) * P; t0 < L; t0 += stride) {
     const long long t = t0 + lane;
     const int q = (int)(t & 3);
@@ -2202,12 +2195,12 @@ __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArg
     const int gc = mine ? queue[t >> 4] : 0;
     int iL = 0, jL = 0, K = 0, pitch = 0;
     bool work = false;
-    const double* X = nullptr;  // the left cell, variable 0
+    const Real* X = nullptr;  // the left cell, variable 0
     long long vs = 0;
     if (mine)
-      site.with(gc, [&](const StageArgs<double>& A, const Grid& g, const Detect&, const double*,
-                        const double*, int off) {
-        work = mood_face_plan<double>(A, g, C, stamp + off, cur, gc - off, f, iL, jL, K);
+      site.with(gc, [&](const StageArgs<Real>& A, const Grid& g, const Detect&, const Real*,
+                        const Real*, int first) {
+        work = mood_face_plan<Real>(A, g, C, stamp + first, cur, gc - first, f, iL, jL, K);
         pitch = g.pitch;
         vs = g.vstride;
         X = A.Xr + gidx(g, 0, iL, jL);
@@ -2215,38 +2208,39 @@ __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArg
     const bool solve = work && q < rule_q(K);
     const int dir = f < 2 ? 0 : 1;
     const int plan = solve ? 1 | K << 1 | dir << 3 | q << 4 : 0;
+#pragma unroll 1
     for (int p = 0; p < P; p += 4) {
       const int src = p + (lane >> 3), v = lane & 3, right = (lane >> 2) & 1;
       const int pl = __shfl_sync(0xffffffffu, plan, src);
-      const double* Xp = (const double*)__shfl_sync(0xffffffffu, (unsigned long long)X, src);
+      const Real* Xp = (const Real*)__shfl_sync(0xffffffffu, (unsigned long long)X, src);
       const long long vsp = __shfl_sync(0xffffffffu, vs, src);
       const int pp = __shfl_sync(0xffffffffu, pitch, src);
       if (pl) {
         const int k = (pl >> 1) & 3, d = (pl >> 3) & 1;
         Xp += v * vsp + (right ? (d ? pp : 1) : 0);
-        st[src][lane & 7] = k == 0 ? *Xp
-                                   : fx_value<2>(Xp, pp, S.z[k - 1][2 * d + right][pl >> 4], k, Wd.off);
+        st[src][lane & 7] =
+            k == 0 ? *Xp : mood_value(Xp, pp, S.z[k - 1][2 * d + right][pl >> 4], k, off);
       }
     }
     __syncwarp();
-    double fq[4] = {0.0, 0.0, 0.0, 0.0};
+    Real fq[4] = {Real(0), Real(0), Real(0), Real(0)};
     bool bl = false, br = false;
     if (solve) {
       // faces: 0 W, 1 E, 2 S, 3 N of the queued cell; the y direction swaps
       // the momenta around the x solver
       const int mn = 1 + dir, mt = 2 - dir;
-      const double* u = st[lane];
-      const double a[4] = {u[0], u[mn], u[mt], u[3]};
-      const double b[4] = {u[4], u[4 + mn], u[4 + mt], u[7]};
-      double h[4], pl, pr;
-      site.with(gc, [&](const StageArgs<double>& A, const Grid& g, const Detect&, const double*,
-                        const double*, int) {
-        riemann_x<double>(g.riemann, a, b, g.gamma, h, pl, pr);
+      const Real* u = st[lane];
+      const Real a[4] = {u[0], u[mn], u[mt], u[3]};
+      const Real b[4] = {u[4], u[4 + mn], u[4 + mt], u[7]};
+      Real h[4], pl, pr;
+      site.with(gc, [&](const StageArgs<Real>& A, const Grid& g, const Detect&, const Real*,
+                        const Real*, int) {
+        riemann_x<Real>(g.riemann, a, b, (Real)g.gamma, h, pl, pr);
         // a recorded step keeps the states of the recomputed face
         if (A.sc->ctl.stape != nullptr) {
           const int qt = rule_q(Wd.top);
-          if (dir == 0) tape_face<double, 0>(A, g, qt, iL, jL, q, u, u + 4);
-          else tape_face<double, 1>(A, g, qt, iL, jL, q, u, u + 4);
+          if (dir == 0) tape_face<Real, 0>(A, g, qt, iL, jL, q, u, u + 4);
+          else tape_face<Real, 1>(A, g, qt, iL, jL, q, u, u + 4);
         }
       });
       fq[0] = h[0];
@@ -2256,14 +2250,14 @@ __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArg
       bl = !(pos_finite(a[0]) && pos_finite(pl));
       br = !(pos_finite(b[0]) && pos_finite(pr));
     }
-    double F[4];
+    Real F[4];
     uint8_t bits;
-    gauss_sum<double>(Wd, K, fq, bl, br, F, bits);
+    gauss_sum<Real>(Wd, K, fq, bl, br, F, bits);
     if (work && q == 0)
-      site.with(gc, [&](const StageArgs<double>& A, const Grid& g, const Detect&, const double*,
-                        const double*, int) {
-        if (dir == 0) store_face<double, 0>(A, g, iL, jL, F, bits);
-        else store_face<double, 1>(A, g, iL, jL, F, bits);
+      site.with(gc, [&](const StageArgs<Real>& A, const Grid& g, const Detect&, const Real*,
+                        const Real*, int) {
+        if (dir == 0) store_face<Real, 0>(A, g, iL, jL, F, bits);
+        else store_face<Real, 1>(A, g, iL, jL, F, bits);
       });
     __syncwarp();  // the states are read before the next points' are written
   }
@@ -2363,13 +2357,12 @@ __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs&
     }
     return blockIdx.x < blocks;
   };
-  __shared__ MoodShared MS;  // FP64 only
+  __shared__ MoodShared<Real> MS;
   if (n > 0) {
     ok = shrink();
     if (ok) {
-      // n is the same in every block; FP32 reads the kernel parameter
       site.prepare();  // for all threads after the barrier
-      if constexpr (sizeof(Real) == sizeof(double)) stage_mood_weights(Wd, MS);
+      stage_mood_weights(Wd, MS);
       uint32_t* st = stamp_of(M, cur);
       for (long long q = mood_lane(blocks); q < n; q += (long long)blocks * blockDim.x) {
         const int gc = M.queue[0][q];
