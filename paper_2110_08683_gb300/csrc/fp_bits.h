@@ -8,6 +8,7 @@
 // host's own IEEE conversion.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -17,10 +18,16 @@
 #define FPB_FN static inline
 #endif
 
+// On the device by the two halves: a test of the pattern of a reinterpreted
+// double (is it zero, an infinity) the compiler turns back into an FP64 compare.
 FPB_FN uint64_t fpb_bits_of_double(double x) {
+#ifdef __CUDA_ARCH__
+  return (uint64_t)(uint32_t)__double2hiint(x) << 32 | (uint32_t)__double2loint(x);
+#else
   uint64_t b;
   memcpy(&b, &x, sizeof b);
   return b;
+#endif
 }
 
 FPB_FN float fpb_float_of_bits(uint32_t b) {
@@ -60,6 +67,57 @@ FPB_FN float fpb_double_to_float_rn(double x) {
   const uint64_t rem = M & ((1ull << s) - 1ull), half = 1ull << (s - 1);
   if (rem > half || (rem == half && (k & 1ull))) k += 1ull;
   return fpb_float_of_bits(sign | (uint32_t)k);
+}
+
+FPB_FN double fpb_double_of_bits(uint64_t b) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double((int)(b >> 32), (int)b);
+#endif
+  double x;
+  memcpy(&x, &b, sizeof x);
+  return x;
+}
+
+// the double difference of two floats, (double)a - (double)b, from the float
+// difference d and its error e (Knuth's two-sum: d + e is exact): e is counted
+// in units of the double's last place and added to d's bit pattern.  *ok: the
+// result is right; not so for infinities, NaNs and subnormals, or, with e not
+// zero, where d is a power of two (the sum may lie in the binade below) or tiny.
+FPB_FN double fpb_diff(float a, float b, int* ok) {
+  const float d = a - b, t = d - a, e = (a - (d - t)) - (b + t);
+  uint32_t bits;
+  memcpy(&bits, &d, sizeof bits);
+  const uint32_t m = bits & 0x7fffffffu;
+  *ok = e == 0.0f ? m - 1u >= 0x007fffffu
+                  : m - 0x1a800000u < 0x7f800000u - 0x1a800000u && (m & 0x007fffffu) != 0;
+  // |e| <= 2^-24 |d|, so |q| <= 2^28
+  const float u = e * fpb_float_of_bits((306u << 23) - (bits & 0x7f800000u));
+#ifdef __CUDA_ARCH__
+  const int q = e == 0.0f ? 0 : __float2int_rn(u);
+#else
+  const int q = e != 0.0f && *ok ? (int)rintf(u) : 0;
+#endif
+  const int s = -(int)(bits >> 31);
+  const uint32_t hi = (bits & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u);
+  return fpb_double_of_bits(((uint64_t)hi << 32 | (uint64_t)(bits << 29)) +
+                            (uint64_t)(int64_t)((q ^ s) - s));
+}
+
+// x c for c a power of two (fpb_is_pow2) as a step of the exponent, where operand
+// and result are normal numbers or x is zero (fpb_pow2_steps)
+FPB_FN int fpb_is_pow2(double c) {  // a normal positive power of two
+  const uint64_t b = fpb_bits_of_double(c);
+  return (b & 0x800fffffffffffffull) == 0 && b != 0 && b != 0x7ff0000000000000ull;
+}
+FPB_FN int fpb_pow2_steps(double x, double c) {
+  const uint64_t b = fpb_bits_of_double(x);
+  const int e = (int)(b >> 52) & 0x7ff, r = e + (int)(fpb_bits_of_double(c) >> 52) - 1023;
+  return (b << 1) == 0 || (e > 0 && e < 0x7ff && r > 0 && r < 0x7ff);
+}
+FPB_FN double fpb_step_exponent(double x, double c) {
+  const uint64_t b = fpb_bits_of_double(x);
+  return (b << 1) == 0 ? x
+                       : fpb_double_of_bits(b + (fpb_bits_of_double(c) - 0x3ff0000000000000ull));
 }
 
 // comparisons of doubles on integer arithmetic.  The IEEE order of doubles

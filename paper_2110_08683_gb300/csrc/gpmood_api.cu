@@ -235,8 +235,8 @@ StageArgs<Real> stage_args(gpmood_t h, int s, int rot) {
     A.Xr = h->U[ix];
     A.outr = nullptr;
   }
-  A.Fx = (double*)h->Fx;
-  A.Fy = (double*)h->Fy;
+  A.Fx = (Real*)h->Fx;
+  A.Fy = (Real*)h->Fy;
   A.fbx = h->fb;
   A.fby = h->fb + (size_t)(h->g.nx + 1) * h->g.ny;
   A.ord = h->ord + s * nc;
@@ -964,7 +964,7 @@ int gpmood_create(const gpmood_grid* grid, double gamma, int R_max, double ell,
 
   // device buffers
   const size_t ncell = (size_t)g.nx * g.ny;
-  const size_t fsz = sizeof(double);  // face fluxes are FP64 on both paths
+  const size_t fsz = h->precision == GPMOOD_FP32 ? sizeof(float) : sizeof(double);
   bool ok = true;
   for (int k = 0; k < h->sch.nbuf; ++k)
     ok = ok && cudaMalloc(&h->U[k], sizeof(double) * 4 * (size_t)g.vstride) == cudaSuccess;
@@ -1516,7 +1516,7 @@ extern "C" int gpmood_step_noalloc(const gpmood_grid* grid, double gamma, int R_
 
   // carve the buffers out of the scratch, 256-byte aligned each
   const size_t ncell = (size_t)g.nx * g.ny;
-  const size_t fsz = sizeof(double);  // face fluxes are FP64 on both paths
+  const size_t fsz = sizeof(double);  // (FP32 uses half of it)
   const size_t sz_state = align256(sizeof(double) * 4 * (size_t)g.vstride);
   const size_t sz_fx = align256(fsz * 4 * (size_t)g.ny * (g.nx + 1));
   const size_t sz_fy = align256(fsz * 4 * (size_t)(g.ny + 1) * g.nx);

@@ -232,8 +232,8 @@ StageArgs<Real> batch_args(gpmood_batch_t b, int s, int ia, int ix, int io) {
     A.Xr = b->U[ix];
     A.outr = nullptr;
   }
-  A.Fx = (double*)b->Fx;
-  A.Fy = (double*)b->Fy;
+  A.Fx = (Real*)b->Fx;
+  A.Fy = (Real*)b->Fy;
   A.fbx = b->fb;
   A.fby = b->fb + b->fx_elems / 4;
   A.ord = b->ord + (size_t)s * b->total_cells;
@@ -633,7 +633,7 @@ int gpmood_batch_create(const gpmood_grid* grids, int nprob, double gamma, int R
   b->hprobs.resize(nprob);
   long long soff = 0, fxo = 0, fyo = 0;
   int coff = 0;
-  const size_t fsz = sizeof(double);  // face fluxes are FP64 on both paths
+  const size_t fsz = b->precision == GPMOOD_FP32 ? sizeof(float) : sizeof(double);
   std::vector<Item> fx4, fx8, fy4, fy8, up, dtl, xy;
   long long max_ghost = 0;
   const bool fp64 = b->precision != GPMOOD_FP32;

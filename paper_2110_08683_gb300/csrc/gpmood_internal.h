@@ -211,8 +211,8 @@ struct StageArgs {
   const double* U0;  // ghosted U^n (combination)
   double* out;       // ghosted stage output
   Real* outr;        // float shadow of out (FP32), null (FP64)
-  double* Fx;        // face-averaged fluxes, FP64 on both paths: each float flux is
-  double* Fy;        // widened once, by the face kernel, not once per neighbour
+  Real* Fx;          // face-averaged fluxes as the Riemann solver made them; their
+  Real* Fy;          // differences are formed exactly (FP32: flux_diffs)
   uint8_t* fbx;      // per x face: bit 0 its left, bit 1 its right state failed the
   uint8_t* fby;      // face-state check (per y face: lower, upper), at the face's radius;
                      // bits 2-3 of an x face: what detection knows of the cell to its

@@ -1485,46 +1485,6 @@ __device__ __forceinline__ StageC stage_coeffs(const StageArgs<Real>& A, const G
   return StageC{hdt * g.inv_dx, hdt * g.inv_dy};
 }
 
-// per variable two differences and two fmas: NV variables from v0 on
-template <int NV, class Real>
-__device__ __forceinline__ void candidate(const StageArgs<Real>& A, const Grid& g, int i, int j,
-                                          int v0, StageC k, double* Y) {
-#pragma unroll
-  for (int n = 0; n < NV; ++n) {
-    const int v = v0 + n;
-    double fe = A.Fx[fxidx(g, v, i + 1, j)], fw = A.Fx[fxidx(g, v, i, j)];
-    double gn = A.Fy[fyidx(g, v, i, j + 1)], gs = A.Fy[fyidx(g, v, i, j)];
-    Y[n] = fma(-k.cx, fe - fw, fma(-k.cy, gn - gs, A.X[gidx(g, v, i, j)]));
-  }
-}
-
-// the SSP-RK combination of the candidate
-// one value of it, at index k: Y the candidate, u0 U^n (read where ca is not
-// zero)
-template <class Real>
-__device__ __forceinline__ void combine_one(const StageArgs<Real>& A, long long k, double Y,
-                                            double u0) {
-  // the first stage's combination is the candidate itself (ca = 0, cb = 1);
-  // compared as integers, an FP64 compare costs what a product does
-  const double o = __double_as_longlong(A.ca) != 0 ? fma(A.ca, u0, A.cb * Y)
-                   : __double_as_longlong(A.cb) == 0x3ff0000000000000ll ? Y
-                                                                        : A.cb * Y;
-  A.out[k] = o;
-  if constexpr (sizeof(Real) == sizeof(float)) A.outr[k] = fpb_double_to_float_rn(o);
-  if (A.out2) A.out2[k] = fma(A.wa, A.W[k], A.wb * Y);
-}
-template <class Real>
-__device__ __forceinline__ void combine_store(const StageArgs<Real>& A, const Grid& g, int i,
-                                              int j, const double* Y) {
-  double u0[4] = {0.0, 0.0, 0.0, 0.0};
-  if (__double_as_longlong(A.ca) != 0) {
-#pragma unroll
-    for (int v = 0; v < 4; ++v) u0[v] = A.U0[gidx(g, v, i, j)];
-  }
-#pragma unroll
-  for (int v = 0; v < 4; ++v) combine_one<Real>(A, gidx(g, v, i, j), Y[v], u0[v]);
-}
-
 // a load issued where it stands: the MOOD loop's few cells an iteration leave
 // every memory latency exposed, and the compiler would move a load that only
 // a branch uses into it, behind the loads that decide the branch
@@ -1542,6 +1502,119 @@ __device__ __forceinline__ unsigned load_now(const uint8_t* p) {
   unsigned v;
   asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+
+// 0 or 1 for the trip count of a loop that stands for an if.  FP64 code under an
+// if of a few instructions is compiled with predicates, and an FP64 instruction
+// no lane takes part in holds the pipe as long as any: the first-pass update
+// issued 33 of them a warp in every stage, where the first stage needs 8.
+__device__ __forceinline__ int branch(bool cond) {
+  int n = cond;
+  asm volatile("" : "+r"(n));
+  return n;
+}
+// and x, tied to the loop: what is invariant in it would be formed ahead of it
+__device__ __forceinline__ double in_loop(double x) {
+  asm volatile("" : "+d"(x));
+  return x;
+}
+
+// the flux differences fe - fw and gn - gs of NV variables from v0 on, as
+// doubles; FP32: on the float and integer pipes (fpb_diff), but for the odd
+// cell that is not for it
+template <int NV, class Real>
+__device__ __forceinline__ void flux_diffs(const StageArgs<Real>& A, const Grid& g, int i, int j,
+                                           int v0, double* dx, double* dy) {
+  const Real* fx = A.Fx + fxidx(g, v0, i, j);
+  const Real* fy = A.Fy + fyidx(g, v0, i, j);
+  const long long px = fxidx(g, 1, 0, 0), py = fyidx(g, 1, 0, 0), up = fyidx(g, 0, 0, 1);
+  if constexpr (sizeof(Real) == sizeof(float)) {
+    bool all = true;
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      int ox, oy;
+      dx[n] = fpb_diff(fx[n * px + 1], fx[n * px], &ox);
+      dy[n] = fpb_diff(fy[n * py + up], fy[n * py], &oy);
+      all = all && ox && oy;
+    }
+#pragma unroll 1
+    for (int t = branch(!all); t > 0; --t)
+#pragma unroll
+      for (int n = 0; n < NV; ++n) {
+        dx[n] = (double)load_now(fx + n * px + 1) - (double)load_now(fx + n * px);
+        dy[n] = (double)load_now(fy + n * py + up) - (double)load_now(fy + n * py);
+      }
+  } else {
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      dx[n] = fx[n * px + 1] - fx[n * px];
+      dy[n] = fy[n * py + up] - fy[n * py];
+    }
+  }
+}
+
+// the candidate, NV variables from v0 on
+template <int NV, class Real>
+__device__ __forceinline__ void candidate(const StageArgs<Real>& A, const Grid& g, int i, int j,
+                                          int v0, StageC k, double* Y) {
+  double dx[NV], dy[NV];
+  flux_diffs<NV, Real>(A, g, i, j, v0, dx, dy);
+#pragma unroll
+  for (int n = 0; n < NV; ++n)
+    Y[n] = fma(-k.cx, dx[n], fma(-k.cy, dy[n], A.X[gidx(g, v0 + n, i, j)]));
+}
+
+// the SSP-RK combination of the candidates Y of NV variables, stored at k0 and
+// vstride apart: ca u0 + cb Y, with u0 U^n (read where ca is not zero).  The
+// first stage's combination is the candidate itself (ca = 0, cb = 1); a cb that
+// is a power of two (the second stage's 1/4) only steps exponents.
+template <int NV, class Real>
+__device__ __forceinline__ void combine(const StageArgs<Real>& A, long long k0, long long vstride,
+                                        const double* Y, const double* u0) {
+  // compared as integers: an FP64 compare costs what a product does
+  const bool with_u0 = __double_as_longlong(A.ca) != 0;
+  double o[NV];
+#pragma unroll
+  for (int n = 0; n < NV; ++n) o[n] = Y[n];
+#pragma unroll 1
+  for (int t = branch(__double_as_longlong(A.cb) != 0x3ff0000000000000ll); t > 0; --t) {
+    const bool pow2 = fpb_is_pow2(A.cb);
+    bool product = !pow2;
+#pragma unroll
+    for (int n = 0; n < NV; ++n) {
+      product = product || !fpb_pow2_steps(o[n], A.cb);
+      if (pow2) o[n] = fpb_step_exponent(o[n], A.cb);
+    }
+#pragma unroll 1
+    for (int u = branch(product); u > 0; --u)
+#pragma unroll
+      for (int n = 0; n < NV; ++n) o[n] = A.cb * in_loop(Y[n]);
+  }
+#pragma unroll 1
+  for (int t = branch(with_u0); t > 0; --t)
+#pragma unroll
+    for (int n = 0; n < NV; ++n) o[n] = fma(A.ca, in_loop(u0[n]), o[n]);
+#pragma unroll
+  for (int n = 0; n < NV; ++n) {
+    A.out[k0 + n * vstride] = o[n];
+    if constexpr (sizeof(Real) == sizeof(float))
+      A.outr[k0 + n * vstride] = fpb_double_to_float_rn(o[n]);
+  }
+#pragma unroll 1
+  for (int t = branch(A.out2 != nullptr); t > 0; --t)
+#pragma unroll
+    for (int n = 0; n < NV; ++n)
+      A.out2[k0 + n * vstride] = fma(A.wa, A.W[k0 + n * vstride], A.wb * in_loop(Y[n]));
+}
+template <class Real>
+__device__ __forceinline__ void combine_store(const StageArgs<Real>& A, const Grid& g, int i,
+                                              int j, const double* Y) {
+  double u0[4] = {0.0, 0.0, 0.0, 0.0};
+  if (__double_as_longlong(A.ca) != 0) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) u0[v] = A.U0[gidx(g, v, i, j)];
+  }
+  combine<4, Real>(A, gidx(g, 0, i, j), g.vstride, Y, u0);
 }
 
 // append to a queue with one atomic per warp
@@ -1590,9 +1663,13 @@ __device__ __forceinline__ void update_cell_w(const StageArgs<Real>& A, const Gr
   queue_push(bad, cell_off + c, A.queue, A.qcount);
 }
 
-// resident blocks an SM: the registers that leaves hold the FP64 tests
+// FP32 at 4096 x 1024: 0.18 ms a launch, bound by issue (60%) and latency; 0.26
+// when it was bound by the FP64 pipe, 33 instructions a warp, of which it needs
+// 8 to 16 (see flux_diffs, combine, branch; fp_bits.h on folded compares).  FP64:
+// 0.22 ms.  Resident blocks an SM: of 3 to 6 the fastest at this size that is
+// not slower on small grids.
 template <class Real>
-__global__ void __launch_bounds__(256, sizeof(Real) == sizeof(double) ? 3 : 5) k_update_first(StageArgs<Real> A, Grid g, Detect D,
+__global__ void __launch_bounds__(256, sizeof(Real) == sizeof(double) ? 4 : 5) k_update_first(StageArgs<Real> A, Grid g, Detect D,
                                                       const __grid_constant__ DirectW<Real> Wd) {
   pdl_wait();
   pdl_trigger();
@@ -2003,8 +2080,7 @@ __device__ __forceinline__ bool mood_update_item(const StageArgs<Real>& A, const
       if (!(f[0] > Real(0)) || !(p > Real(0))) atomicAdd(&A.scw->nfog_pad[A.stage], 1);
     }
   }
-#pragma unroll
-  for (int v = 0; v < NV; ++v) combine_one<Real>(A, k0 + (v0 + v) * g.vstride, y[v], u0[v]);
+  combine<NV, Real>(A, k0 + v0 * g.vstride, g.vstride, y, u0);
   return flag;
 }
 
