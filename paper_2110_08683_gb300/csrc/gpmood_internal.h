@@ -247,7 +247,7 @@ struct MoodArgs {
 
 // a one-dimensional handle as the one-block step kernel sees it: its buffers,
 // the RK scheme, the buffer rotation and the steps to take
-constexpr int kMaxCells1D = 1024;
+constexpr int kMaxCells1D = 512;
 struct Steps1D {
   double* U[5];
   double *Fx, *Fy;
