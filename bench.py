@@ -99,8 +99,21 @@ def faces_flops_per_face(R=3, fused=False):
     return (256 * sums + (224 + 256) * dots) / (2 * 7 * 31) + riemann
 
 
-FACE_KERNEL_SOURCES = ("gpmood_kernels.cuh", "gpmood_internal.h", "kernels_impl.cuh",
-                       "fp_bits.h")
+# FP64 instructions of one HLLC flux in the FP64 face kernel (reciprocals, square
+# roots and comparisons are integer work there)
+HLLC_FP64_INSTRUCTIONS = 41
+
+
+def fp64_instructions_per_face(R=3):
+    """FP64 instructions of the FP64 face kernel per face: q HLLC fluxes and the
+    Gauss sum (an add and an FMA a mirror pair and variable).  The
+    reconstruction is exact fixed-point arithmetic on the integer pipes."""
+    q = R + 1
+    return q * HLLC_FP64_INSTRUCTIONS + 4 * (2 * (q // 2) + q % 2)
+
+
+FACE_KERNEL_SOURCES = ("faces_fp64.cuh", "fixed_dot.h", "fp_newton.h", "gpmood_kernels.cuh",
+                       "gpmood_internal.h", "kernels_impl.cuh", "fp_bits.h")
 
 
 def kernel_source_hash():
@@ -476,26 +489,36 @@ def measure(kind, nx, ny, precision, scheme, steps, warmup, world, local, eager=
         faces = (nx + 1) * ny + (nx * (ny + 1) if fused else 0)
         peak = FP64_PEAK_TFLOPS if real64 else FP32_PEAK_TFLOPS
         alg = faces * algorithmic_flops_per_face(R)
-        exe = faces * faces_flops_per_face(R, fused)
+        if real64:
+            n = fp64_instructions_per_face(R)
+            # lane-instructions a second against the pipe's rate (2 flop each)
+            executed = {"fp64_instructions_per_face": n,
+                        "frac": round(2 * faces * n / per_launch_s / 1e12 / peak, 4),
+                        "count": "FP64 instructions of the Riemann solver and the Gauss sum; "
+                                 "the reconstruction runs in fixed point on the integer pipes"}
+        else:
+            exe = faces * faces_flops_per_face(R, fused)
+            executed = {"flops_per_face": round(faces_flops_per_face(R, fused), 1),
+                        "flops_per_launch": exe,
+                        "achieved": round(exe / per_launch_s / 1e12, 4),
+                        "frac": round(exe / per_launch_s / 1e12 / peak, 4),
+                        "count": "the kernel's own arithmetic after the parity-sum "
+                                 "reconstruction (mirror-orbit sums, q/2 dot products, "
+                                 "butterflies)"}
         roofline = {
             "bound": "alu", "achieved": round(alg / per_launch_s / 1e12, 4),
             "peak": round(peak, 4), "unit": "TFLOP/s",
             "frac": round(alg / per_launch_s / 1e12 / peak, 4),
             "traffic": ncu_traffic(precision, kind, scheme),
-            "kernel": ("k_faces_xy<R=%d,%s> (x and y faces)" if fused else "k_faces<R=%d,%s,x>")
-                      % (R, "double" if real64 else "float"),
+            "kernel": ("k_faces_fx<R=%d>" % R if real64 else
+                       ("k_faces_xy<R=%d,float>" if fused else "k_faces<R=%d,float,x>") % R)
+                      + (" (x and y faces)" if fused else ""),
             "flops_per_launch": alg,
             "flops_per_face": algorithmic_flops_per_face(R),
             "count": "algorithmic: 8 q N reconstruction FMA (2 flop), q HLLC at %d flop, the "
                      "Gauss sum; per face, x %s faces a launch"
                      % (HLLC_FLOPS, "(nx+1) ny + nx (ny+1)" if fused else "(nx+1) ny"),
-            "executed": {"flops_per_face": round(faces_flops_per_face(R, fused), 1),
-                         "flops_per_launch": exe,
-                         "achieved": round(exe / per_launch_s / 1e12, 4),
-                         "frac": round(exe / per_launch_s / 1e12 / peak, 4),
-                         "count": "the kernel's own arithmetic after the parity-sum "
-                                  "reconstruction (mirror-orbit sums, q/2 dot products, "
-                                  "butterflies)"},
+            "executed": executed,
             "launch_ms": round(per_launch_s * 1e3, 4),
             "timing": "event nodes around every x-face launch in the step graph, second timed "
                       "pass of the same steps (L2 flushed between steps)",

@@ -1,11 +1,10 @@
-// fp_bits.h -- IEEE-754 operations computed on bit patterns with integer
-// arithmetic.  On GB300 a conversion between double and float occupies the
-// FP64 pipe as long as an FMA does (about 64 cycles per warp instruction per
-// sub-partition), while the integer pipes are otherwise idle in the FP64-bound
-// kernels; these functions give the same result as the hardware instruction
-// (bit for bit, save for which NaN a NaN becomes).
-// Plain C as well as CUDA, so that a host unit test checks them against the
-// host's own IEEE conversion.
+// fp_bits.h -- IEEE-754 operations on doubles computed with integer (and float)
+// arithmetic.  On GB300 a double operation, a comparison and a conversion each
+// hold the FP64 pipe for about 64 cycles per warp instruction per sub-partition,
+// while the integer pipes are otherwise idle in the FP64-bound kernels; these
+// functions give the same result as the hardware instruction (bit for bit, save
+// for which NaN a NaN becomes).  Plain C as well as CUDA, so that host unit
+// tests check them against the host's own IEEE arithmetic.
 #pragma once
 
 #include <math.h>

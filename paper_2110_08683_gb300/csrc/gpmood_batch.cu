@@ -1,8 +1,8 @@
 // gpmood_batch.cu -- many independent GP-MOOD problems of uneven sizes
 // advanced together (include/gpmood.h, gpmood_batch_*): pooled buffers, one
-// persistent launch per kernel class walking (problem, block) work items,
-// one captured graph per step with the MOOD loops as conditional WHILE
-// nodes, per-problem time steps, and a small autotuner for the face kernels.
+// launch per kernel class over (problem, block) work items, the MOOD loops of
+// a stage in one cooperative launch, one captured graph per step, per-problem
+// time steps, and a small autotuner for the FP32 face kernels and the update.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdlib.h>

@@ -1,19 +1,21 @@
 // gpmood_kernels.cuh -- CUDA kernels of the GP-MOOD stage (sm_103a).
 //
 // One RK stage (Sec. 4, Steps 3-10) of a single problem runs as
-//   fill_ghosts -> x_faces -> y_faces -> update_first    (first pass, all cells)
+//   fill_ghosts -> faces -> update_first                  (first pass, all cells)
 //   mood_loop                                             (troubled cells only)
-// x_faces / y_faces reconstruct the pointwise Riemann states of eq.
-// gp_reconstructor at the Gauss points of Table QR, apply face-state CAD
-// (Sec. 3.3.1), solve HLLC and store the face-averaged flux of eq. fvm_F.
+// faces (FP64: faces_fp64.cuh; FP32: k_faces_xy, or k_faces a direction)
+// reconstruct the pointwise Riemann states of eq. gp_reconstructor at the Gauss
+// points of Table QR, apply face-state CAD (Sec. 3.3.1), solve HLLC and store
+// the face-averaged flux of eq. fvm_F.
 // update_first forms the candidate of eq. fvm_discrete, runs Steps 4-9,
 // writes the SSP-RK3 combination (eq. rk3) and appends troubled cells to a
 // queue with one atomic per warp.  mood_loop iterates on the device, with
-// grid-wide barriers between its phases: it lowers the order of queued cells
+// barriers between its phases among as many blocks as the queue is worth: it
+// lowers the order of queued cells
 // by one cascade level, recomputes the faces whose EDP1 order changed (Sec.
 // 3.6) and re-updates + re-detects the queued cells and their face
-// neighbours, until no cell is troubled.  Batches run the same phases as one
-// kernel per phase, the loop a conditional WHILE node of the step graph.
+// neighbours, until no cell is troubled.  Batches run the same kernels over the
+// work items and the pooled queue of many problems.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -989,8 +991,10 @@ __global__ void __launch_bounds__(32 * FW) k_faces(StageArgs<Real> A, Grid g,
 }
 
 // ---------------------------------------------------------------------------
-// both first-pass face sweeps in one block (two-dimensional grids).  A block
-// of 8 warps covers 8 rows of a 32-cell segment: lane l, warp w hold cell
+// both first-pass face sweeps in one block (two-dimensional grids, FP32).
+// Bound by issue (76%; FMA and ALU pipes 38% each): 0.35 ms a launch at
+// 4096 x 1024, R = 3, 2200 instructions a warp, half of them in the eight
+// Riemann solves.  A block of 8 warps covers 8 rows of a 32-cell segment: lane l, warp w hold cell
 // (i0 + l, j0 + w), i0 = 31 seg - 1, j0 = 7 band - 1, so segments overlap by
 // one column and bands by one row.  Each cell forms its parity sums once per
 // variable and from them both its x states (E/W, kept in registers for the
