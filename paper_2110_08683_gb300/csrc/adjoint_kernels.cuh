@@ -560,13 +560,13 @@ __global__ void __launch_bounds__(256) k_adj_gather(Grid g, const __grid_constan
 // takes about a quarter.  A block covers 32 x 8 cells of the ghosted grid; a
 // variable at a time, the state adjoints of the cells n whose faces reach them
 // are staged as integers with one exponent a cell n (the largest of its up to
-// 4 q values), each output cell sums its neighbours' products exactly and
-// rounds each sum to 2^-57 of n's scale, and the sums are added at the largest
-// scale of the neighbourhood.
+// 4 q values), each output cell sums its neighbours' products exactly, and the
+// sums are added at the largest scale of the neighbourhood, cut at 2^-86 of it.
+// 1024^2, R = 2: 0.55 ms a launch, bound by issue.
 template <int R>
 struct GatherShared {
   static constexpr int TX = 32 + 2 * R, TY = 8 + 2 * R, NV = 4 * rule_q(R);
-  long long X[NV][TY * TX];  // [face E, W, N, S][point] of cell n
+  int2 X[NV][TY * TX];       // limbs (high, low), [face E, W, N, S][point] of cell n
   int E[TY * TX];
   uint32_t K[TY * TX];       // the four faces' radii, a byte each (0xff: no face)
 };
@@ -593,7 +593,10 @@ __device__ __forceinline__ double gather_sum(const GatherW<double>& W, const Gat
 #pragma unroll
     for (int a = -R; a <= R; ++a)
       if ((a < 0 ? -a : a) + (b < 0 ? -b : b) <= R) E = max(E, S.E[(ly + R - b) * TX + lx + R - a]);
-  long long sum = 0;
+  // the sum as hi 2^29 + lo, in units of 2^-86 of the largest scale: a cell at the
+  // rim of what a localised cotangent reaches has a small weight's product alone
+  constexpr long long kLow = (1ll << FXD_SPLIT) - 1;
+  long long hi = 0, lo = 0;
   auto neighbour = [&](int a, int b) {
     const int t = (ly + R - b) * TX + lx + R - a, slot = diamond3_slot(a, b);
     fxd_acc acc = {0, 0, 0};
@@ -603,14 +606,16 @@ __device__ __forceinline__ double gather_sum(const GatherW<double>& W, const Gat
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
         const int2 z = W.z[K][face][q][slot];
-        const long long x = S.X[face * Q + q][t];
-        fxd_mac(&acc, z.x, z.y, fxd_limb_hi(x), fxd_limb_lo(x));
+        const int2 x = S.X[face * Q + q][t];
+        fxd_mac(&acc, z.x, z.y, x.x, x.y);
       }
     }
     const long long m = acc.mid + (acc.ll >> FXD_SPLIT);
-    const long long r = acc.hh + ((m + (1ll << (FXD_SPLIT - 1))) >> FXD_SPLIT);
-    const int d = E - S.E[t];
-    sum += d > 62 ? 0 : r >> d;
+    const long long h = acc.hh + (m >> FXD_SPLIT), l = m & kLow;
+    const int d = E - S.E[t];  // down by d
+    hi += h >> min(d, 63);
+    lo += (d <= 35 ? (long long)(((unsigned long long)h << FXD_SPLIT | l) >> d)
+                   : h >> min(d - FXD_SPLIT, 63)) & kLow;
   };
   if constexpr (UNI) {
 #pragma unroll
@@ -626,7 +631,13 @@ __device__ __forceinline__ double gather_sum(const GatherW<double>& W, const Gat
       for (int a = -hb; a <= hb; ++a) neighbour(a, b);
     }
   }
-  return fxd_to_double(sum, E, W.off, E == 0x7ff ? 0x7ff80000u : 0u);
+  hi += lo >> FXD_SPLIT;
+  lo &= kLow;
+  // as many of the low bits as there is room for (|hi| < 2^62)
+  const int z = __clzll(hi ^ (hi >> 63)) - 2;
+  const int k = E > 128 ? max(min(z, FXD_SPLIT), 0) : 0;
+  return fxd_to_double((long long)((unsigned long long)hi << k) + (lo >> (FXD_SPLIT - k)), E,
+                       W.off - k, E == 0x7ff ? 0x7ff80000u : 0u);
 }
 
 template <int R>
@@ -674,7 +685,10 @@ __global__ void __launch_bounds__(256) k_adj_gather_fx(Grid g,
       }
       const int E = (int)(most >> 20);
 #pragma unroll
-      for (int k = 0; k < 4 * Q; ++k) S.X[k][t] = fxd_from_double(x[k], E);
+      for (int k = 0; k < 4 * Q; ++k) {
+        const long long m = fxd_from_double(x[k], E);
+        S.X[k][t] = make_int2(fxd_limb_hi(m), fxd_limb_lo(m));
+      }
       S.E[t] = E;
     }
     __syncthreads();
