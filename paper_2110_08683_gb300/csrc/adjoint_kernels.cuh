@@ -556,9 +556,9 @@ __global__ void __launch_bounds__(256) k_adj_gather(Grid g, const __grid_constan
 }
 
 // the same, FP64, in fixed point (fixed_dot.h): on the FP64 pipe its 4 x 156
-// (R = 2) products a cell take 40000 cycles a warp, 1.11 ms at 1024^2.  A block covers 32 x 8 cells of the ghosted grid; a
-// variable at a time, the state adjoints of the cells n whose faces reach them
-// are staged as integers with one exponent a cell n (the largest of its up to
+// (R = 2) products a cell take 40000 cycles a warp, 1.11 ms at 1024^2.  A block
+// covers 32 x 8 cells of the ghosted grid; a variable at a time, the state
+// adjoints of the cells n whose faces reach them are staged as integers with one exponent a cell n (the largest of its up to
 // 4 q values), each output cell sums its neighbours' products exactly, and the
 // sums are added at the largest scale of the neighbourhood, cut at 2^-86 of it.
 // 1024^2, R = 2: 0.63 ms a launch, bound by issue.
