@@ -175,6 +175,7 @@ struct Detect {
   // no kernel converts or combines them once per cell
   double gm1, hx, hy;   // gamma - 1, 1 / (2 dx), 1 / (2 dy)
   float sigma_v_f, sigma_p_f, plateau_thr_f, delta_f, gm1_f, hx_f, hy_f;
+  int quick;            // FP64: the tests may be tried in float first (quick_csd, quick_u2)
 };
 
 // the derived members of D, once its own members and the grid are set
@@ -189,6 +190,10 @@ inline void detect_derive(Detect& D, const Grid& g) {
   D.gm1_f = (float)(g.gamma - 1.0);
   D.hx_f = 0.5f * (float)g.inv_dx;
   D.hy_f = 0.5f * (float)g.inv_dy;
+  // the float tests' error bounds hold for constants well inside the float range
+  const double range[5] = {D.sigma_v, D.sigma_p, D.delta, D.hx, g.dim == 2 ? D.hy : D.hx};
+  D.quick = 1;
+  for (int k = 0; k < 5; ++k) D.quick = D.quick && range[k] > 0x1p-60 && range[k] < 0x1p60;
 }
 
 // one RK stage as buffer roles (slots relative to the step's rotation of

@@ -1227,15 +1227,21 @@ __device__ __forceinline__ void keep_verdict(const StageArgs<Real>& A, const Gri
 // Detection in float, FP64 path, where the float values decide a test whatever
 // the rounding.  quick_csd: kVerdictAccept (CAD, PAD and CSD pass),
 // kVerdictCsdFailed (CAD and PAD pass, CSD fails) or kVerdictNone (too close
-// to a threshold, or CAD or PAD may fail).  Few cells are close, and an FP64
-// operation costs 64 times a float one: 0.26 ms a launch at 4096 x 1024 (the
-// candidate and the RK sums) for 0.78 with the tests in FP64.
+// to a threshold, or CAD or PAD may fail, or out of float's range).  Few cells
+// are close, and an FP64 operation costs 64 times a float one: 0.26 ms a launch
+// at 4096 x 1024 (the candidate and the RK sums) for 0.78 with the tests in FP64.
 // The double -> float cut is below 2^-23 relative and so is every float
-// operation; |u|, K = |m|^2 / (2 rho) and E carry at most 8 such errors, so
-// 2^-19 of their magnitudes bounds each.  A NaN or an infinity fails every
-// comparison.
+// operation on normal numbers; |u|, K = |m|^2 / (2 rho) and E carry at most 8
+// such errors, so 2^-19 of their magnitudes bounds each.  Floats lose relative
+// accuracy below 2^-126: a momentum cut to zero there moves u by 2^-126 / rho
+// (du) and K by nothing, and a square that underflows is off by 2^-149, K by
+// 2^-149 / rho, which stays below 2^-28 of E where rho E > 2^-120; elsewhere
+// the pressure is not known.  (Detect::quick: the thresholds and mesh widths
+// lie within 2^+-60, so that no sum or bound below under- or overflows.)  A NaN
+// or an infinity fails every comparison.
 struct QuickPrim {
-  float w, p, dp;  // normal velocity, pressure / (gamma - 1) and its error bound
+  float w, dw;  // normal velocity and its error bound over 2^-18
+  float p, dp;  // pressure / (gamma - 1) and its error bound
 };
 __device__ __forceinline__ float cut_float(double x) {
   // the leading 24 bits; below the float range zero, beyond it an infinity
@@ -1251,20 +1257,20 @@ __device__ __forceinline__ QuickPrim quick_prim(double r, double mn, double mt, 
   const float K = 0.5f * (nf * nf + tf * tf) * ir;
   QuickPrim q;
   q.w = nf * ir;
-  q.p = rf > 0x1p-100f ? ef - K : -1.0f;
+  q.dw = fmaf(0x1p-106f, ir, fabsf(q.w));
+  q.p = rf > 0x1p-100f && rf < 0x1p100f && rf * ef > 0x1p-120f ? ef - K : -1.0f;
   q.dp = 0x1p-19f * (fabsf(ef) + K);
   return q;
 }
 // CAD and PAD pass
 __device__ __forceinline__ bool quick_pad(const double* Y) {
   const QuickPrim y = quick_prim(Y[0], Y[1], Y[2], Y[3]);
-  const float r = cut_float(Y[0]);
-  return r > 0x1p-100f && r < 0x1p100f && y.p - y.dp > 0x1p-100f && y.p < 0x1p100f;
+  return y.p - y.dp > 0x1p-100f && y.p < 0x1p100f;
 }
 template <class LX>
 __device__ __forceinline__ int quick_csd(const LX& X, const Grid& g, const Detect& D,
                                          const double* Y) {
-  if (!D.csd_on) return kVerdictNone;
+  if (!D.csd_on || !D.quick) return kVerdictNone;
   bool sure = quick_pad(Y);
   float div = 0.0f, ediv = 0.0f, most = 0.0f, least = 0.0f;  // bounds of the pressure gradient
 #pragma unroll
@@ -1275,12 +1281,12 @@ __device__ __forceinline__ int quick_csd(const LX& X, const Grid& g, const Detec
     const QuickPrim w = quick_prim(X(0, -a, -b), X(1 + d, -a, -b), X(2 - d, -a, -b), X(3, -a, -b));
     const float h = d == 0 ? D.hx_f : D.hy_f;
     div += (e.w - w.w) * h;
-    ediv += (fabsf(e.w) + fabsf(w.w)) * h;
+    ediv += (e.dw + w.dw) * h;
     const float low = fminf(e.p - e.dp, w.p - w.dp), high = fminf(e.p + e.dp, w.p + w.dp);
     const float jump = fabsf(e.p - w.p), off = e.dp + w.dp;
     sure = sure && low > 0x1p-100f && high < 0x1p100f;
-    most += (jump + off) * h * recip(low);
-    least += fmaxf(jump - off, 0.0f) * h * recip(high);
+    most += (jump + off) * recip(low) * h;
+    least += fmaxf(jump - off, 0.0f) * recip(high) * h;
   }
   // 2^-18 of the sums of magnitudes covers the errors of the sums too
   const float up = 1.0f + 0x1p-18f, down = 1.0f - 0x1p-18f;
@@ -1293,8 +1299,11 @@ __device__ __forceinline__ int quick_csd(const LX& X, const Grid& g, const Detec
 }
 
 // u2: 1 passes, 0 fails, -1 too close.  With S the sum of |w| |rho| of a
-// curvature (the largest of the five) a float curvature is within 2^-21 S:
-// cuts of 2^-23 in both factors, a rounded product, four rounded sums.
+// curvature (the largest of the five) a float curvature is within 2^-20.8 S:
+// cuts of 2^-23 in both factors, a rounded product, four rounded sums.  What
+// underflows, a rho below 2^-126 or a product, moves it by 2^-126 of the sum of
+// |w| and by 5 2^-149: nothing next to that where S is above 2^-100 of that sum
+// and above 2^-90.
 template <class LX>
 __device__ __forceinline__ int quick_u2(const LX& X, const Grid& g, const Detect& D,
                                         const double* d2x, const double* d2y) {
@@ -1302,13 +1311,17 @@ __device__ __forceinline__ int quick_u2(const LX& X, const Grid& g, const Detect
   const int ci[5] = {0, -1, 1, 0, 0}, cj[5] = {0, 0, 0, 1, -1};
   const float lowd = D.delta_f * (1.0f - 0x1p-18f), highd = D.delta_f * (1.0f + 0x1p-18f);
   const float up = 1.0f + 0x1p-18f, down = 1.0f - 0x1p-18f;
+  if (!D.quick) return -1;
   int pass = 1;
 #pragma unroll
   for (int d = 0; d < 2; ++d) {
     if (d == 1 && !two) break;
-    float w[5];
+    float w[5], least = 0x1p-90f;
 #pragma unroll
-    for (int m = 0; m < 5; ++m) w[m] = cut_float((d == 0 ? d2x : d2y)[m]);
+    for (int m = 0; m < 5; ++m) {
+      w[m] = cut_float((d == 0 ? d2x : d2y)[m]);
+      least = fmaf(0x1p-100f, fabsf(w[m]), least);
+    }
     float cmin = 0.0f, cmax = 0.0f, S = 0.0f;
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
@@ -1323,7 +1336,7 @@ __device__ __forceinline__ int quick_u2(const LX& X, const Grid& g, const Detect
       cmax = m == 0 ? k : fmaxf(cmax, k);
     }
     const float e = 0x1p-20f * S;
-    if (!(S < 0x1p60f)) return -1;  // also a NaN
+    if (!(S < 0x1p60f && S > least)) return -1;  // also a NaN
     // the product over the intervals of cmin and cmax
     const float p1 = (cmin - e) * (cmax - e), p2 = (cmin - e) * (cmax + e);
     const float p3 = (cmin + e) * (cmax - e), p4 = (cmin + e) * (cmax + e);
