@@ -70,6 +70,7 @@ struct Scalars {
   int nactive;                  // batches: problems still advancing in this step
   unsigned long long bar_all;   // arrivals so far at the grid barrier of the MOOD loop kernel
   unsigned long long bar_small; // and at the barrier of its first kSmallBlocks blocks
+  unsigned long long progress;  // grows while that kernel's first block works
   int rate_ready;               // rate_bits holds the CFL rate of the current state
   int rate_bad;                 // and that state had a cell with no admissible rate
   int next[2][2];               // queue lengths of the MOOD loop's iterations, with the

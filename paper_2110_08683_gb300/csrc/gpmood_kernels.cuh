@@ -26,6 +26,7 @@
 #include "fixed_dot.h"
 #include "fp_bits.h"
 #include "fp_newton.h"
+#include "spin_limit.h"
 
 namespace gpm {
 
@@ -2120,9 +2121,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // barrier among `blocks` co-resident blocks on a running count of arrivals
 // (never reset: the count at rest is a multiple of `blocks`): one atomic to
 // arrive, and everyone polls for the count that completes the round.  A wait
-// gives up after about a second (or 2^26 polls) without a change of *alive
-// (null: none to look at), latches kErrSync and returns false; a block that
-// sees the error leaves the loop, so no wait can outlast the limit.
+// gives up as spin_limit.h says, after about a second without a change of
+// *alive (null: none to look at), latches kErrSync and returns false; a block
+// that sees the error leaves the loop, so no wait can outlast the limit.
 __device__ __forceinline__ unsigned long long load_acquire(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -2139,19 +2140,15 @@ __device__ __forceinline__ bool block_barrier(Scalars* sc, unsigned long long* c
     asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(old) : "l"(count) : "memory");
     const unsigned long long target = (old / blocks + 1) * blocks;
     int good = 1;
-    unsigned long long t0 = 0, seen = 0;
-    for (unsigned polls = 0; load_acquire(count) < target; ++polls) {
-      if (polls == 0) {
-        t0 = global_ns();
-        seen = alive ? load_acquire(alive) : 0;
-      } else if (polls > (1u << 26) || global_ns() - t0 > 1000000000ull) {
-        const unsigned long long now = alive ? load_acquire(alive) : seen;
-        if (now == seen || (*err & kErrSync)) {
-          atomicOr(&sc->err, kErrSync);
-          good = 0;
-          break;
-        }
-        polls = 0;
+    spin_limit w;
+    spin_start(&w, alive ? load_acquire(alive) : 0);
+    while (load_acquire(count) < target) {
+      const unsigned long long now = global_ns();
+      if (spin_due(&w, now) &&
+          ((*err & kErrSync) || spin_over(&w, now, alive ? load_acquire(alive) : 0))) {
+        atomicOr(&sc->err, kErrSync);
+        good = 0;
+        break;
       }
       __nanosleep(pause);
     }
@@ -2203,6 +2200,13 @@ struct SingleSite {
     f(A, g, D, d2x, d2y, 0);
   }
 };
+
+// a sign of life for the blocks that wait for the working ones: block 0, which
+// always works, counts its trips through the phases' loops (fire and forget)
+__device__ __forceinline__ void mood_progress(Scalars* sc, unsigned blocks) {
+  if (blocks != gridDim.x && blockIdx.x == 0 && threadIdx.x == 0)
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], 1;" ::"l"(&sc->progress) : "memory");
+}
 
 // lane index of a MOOD phase worked on by `blocks` blocks: the warps are
 // ranked block-minor (warp 0 of every block, then warp 1, ...), so the few
@@ -2281,6 +2285,7 @@ __device__ __forceinline__ void mood_faces_phase(const Site& site, const MoodArg
   const long long stride = (long long)blocks * (blockDim.x >> 5) * P;
   Real (*st)[8] = S.st[warp];
   for (long long t0 = ((long long)warp * blocks + blockIdx.x) * P; t0 < L; t0 += stride) {
+    mood_progress(M.sc, blocks);
     const long long t = t0 + lane;
     const int q = (int)(t & 3);
     const int f = (int)((t >> 2) & 3);
@@ -2369,6 +2374,7 @@ __device__ __forceinline__ void mood_update_items(const Site& site, const MoodAr
   const uint32_t* stamp = stamp_of(M, cur);
   uint32_t* next_stamp = stamp_of(M, cur + 1);
   for (long long l = mood_lane(blocks); l < 5LL * VL * n; l += stride) {
+    mood_progress(M.sc, blocks);
     const int t = (int)(l / VL);
     const int gc = queue[t / 5];
     int dg = -1;
@@ -2488,10 +2494,10 @@ __device__ __forceinline__ void mood_loop_body(const Site& site, const MoodArgs&
     slot ^= 1;
     cur += 1;
   }
-  // the waiting blocks look at the others' barrier, so a long loop is no
-  // timeout; the error flag of a failed wait also ends this one
+  // the waiting blocks look at the leader's progress (mood_progress), so a long
+  // loop is no timeout; the error flag of a failed wait also ends this one
   if (blocks != gridDim.x && tail)
-    block_barrier(sc, &sc->bar_all, gridDim.x, &sc->bar_small, 256);
+    block_barrier(sc, &sc->bar_all, gridDim.x, &sc->progress, 256);
   if (leader) {
     sc->nbad_first[stage] = nfirst;
     sc->nbad_total[stage] = total;
