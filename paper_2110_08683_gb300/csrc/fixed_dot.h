@@ -19,6 +19,7 @@
 // Plain C as well as CUDA, so that a host unit test can check it.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -79,9 +80,9 @@ FXD_FN int32_t fxd_limb_lo(int64_t s) { return (int32_t)s & ((1 << FXD_SPLIT) - 
 
 // the limbs of a weight |c| 2^T < 2^60: C = hi 2^29 + lo, |lo| <= 2^28
 FXD_FN void fxd_weight(double c, int T, int32_t* hi, int32_t* lo) {
-  // c 2^T to the nearest integer; a product by a power of two is exact
-  const double f = c * (double)(1ll << T);
-  const int64_t C = (int64_t)(f < 0.0 ? f - 0.5 : f + 0.5);
+  // c 2^T to the nearest integer; a product by a power of two is exact (a half
+  // added would be rounded itself from 2^52 on)
+  const int64_t C = (int64_t)rint(c * (double)(1ll << T));
   const int64_t h = (C + (1ll << (FXD_SPLIT - 1))) >> FXD_SPLIT;
   *hi = (int32_t)h;
   *lo = (int32_t)(C - h * (1ll << FXD_SPLIT));
