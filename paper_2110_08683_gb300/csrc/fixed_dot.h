@@ -8,7 +8,8 @@
 //           the stencil (57 bits and a sign; bits below are cut off),
 //   z_m  -> C_m, an integer multiple of 2^-T, T = 60 where |z| < 1,
 //   the sum of products exactly, in two limbs of 29 low bits and the rest,
-//   the sum rounded to 2^-61 of the stencil's scale, and once to a double.
+//   the sum cut to 2^-61 of the stencil's scale (to odd, fxd_round), and
+//   rounded once to a double.
 // A value within a factor of 16 of the stencil's largest is converted
 // without loss, so the sum carries the rounding of its weights (2^-61) and
 // the one to double: about half a unit in the last place of the result,
@@ -31,6 +32,7 @@
 
 #define FXD_SPLIT 29     // bits of the low limbs
 #define FXD_EMIN 64      // smallest reference exponent (all-zero stencils)
+#define FXD_ROUND 56     // bits of a sum of products that fxd_round takes off
 
 // the words of a double
 FXD_FN uint32_t fxd_hi(double x) {
@@ -98,11 +100,16 @@ FXD_FN void fxd_mac(fxd_acc* a, int32_t ch, int32_t cl, int32_t sh, int32_t sl) 
   a->mid += (int64_t)cl * sh;
   a->ll += (int64_t)cl * sl;
 }
-// the sum over 2^56, to the nearest (halves away from zero: odd)
+// the sum over 2^56, exact or the odd one of its two neighbours (the last bit
+// set where anything is cut off).  Odd as a function: the sum alone decides, not
+// how it is spread over the limbs, and a sum and its negative have the same
+// neighbours.  (To the nearest would need the sign of the whole sum for ties.)
 FXD_FN int64_t fxd_round(fxd_acc a) {
   const int64_t m = a.mid + (a.ll >> FXD_SPLIT);
-  const int64_t r = (m + (m >> 63) + (1ll << 26)) >> 27;
-  return (int64_t)((uint64_t)a.hh << 2) + r;
+  const int shift = FXD_ROUND - FXD_SPLIT;
+  const uint32_t cut = ((uint32_t)m & ((1u << shift) - 1u)) |
+                       ((uint32_t)a.ll & ((1u << FXD_SPLIT) - 1u));
+  return (int64_t)((uint64_t)a.hh << (2 * FXD_SPLIT - FXD_ROUND)) + ((m >> shift) | (cut != 0u));
 }
 
 // the double nearest r 2^(E + off - 1086): off = 3 + 60 - T takes the sums of
