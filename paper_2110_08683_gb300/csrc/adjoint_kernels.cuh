@@ -592,7 +592,7 @@ __device__ __forceinline__ double gather_sum(const GatherW<double>& W, const Gat
 #pragma unroll
     for (int a = -R; a <= R; ++a)
       if ((a < 0 ? -a : a) + (b < 0 ? -b : b) <= R) E = max(E, S.E[(ly + R - b) * TX + lx + R - a]);
-  // the sum as hi 2^29 + lo, in units of 2^-86 of the largest scale: a cell at the
+  // the sum as hi 2^30 + lo, in units of 2^-86 of the largest scale: a cell at the
   // rim of what a localised cotangent reaches has a small weight's product alone
   constexpr long long kLow = (1ll << FXD_SPLIT) - 1;
   long long hi = 0, lo = 0;
@@ -613,7 +613,7 @@ __device__ __forceinline__ double gather_sum(const GatherW<double>& W, const Gat
     const long long h = acc.hh + (m >> FXD_SPLIT), l = m & kLow;
     const int d = E - S.E[t];  // down by d
     hi += h >> min(d, 63);
-    lo += (d <= 35 ? (long long)(((unsigned long long)h << FXD_SPLIT | l) >> d)
+    lo += (d <= 64 - FXD_SPLIT ? (long long)(((unsigned long long)h << FXD_SPLIT | l) >> d)
                    : h >> min(d - FXD_SPLIT, 63)) & kLow;
   };
   if constexpr (UNI) {

@@ -61,13 +61,25 @@ void set_parity(const double (*cx)[kMaxN], const double (*cy)[kMaxN], const gpw_
       for (int m = 0; m < w.n; ++m) s += fabs(w.z[face][k][m]);
       l1 = fmax(l1, s);
     }
-  const int T = weight_bits(big, l1);
-  P.off = 63 - T;
-  for (int kk = 0; kk < 2; ++kk)
-    for (int c = 0; c < kMaxN; ++c) {
-      fxd_weight(cx[kk][c], T, &P.cx[kk][c].x, &P.cx[kk][c].y);
-      fxd_weight(cy[kk][c], T, &P.cy[kk][c].x, &P.cy[kk][c].y);
+  const int R = w.q - 1;
+  int T = weight_bits(big, l1) + 1;
+  for (bool fits = false; !fits;) {
+    --T;
+    fits = true;
+    for (int t = 0; t < 4; ++t) {
+      const double* z = t < 2 ? cx[t] : cy[t - 2];
+      int2* C = t < 2 ? P.cx[t] : P.cy[t - 2];
+      fxd_load load[4] = {};  // of the sum of each parity
+      for (int c = 0; c < kMaxN; ++c) {
+        fxd_weight(z[c], T, &C[c].x, &C[c].y);
+        if (c >= stencil_n(R)) continue;
+        const Comp cm = comp_at(R, c);  // of 1, 2 or 4 cells
+        fxd_count(&load[2 * cm.px + cm.py], C[c].x, C[c].y, (cm.a ? 2 : 1) * (cm.b ? 2 : 1));
+      }
+      for (int k = 0; k < 4; ++k) fits = fits && fxd_fits(&load[k]);
     }
+  }
+  P.off = 63 - T;
 }
 
 // the direct weights of every radius
@@ -96,16 +108,24 @@ void set_direct(const gpw_radius* wr, DirectW<float>& D) { plain_weights<float>(
 void set_direct(const gpw_radius* wr, DirectW<double>& D) {
   double big = 0.0, l1 = 0.0;
   largest_weights(wr, big, l1);
-  const int T = weight_bits(big, l1);
-  D.off = 63 - T;
-  for (int R = 1; R <= 3; ++R)
-    for (int face = 0; face < 4; ++face)
-      for (int k = 0; k < wr[R].q && wr[R].n; ++k)
-        for (int m = 0; m < wr[R].n; ++m) {
-          const int a = wr[R].da[m], b = wr[R].db[m];
-          int2& z = D.z[R][face][k][diamond3_slot(a, b)];
-          fxd_weight(direct_weight(wr[R], face, k, a, b), T, &z.x, &z.y);
+  int T = weight_bits(big, l1) + 1;
+  for (bool fits = false; !fits;) {
+    --T;
+    fits = true;
+    for (int R = 1; R <= 3; ++R)
+      for (int face = 0; face < 4; ++face)
+        for (int k = 0; k < wr[R].q && wr[R].n; ++k) {
+          fxd_load load = {0, 0, 0};
+          for (int m = 0; m < wr[R].n; ++m) {
+            const int a = wr[R].da[m], b = wr[R].db[m];
+            int2& z = D.z[R][face][k][diamond3_slot(a, b)];
+            fxd_weight(direct_weight(wr[R], face, k, a, b), T, &z.x, &z.y);
+            fxd_count(&load, z.x, z.y, 1);
+          }
+          fits = fits && fxd_fits(&load);
         }
+  }
+  D.off = 63 - T;
 }
 
 void fill_gather(const gpw_radius* wr, int top, GatherW<float>& G) {
@@ -118,21 +138,43 @@ void fill_gather(const gpw_radius* wr, int top, GatherW<double>& G) {
   G.top = top;
   double big = 0.0, l1 = 1.0;
   largest_weights(wr, big, l1);
+  // a cell's sum over its neighbours' faces (4 q values each, every face at a
+  // radius of its own) stays below 2^63 of the products' high limbs
   int T = 58;
   while (T > 30 && (ldexp(big, T - 58) > 1.0 || ldexp(l1, T - 58) >= 3.9)) --T;
-  G.off = 65 - T;
-  for (int face = 0; face < 4; ++face) {
-    int2& c = G.z[0][face][0][diamond3_slot(0, 0)];
-    fxd_weight(1.0, T, &c.x, &c.y);
-  }
-  for (int R = 1; R <= 3; ++R)
-    for (int face = 0; face < 4; ++face)
-      for (int k = 0; k < wr[R].q && wr[R].n; ++k)
-        for (int m = 0; m < wr[R].n; ++m) {
-          const int a = wr[R].da[m], b = wr[R].db[m];
-          int2& z = G.z[R][face][k][diamond3_slot(a, b)];
-          fxd_weight(direct_weight(wr[R], face, k, a, b), T, &z.x, &z.y);
+  ++T;
+  for (bool fits = false; !fits;) {
+    --T;
+    fits = true;
+    for (int face = 0; face < 4; ++face) {
+      int2& c = G.z[0][face][0][diamond3_slot(0, 0)];
+      fxd_weight(1.0, T, &c.x, &c.y);
+    }
+    for (int R = 1; R <= 3; ++R)
+      for (int face = 0; face < 4; ++face)
+        for (int k = 0; k < wr[R].q && wr[R].n; ++k)
+          for (int m = 0; m < wr[R].n; ++m) {
+            const int a = wr[R].da[m], b = wr[R].db[m];
+            int2& z = G.z[R][face][k][diamond3_slot(a, b)];
+            fxd_weight(direct_weight(wr[R], face, k, a, b), T, &z.x, &z.y);
+          }
+    // the limbs of one neighbour's sum: of each face the radius with the most
+    for (int slot = 0; slot < kMaxN; ++slot) {
+      fxd_load load = {0, 0, 0};
+      for (int face = 0; face < 4; ++face) {
+        fxd_load most = {0, 0, 0};
+        for (int R = 0; R <= 3; ++R) {
+          fxd_load one = {0, 0, 0};
+          for (int k = 0; k < kMaxQ; ++k)
+            fxd_count(&one, G.z[R][face][k][slot].x, G.z[R][face][k][slot].y, 1);
+          most = {fmax(most.mid, one.mid), fmax(most.up, one.up), fmax(most.down, one.down)};
         }
+        load = {load.mid + most.mid, load.up + most.up, load.down + most.down};
+      }
+      fits = fits && fxd_fits(&load);
+    }
+  }
+  G.off = 65 - T;
 }
 
 template <class Real>
