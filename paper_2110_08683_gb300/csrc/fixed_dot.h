@@ -134,9 +134,10 @@ FXD_FN int64_t fxd_round(fxd_acc a) {
 }
 
 // the double nearest r 2^(E + off - 1086): off = 3 + 60 - T takes the sums of
-// fxd_round with weights of T bits and values of reference exponent E.
-// `special`: bits OR-ed into the high word (0x7ff80000: a NaN, for a stencil
-// that holds a NaN or an infinity; else 0).
+// fxd_round with weights of T bits and values of reference exponent E.  Beyond
+// the largest double: a NaN (or an infinity).  `special`: bits OR-ed into the
+// high word (0x7ff80000: a NaN, for a stencil that holds a NaN or an infinity;
+// else 0).
 FXD_FN double fxd_to_double(int64_t r, int E, int off, uint32_t special) {
   const uint64_t s = (uint64_t)(r >> 63);
   const uint64_t m = ((uint64_t)r ^ s) - s;
@@ -147,10 +148,14 @@ FXD_FN double fxd_to_double(int64_t r, int E, int off, uint32_t special) {
     l = 0;
     e -= 32;
   }
-  const int z = fxd_clz(h);
-  const uint64_t n = z > 31 ? 0 : ((uint64_t)h << 32 | l) << z;
+  const int z = fxd_clz(h);  // 32 for r = 0
+  const uint64_t n = ((uint64_t)h << 32 | l) << z;
   const uint64_t q = (n >> 11) + ((n >> 10) & 1u);  // halves away from zero
   uint64_t b = q + ((uint64_t)(uint32_t)(e - z) << 52);
+  // an exponent past the range stays there, and out of the sign
+  uint32_t bh = (uint32_t)(b >> 32);
+  bh = bh < 0x7ff80000u ? bh : 0x7ff80000u;
+  b = (uint64_t)bh << 32 | (uint32_t)b;
   if (h == 0) b = 0;
   b |= (s & 0x8000000000000000ull) | ((uint64_t)special << 32);
   double x;
