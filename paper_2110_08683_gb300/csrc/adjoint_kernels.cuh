@@ -183,7 +183,7 @@ __device__ __forceinline__ void hllc_x_vjp(const Real* UL, const Real* UR, Real 
 
 // The same in FP64, the reverse of hllc_x_fp64 and written like it for few FP64
 // operations: about 125 a point where the form above takes 220.  The forward
-// values are hllc_x_fp64's bit for bit.
+// decisions are hllc_x_fp64's bit for bit.
 struct SideBar {
   double u, v, p, E, c, m, r;  // adjoints of the side's quantities, m the x momentum
 };
@@ -191,8 +191,8 @@ struct SideBar {
 __device__ __forceinline__ double where(bool on, double x) { return on ? x : 0.0; }
 
 // through one side's primitives, pressure and sound speed to its state
-__device__ __forceinline__ void side_vjp(const double* U, const Side& s, double v, double gam,
-                                         double gm1, const SideBar& b, double* Ub) {
+__device__ __forceinline__ void side_vjp(const double* U, const Side& s, double gam, double gm1,
+                                         const SideBar& b, double* Ub) {
   double pb = b.p, irb = 0.0;
   if (nonzero(b.c)) {
     // c = sqrt(z), z = gam p / rho: dc/dz = 1 / (2 c)
@@ -202,11 +202,10 @@ __device__ __forceinline__ void side_vjp(const double* U, const Side& s, double 
   }
   // p = gm1 (E - (m_x^2 + m_y^2) / (2 rho)), u = m_x / rho, v = m_y / rho
   const double eb = __dmul_rn(pb, gm1);
-  const double m2 = fma(U[1], U[1], __dmul_rn(U[2], U[2]));
-  irb = fma(b.u, U[1], fma(b.v, U[2], fma(-0.5 * eb, m2, irb)));
-  Ub[0] = fma(-__dmul_rn(irb, s.ir), s.ir, b.r);
+  irb = fma(b.u, U[1], fma(b.v, U[2], irb));
+  Ub[0] = fma(-fma(irb, s.ir, __dmul_rn(-0.5 * eb, s.k)), s.ir, b.r);
   Ub[1] = fma(-eb, s.u, fma(b.u, s.ir, b.m));
-  Ub[2] = fma(-eb, v, __dmul_rn(b.v, s.ir));
+  Ub[2] = fma(-eb, s.v, __dmul_rn(b.v, s.ir));
   Ub[3] = b.E + eb;
 }
 
@@ -214,7 +213,6 @@ __device__ __forceinline__ void hllc_x_vjp_fp64(const double* UL, const double* 
                                                 const double* Fb, double* UbL, double* UbR) {
   const double gm1 = gam - 1.0;
   const Side L = side_of(UL, gam, gm1), R = side_of(UR, gam, gm1);
-  const double vL = __dmul_rn(UL[2], L.ir), vR = __dmul_rn(UR[2], R.ir);
   const double aL = L.u - L.c, bL = R.u - R.c, aR = L.u + L.c, bR = R.u + R.c;
   const bool selA = lt_num(aL, bL), selAR = lt_num(bR, aR);  // the branches of min and max
   const double SL = selA ? aL : bL, SR = selAR ? aR : bR;
@@ -227,7 +225,7 @@ __device__ __forceinline__ void hllc_x_vjp_fp64(const double* UL, const double* 
   const bool useS = left || gt0_num(SR);
   const bool star = !useL && useS, sideL = useL || (useS && left);
   const double uK = sideL ? L.u : R.u, pK = sideL ? L.p : R.p, EK = sideL ? UL[3] : UR[3];
-  const double vK = sideL ? vL : vR;
+  const double vK = sideL ? L.v : R.v;
   SideBar Lb = {0, 0, 0, 0, 0, 0, 0}, Rb = {0, 0, 0, 0, 0, 0, 0};
   if (star) {
     const double dK = sideL ? dL : dR, qK = sideL ? qL : qR, SK = sideL ? SL : SR;
@@ -279,8 +277,8 @@ __device__ __forceinline__ void hllc_x_vjp_fp64(const double* UL, const double* 
     if (sideL) Lb = K;
     else Rb = K;
   }
-  side_vjp(UL, L, vL, gam, gm1, Lb, UbL);
-  side_vjp(UR, R, vR, gam, gm1, Rb, UbR);
+  side_vjp(UL, L, gam, gm1, Lb, UbL);
+  side_vjp(UR, R, gam, gm1, Rb, UbR);
 }
 
 // EDP1 radius of the face between (iL,jL) and (iR,jR) from a radius map

@@ -424,11 +424,12 @@ __device__ __forceinline__ void hll_x(const Real* UL, const Real* UR, Real gam, 
 // point (76 as hllc_x above, whose reciprocals and roots took 24):
 //  - reciprocals and square roots on the integer pipes (fp_newton.h);
 //  - products rho u are the momenta themselves;
-//  - one flux formula f = (f0, f0 u + p, f0 v, u (E + p)) for the physical
-//    flux of a side, f0 = rho u, and for the star region, whose velocity is
-//    the contact's: u = S*, f0 = rho* S*, with p* = p_K + q_K (S* - u_K),
-//    E* = (d_K E_K + p* S* - p_K u_K) / (S_K - S*), rho* = q_K / (S_K - S*),
-//    d_K = S_K - u_K and q_K = rho_K d_K (Rankine-Hugoniot across S_K).
+//  - one flux formula f = (f0, f0 u + p, f0 v, u H) for the star region, whose
+//    velocity is the contact's, u = S*, and for the physical flux of a side,
+//    which is what u = u_K makes of it: with d_K = S_K - u_K, q_K = rho_K d_K
+//    (Rankine-Hugoniot across S_K)
+//      p = p_K + q_K (u - u_K), f0 = q_K / (S_K - u) u (or the momentum itself),
+//      H = E + p = (d_K E_K + p S_K - p_K u_K) / (S_K - u).
 // All products and sums are rounded one by one or explicit FMAs, so every
 // kernel gets the same flux bit for bit.
 // ---------------------------------------------------------------------------
@@ -452,18 +453,22 @@ __device__ __forceinline__ bool pos_normal(double x) {
   return b >= 0x0010000000000000ll && b < 0x7ff0000000000000ll;
 }
 
-// one side of a face: velocity along x, pressure, sound speed and 1/rho
+// one side of a face: velocities, twice the kinetic energy, pressure, sound
+// speed and 1/rho
 struct Side {
-  double u, p, c, ir;
+  double u, v, k, p, c, ir;
   bool ok;  // inside the solver's domain
 };
 __device__ __forceinline__ Side side_of(const double* U, double gam, double gm1) {
   Side s;
   s.ir = recip_int(U[0]);
   s.u = __dmul_rn(U[1], s.ir);
-  const double m2 = fma(U[1], U[1], __dmul_rn(U[2], U[2]));
-  // a subnormal ir / 2 (rho beyond 2^1020) has no use here
-  s.p = __dmul_rn(gm1, fma(-half_of(s.ir), m2, U[3]));
+  // by the velocities, although (m_x^2 + m_y^2) / rho is a product less where v
+  // has no other use: squares of momenta leave the range of doubles long before
+  // the state does (below 1e-154 and above 1e154)
+  s.v = __dmul_rn(U[2], s.ir);
+  s.k = fma(U[1], s.u, __dmul_rn(U[2], s.v));
+  s.p = __dmul_rn(gm1, fma(-0.5, s.k, U[3]));
   s.ok = pos_normal(U[0]) && pos_normal(s.p);
   s.c = sqrt_int(__dmul_rn(__dmul_rn(gam, s.p), s.ir));
   // what the caller checks: outside the domain the pressure is not a number
@@ -492,18 +497,18 @@ __device__ __forceinline__ void hllc_x_fp64(const double* UL, const double* UR, 
   const bool sideL = useL || (useS && left);
   const double uK = sideL ? L.u : R.u, pK = sideL ? L.p : R.p, EK = sideL ? UL[3] : UR[3];
   const double mK = sideL ? UL[1] : UR[1];
-  const double vK = __dmul_rn(sideL ? UL[2] : UR[2], sideL ? L.ir : R.ir);
+  const double vK = sideL ? L.v : R.v;
   const double SK = sideL ? SL : SR, dK = sideL ? dL : dR, qK = sideL ? qL : qR;
-  const double iD = recip_int(SK - Ss);
-  const double ps = fma(qK, Ss - uK, pK);
-  const double Es = __dmul_rn(iD, fma(dK, EK, fma(ps, Ss, -__dmul_rn(pK, uK))));
-  const double fs = __dmul_rn(__dmul_rn(qK, iD), Ss);
-  const double u = star ? Ss : uK, p = star ? ps : pK, E = star ? Es : EK;
+  const double u = star ? Ss : uK;
+  const double iD = recip_int(SK - u);
+  const double p = fma(qK, u - uK, pK);
+  const double H = __dmul_rn(iD, fma(dK, EK, fma(p, SK, -__dmul_rn(pK, uK))));
+  const double fs = __dmul_rn(__dmul_rn(qK, iD), u);
   const double f = star ? fs : mK;
   F[0] = f;
   F[1] = fma(f, u, p);
   F[2] = __dmul_rn(f, vK);
-  F[3] = __dmul_rn(u, E + p);
+  F[3] = __dmul_rn(u, H);
   if (!(L.ok && R.ok)) {
 #pragma unroll
     for (int v = 0; v < 4; ++v) qnan(F[v]);
@@ -519,10 +524,9 @@ __device__ __forceinline__ void hll_x_fp64(const double* UL, const double* UR, d
   const double SL = min_num(L.u - L.c, R.u - R.c);
   const double SR = max_num(L.u + L.c, R.u + R.c);
   // physical fluxes by the same rounded sequence on both sides
-  const double vL = __dmul_rn(UL[2], L.ir), vR = __dmul_rn(UR[2], R.ir);
-  const double FL[4] = {UL[1], fma(UL[1], L.u, L.p), __dmul_rn(UL[1], vL),
+  const double FL[4] = {UL[1], fma(UL[1], L.u, L.p), __dmul_rn(UL[1], L.v),
                         __dmul_rn(L.u, UL[3] + L.p)};
-  const double FR[4] = {UR[1], fma(UR[1], R.u, R.p), __dmul_rn(UR[1], vR),
+  const double FR[4] = {UR[1], fma(UR[1], R.u, R.p), __dmul_rn(UR[1], R.v),
                         __dmul_rn(R.u, UR[3] + R.p)};
   // F = a F_L - b F_R + c (U_R - U_L), a = S_R / w, b = S_L / w, c = S_L S_R / w,
   // w = S_R - S_L
