@@ -556,17 +556,27 @@ __global__ void __launch_bounds__(256) k_adj_gather(Grid g, const __grid_constan
 // the same, FP64, in fixed point (fixed_dot.h): on the FP64 pipe its 4 x 156
 // (R = 2) products a cell take 40000 cycles a warp, 1.11 ms at 1024^2.  A block
 // covers 32 x 8 cells of the ghosted grid; a variable at a time, the state
-// adjoints of the cells n whose faces reach them are staged as integers with one exponent a cell n (the largest of its up to
-// 4 q values), each output cell sums its neighbours' products exactly, and the
-// sums are added at the largest scale of the neighbourhood, cut at 2^-86 of it.
+// adjoints of the cells n whose faces reach them are staged as integers with one
+// exponent a cell n (the largest of its up to 4 q values; one a face where the
+// tile has faces below the top radius, which do not reach as far), each output
+// cell sums its neighbours' products exactly, and the sums are added at the
+// largest scale of what reaches it, cut at 2^-86 of it.
 // 1024^2, R = 2: 0.63 ms a launch, bound by issue.
 template <int R>
 struct GatherShared {
   static constexpr int TX = 32 + 2 * R, TY = 8 + 2 * R, NV = 4 * rule_q(R);
   int2 X[NV][TY * TX];       // limbs (high, low), [face E, W, N, S][point] of cell n
-  int E[TY * TX];
-  uint32_t K[TY * TX];       // the four faces' radii, a byte each (0xff: no face)
+  // reference exponents of the values, one a face in 16 bits (kWild: one of the
+  // face's values is not finite); in a tile whose faces are all at the top radius
+  // the cell's largest for all four
+  uint2 E[TY * TX];
+  uint32_t K[TY * TX];       // the four faces' radii, a byte each (kNoFace: no face)
 };
+constexpr uint32_t kNoFace = 0x40;  // (radius 0 in the low bits: the values are zero)
+constexpr uint32_t kWild = 0x8000;
+__device__ __forceinline__ uint32_t face_exponent(uint2 e, int face) {
+  return (face < 2 ? e.x : e.y) >> (16 * (face & 1)) & 0xffffu;
+}
 
 // the radius-independent part of a face: its index, or -1 beyond the grid
 __device__ __forceinline__ long long gather_face_index(const Grid& g, int face, int i, int j) {
@@ -584,57 +594,65 @@ template <int R, bool UNI>
 __device__ __forceinline__ double gather_sum(const GatherW<double>& W, const GatherShared<R>& S,
                                              int lx, int ly) {
   constexpr int Q = rule_q(R), TX = GatherShared<R>::TX;
+  // f(t, a, b) for every cell t of the diamond, this one at its offset (a, b)
+  auto diamond = [&](auto&& f) {
+#pragma unroll(UNI ? 2 * R + 1 : 1)
+    for (int b = -R; b <= R; ++b)
+#pragma unroll(UNI ? 2 * R + 1 : 1)
+      for (int a = -R; a <= R; ++a)
+        if ((a < 0 ? -a : a) + (b < 0 ? -b : b) <= R) f((ly + R - b) * TX + lx + R - a, a, b);
+  };
+  auto reaches = [&](int t, int face, int a, int b) {
+    return UNI || (int)(S.K[t] >> (8 * face) & 3) >= (a < 0 ? -a : a) + (b < 0 ? -b : b);
+  };
+  // the largest exponent of what reaches this cell
   int E = FXD_EMIN;
-#pragma unroll
-  for (int b = -R; b <= R; ++b)
-#pragma unroll
-    for (int a = -R; a <= R; ++a)
-      if ((a < 0 ? -a : a) + (b < 0 ? -b : b) <= R) E = max(E, S.E[(ly + R - b) * TX + lx + R - a]);
+  diamond([&](int t, int a, int b) {
+    const uint2 e = S.E[t];
+    for (int face = 0; face < (UNI ? 1 : 4); ++face)
+      if (reaches(t, face, a, b)) E = max(E, (int)face_exponent(e, face));
+  });
+  uint32_t special = 0;
+  if (E >= (int)kWild) {  // a NaN or an infinity among it
+    special = 0x7ff80000u;
+    E &= (int)kWild - 1;
+  }
   // the sum as hi 2^30 + lo, in units of 2^-86 of the largest scale: a cell at the
   // rim of what a localised cotangent reaches has a small weight's product alone
   constexpr long long kLow = (1ll << FXD_SPLIT) - 1;
   long long hi = 0, lo = 0;
-  auto neighbour = [&](int a, int b) {
-    const int t = (ly + R - b) * TX + lx + R - a, slot = diamond3_slot(a, b);
+  auto add = [&](const fxd_acc& acc, uint32_t e) {
+    const long long m = acc.mid + (acc.ll >> FXD_SPLIT);
+    const long long h = acc.hh + (m >> FXD_SPLIT), l = m & kLow;
+    const int d = max(E - (int)(e & (kWild - 1)), 0);  // down by d
+    hi += h >> min(d, 63);
+    lo += (d <= 64 - FXD_SPLIT ? (long long)(((unsigned long long)h << FXD_SPLIT | l) >> d)
+                   : h >> min(d - FXD_SPLIT, 63)) & kLow;
+  };
+  diamond([&](int t, int a, int b) {
+    const int slot = diamond3_slot(a, b);
+    const uint2 e = S.E[t];
     fxd_acc acc = {0, 0, 0};
 #pragma unroll
     for (int face = 0; face < 4; ++face) {
-      const int K = UNI ? R : (S.K[t] >> (8 * face)) & 3;  // no face: the values are zero
+      const int K = UNI ? R : S.K[t] >> (8 * face) & 3;
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
         const int2 z = W.z[K][face][q][slot];
         const int2 x = S.X[face * Q + q][t];
         fxd_mac(&acc, z.x, z.y, x.x, x.y);
       }
+      if (UNI ? face == 3 : reaches(t, face, a, b)) add(acc, face_exponent(e, face));
+      if (!UNI) acc = {0, 0, 0};
     }
-    const long long m = acc.mid + (acc.ll >> FXD_SPLIT);
-    const long long h = acc.hh + (m >> FXD_SPLIT), l = m & kLow;
-    const int d = E - S.E[t];  // down by d
-    hi += h >> min(d, 63);
-    lo += (d <= 64 - FXD_SPLIT ? (long long)(((unsigned long long)h << FXD_SPLIT | l) >> d)
-                   : h >> min(d - FXD_SPLIT, 63)) & kLow;
-  };
-  if constexpr (UNI) {
-#pragma unroll
-    for (int b = -R; b <= R; ++b)
-#pragma unroll
-      for (int a = -R; a <= R; ++a)
-        if ((a < 0 ? -a : a) + (b < 0 ? -b : b) <= R) neighbour(a, b);
-  } else {
-#pragma unroll 1
-    for (int b = -R; b <= R; ++b) {
-      const int hb = R - (b < 0 ? -b : b);
-#pragma unroll 1
-      for (int a = -hb; a <= hb; ++a) neighbour(a, b);
-    }
-  }
+  });
   hi += lo >> FXD_SPLIT;
   lo &= kLow;
   // as many of the low bits as there is room for (|hi| < 2^62)
   const int z = __clzll(hi ^ (hi >> 63)) - 2;
   const int k = E > 128 ? max(min(z, FXD_SPLIT), 0) : 0;
   return fxd_to_double((long long)((unsigned long long)hi << k) + (lo >> (FXD_SPLIT - k)), E,
-                       W.off - k, E == 0x7ff ? 0x7ff80000u : 0u);
+                       W.off - k, special);
 }
 
 template <int R>
@@ -651,7 +669,7 @@ __global__ void __launch_bounds__(256) k_adj_gather_fx(Grid g,
     uint32_t k4 = 0;
     for (int face = 0; face < 4; ++face) {
       const long long f = gather_face_index(g, face, i, j);
-      const uint32_t k = f < 0 ? 0xffu : (face < 2 ? Ax.K : Ay.K)[f];
+      const uint32_t k = f < 0 ? kNoFace : (face < 2 ? Ax.K : Ay.K)[f];
       top = top && (f < 0 || k == R);
       k4 |= k << (8 * face);
     }
@@ -665,28 +683,38 @@ __global__ void __launch_bounds__(256) k_adj_gather_fx(Grid g,
     for (int t = threadIdx.x; t < TX * TY; t += 256) {
       const int i = i0 - R + t % TX, j = j0 - R + t / TX;
       double x[4 * Q];
-      uint32_t most = (uint32_t)FXD_EMIN << 20;
+      uint32_t most[4], all = 0;
 #pragma unroll
       for (int face = 0; face < 4; ++face) {
         const uint32_t K = (S.K[t] >> (8 * face)) & 0xffu;
         const AdjFaces& F = face < 2 ? Ax : Ay;
         const double* s = (const double*)((face & 1) ? F.R : F.L);
         const long long f = gather_face_index(g, face, i, j);
-        const int n = K == 0xffu ? 0 : rule_q((int)K);  // the points in use
+        const int n = K == kNoFace ? 0 : rule_q((int)K);  // the points in use
+        uint32_t wild = 0;
+        most[face] = (uint32_t)FXD_EMIN << 20;
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
           const double u = q < n ? s[((long long)v * kMaxQ + q) * F.nf + f] : 0.0;
-          x[face * Q + q] = u;
-          most = max(most, fxd_hi(u) & 0x7fffffffu);
+          const uint32_t h = fxd_hi(u) & 0x7fffffffu;
+          const bool finite = h < 0x7ff00000u;
+          x[face * Q + q] = finite ? u : 0.0;
+          most[face] = max(most[face], finite ? h : 0u);
+          wild |= finite ? 0u : kWild;
+        }
+        most[face] = most[face] >> 20 | wild;
+        all = max(all & (kWild - 1), most[face] & (kWild - 1)) | ((all | most[face]) & kWild);
+      }
+#pragma unroll
+      for (int face = 0; face < 4; ++face) {
+        if (uni) most[face] = all;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const long long m = fxd_from_double(x[face * Q + q], (int)(most[face] & (kWild - 1)));
+          S.X[face * Q + q][t] = make_int2(fxd_limb_hi(m), fxd_limb_lo(m));
         }
       }
-      const int E = (int)(most >> 20);
-#pragma unroll
-      for (int k = 0; k < 4 * Q; ++k) {
-        const long long m = fxd_from_double(x[k], E);
-        S.X[k][t] = make_int2(fxd_limb_hi(m), fxd_limb_lo(m));
-      }
-      S.E[t] = E;
+      S.E[t] = make_uint2(most[0] | most[1] << 16, most[2] | most[3] << 16);
     }
     __syncthreads();
     if (out) {
