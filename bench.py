@@ -489,42 +489,52 @@ def measure(kind, nx, ny, precision, scheme, steps, warmup, world, local, eager=
         faces = (nx + 1) * ny + (nx * (ny + 1) if fused else 0)
         peak = FP64_PEAK_TFLOPS if real64 else FP32_PEAK_TFLOPS
         alg = faces * algorithmic_flops_per_face(R)
+        alg_count = ("algorithmic: 8 q N reconstruction FMA (2 flop), q HLLC at %d flop, the "
+                     "Gauss sum; per face, x %s faces a launch"
+                     % (HLLC_FLOPS, "(nx+1) ny + nx (ny+1)" if fused else "(nx+1) ny"))
+        roofline = {"bound": "alu", "peak": round(peak, 4), "unit": "TFLOP/s",
+                    "traffic": ncu_traffic(precision, kind, scheme)}
         if real64:
+            # against the FP64 pipe: the lane-instructions a second that the kernel
+            # issues to it (2 flop each); its reconstruction is integer work
             n = fp64_instructions_per_face(R)
-            # lane-instructions a second against the pipe's rate (2 flop each)
-            executed = {"fp64_instructions_per_face": n,
-                        "frac": round(2 * faces * n / per_launch_s / 1e12 / peak, 4),
-                        "count": "FP64 instructions of the Riemann solver and the Gauss sum; "
-                                 "the reconstruction runs in fixed point on the integer pipes"}
+            exe = 2 * faces * n
+            roofline.update({
+                "achieved": round(exe / per_launch_s / 1e12, 4),
+                "frac": round(exe / per_launch_s / 1e12 / peak, 4),
+                "kernel": "k_faces_fx<R=%d>" % R + (" (x and y faces)" if fused else ""),
+                "fp64_instructions_per_face": n,
+                "count": "FP64 instructions of the Riemann solver and the Gauss sum, 2 flop each; "
+                         "the reconstruction runs in fixed point on the integer pipes",
+                "algorithmic": {"flops_per_face": algorithmic_flops_per_face(R),
+                                "flops_per_launch": alg,
+                                "tflops": round(alg / per_launch_s / 1e12, 4),
+                                "count": alg_count + "; most of it runs on the integer pipes, "
+                                                     "so no fraction of the FP64 peak"}})
         else:
             exe = faces * faces_flops_per_face(R, fused)
-            executed = {"flops_per_face": round(faces_flops_per_face(R, fused), 1),
-                        "flops_per_launch": exe,
-                        "achieved": round(exe / per_launch_s / 1e12, 4),
-                        "frac": round(exe / per_launch_s / 1e12 / peak, 4),
-                        "count": "the kernel's own arithmetic after the parity-sum "
-                                 "reconstruction (mirror-orbit sums, q/2 dot products, "
-                                 "butterflies)"}
-        roofline = {
-            "bound": "alu", "achieved": round(alg / per_launch_s / 1e12, 4),
-            "peak": round(peak, 4), "unit": "TFLOP/s",
-            "frac": round(alg / per_launch_s / 1e12 / peak, 4),
-            "traffic": ncu_traffic(precision, kind, scheme),
-            "kernel": ("k_faces_fx<R=%d>" % R if real64 else
-                       ("k_faces_xy<R=%d,float>" if fused else "k_faces<R=%d,float,x>") % R)
-                      + (" (x and y faces)" if fused else ""),
-            "flops_per_launch": alg,
-            "flops_per_face": algorithmic_flops_per_face(R),
-            "count": "algorithmic: 8 q N reconstruction FMA (2 flop), q HLLC at %d flop, the "
-                     "Gauss sum; per face, x %s faces a launch"
-                     % (HLLC_FLOPS, "(nx+1) ny + nx (ny+1)" if fused else "(nx+1) ny"),
-            "executed": executed,
+            roofline.update({
+                "achieved": round(alg / per_launch_s / 1e12, 4),
+                "frac": round(alg / per_launch_s / 1e12 / peak, 4),
+                "kernel": ("k_faces_xy<R=%d,float>" if fused else "k_faces<R=%d,float,x>") % R
+                          + (" (x and y faces)" if fused else ""),
+                "flops_per_launch": alg,
+                "flops_per_face": algorithmic_flops_per_face(R),
+                "count": alg_count,
+                "executed": {"flops_per_face": round(faces_flops_per_face(R, fused), 1),
+                             "flops_per_launch": exe,
+                             "achieved": round(exe / per_launch_s / 1e12, 4),
+                             "frac": round(exe / per_launch_s / 1e12 / peak, 4),
+                             "count": "the kernel's own arithmetic after the parity-sum "
+                                      "reconstruction (mirror-orbit sums, q/2 dot products, "
+                                      "butterflies)"}})
+        roofline.update({
             "launch_ms": round(per_launch_s * 1e3, 4),
             "timing": "event nodes around every x-face launch in the step graph, second timed "
                       "pass of the same steps (L2 flushed between steps)",
             "peak_source": "derived: 152 SMs x %s/clk x 2.07 GHz (of nominal; measured DFMA "
                            "1.19 TFLOP/s, FFMA 69.9 TFLOP/s)" % ("4 FP64 flop" if real64
-                                                                 else "256 FP32 flop")}
+                                                                 else "256 FP32 flop")})
     total_kernel_ms = sum(v[0] for v in kt.values())
     shares = {k: round(v[0] / total_kernel_ms, 4) if total_kernel_ms else None
               for k, v in kt.items()} if prof else None

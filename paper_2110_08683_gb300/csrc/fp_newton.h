@@ -3,7 +3,8 @@
 // step in 32-bit fixed point, and a second one whose residual is exact in
 // 64 bits, rounded once to the nearest double.  About 35 and 45 integer
 // instructions, next to 3 and 6 FP64 ones that hold the FP64 pipe 64 cycles
-// each.  Errors below 0.51 units in the last place.
+// each.  Errors below 0.54 (reciprocal) and 0.52 (square root) units in the last
+// place for seeds within 2^-22; the largest met in 4 million are 0.517 and 0.509.
 // For finite normal arguments (sqrt: positive); anything else gives an
 // unspecified value.
 // Plain C as well as CUDA: on the host the seeds are passed in, so that a

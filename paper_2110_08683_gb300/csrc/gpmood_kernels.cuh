@@ -1233,7 +1233,7 @@ __device__ __forceinline__ void keep_verdict(const StageArgs<Real>& A, const Gri
 // the rounding.  quick_csd: kVerdictAccept (CAD, PAD and CSD pass),
 // kVerdictCsdFailed (CAD and PAD pass, CSD fails) or kVerdictNone (too close
 // to a threshold, or CAD or PAD may fail, or out of float's range).  Few cells
-// are close, and an FP64 operation costs 64 times a float one: 0.26 ms a launch
+// are close, and an FP64 operation costs 64 times a float one: 0.21 ms a launch
 // at 4096 x 1024 (the candidate and the RK sums) for 0.78 with the tests in FP64.
 // The double -> float cut is below 2^-23 relative and so is every float
 // operation on normal numbers; |u|, K = |m|^2 / (2 rho) and E carry at most 8

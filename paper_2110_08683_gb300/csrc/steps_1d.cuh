@@ -7,7 +7,7 @@
 // and finds what the phase before wrote in its own L1, and a run needs no launch
 // a step.  Its FP64 pipes are one SM's, so the general step is the faster one
 // above kMaxCells1D cells: a step of the R = 2 shock tube takes, in one block
-// and in general, 81 and 126 us at 128 cells, 112 and 142 at 256, 153 and 151 at
+// and in general, 81 and 124 us at 128 cells, 114 and 142 at 256, 153 and 152 at
 // 512, 168 and 155 at 640 (R = 1 and 3 cross between 512 and 640 too).
 #pragma once
 
