@@ -182,7 +182,7 @@ __device__ __forceinline__ void hllc_x_vjp(const Real* UL, const Real* UR, Real 
 }
 
 // The same in FP64, the reverse of hllc_x_fp64 and written like it for few FP64
-// operations: about 125 a point where the form above takes 220.  The forward
+// operations: about 129 a point where the form above takes 220.  The forward
 // decisions are hllc_x_fp64's bit for bit.
 struct SideBar {
   double u, v, p, E, c, m, r;  // adjoints of the side's quantities, m the x momentum
